@@ -60,7 +60,8 @@ typedef enum {
  * tdks_magnus_step) and the density interpolation of a Magnus step are
  * double-float as well. */
 typedef enum {
-  TDKS_FP64 = 0,   /* double contractions                                  */
+  TDKS_FP64 = 0,   /* FP64-accurate contractions (55-bit fixed point with a
+                      float tail per element: below the FP64 rounding)     */
   TDKS_FP32 = 1,   /* float contractions with float accumulation, FP64 I/O  */
   TDKS_DF64 = 2,   /* double-float (compensated float-pair) contractions:
                       ~48-bit accurate products and sums on the FP32 pipe   */

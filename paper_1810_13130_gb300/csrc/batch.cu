@@ -600,7 +600,7 @@ tdks_status tdks_batch_create(int n_sys, const tdks_mesh_desc* meshes, const tdk
       d.P1 = c->P1;
       d.tab = prec == TDKS_FP32 ? (const void*)c->d_tabf
               : (prec == TDKS_DF64 || prec == TDKS_MIXED) ? (const void*)c->d_tabdf
-                                                          : (const void*)c->d_tab;
+                                                          : (const void*)&c->fx;
       d.tab32 = c->d_tabf;
       b->degs.push_back(d);
     }

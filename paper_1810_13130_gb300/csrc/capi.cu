@@ -81,6 +81,7 @@ void free_ctx(tdks_ctx* c) {
   cudaFree(c->d_tabf);
   cudaFree(c->d_tabdf);
   cudaFree(c->d_tabbf);
+  cudaFree(c->d_fxK);
   cudaFree(c->d_occ);
   cudaFree(c->d_R);
   cudaFree(c->d_Z);
@@ -131,18 +132,20 @@ float round_bf16(float x) {
 }
 
 // Folded storage of a centrosymmetric n x n matrix (layout in tdks_internal.h).
-void fold_centrosymmetric(const double* M, int n, double* out) {
+template <typename T>
+void fold_centrosymmetric(const T* M, int n, T* out) {
   const int h = n / 2;
+  const T half = (T)0.5;
   for (int q = 0; q < h; ++q)
     for (int i = 0; i < h; ++i) {
-      out[q * h + i] = 0.5 * (M[q * n + i] + M[q * n + (n - 1 - i)]);
-      out[h * h + q * h + i] = 0.5 * (M[q * n + i] - M[q * n + (n - 1 - i)]);
+      out[q * h + i] = half * (M[q * n + i] + M[q * n + (n - 1 - i)]);
+      out[h * h + q * h + i] = half * (M[q * n + i] - M[q * n + (n - 1 - i)]);
     }
-  double* mc = out + 2 * h * h;
-  double* mr = mc + h;
-  for (int q = 0; q < h; ++q) mc[q] = (n & 1) ? M[q * n + h] : 0.0;
-  for (int i = 0; i < h; ++i) mr[i] = (n & 1) ? M[h * n + i] : 0.0;
-  mr[h] = (n & 1) ? M[h * n + h] : 0.0;
+  T* mc = out + 2 * h * h;
+  T* mr = mc + h;
+  for (int q = 0; q < h; ++q) mc[q] = (n & 1) ? M[q * n + h] : (T)0;
+  for (int i = 0; i < h; ++i) mr[i] = (n & 1) ? M[h * n + i] : (T)0;
+  mr[h] = (n & 1) ? M[h * n + h] : (T)0;
 }
 
 tdks_status check_orb(tdks_ctx* c, int n_orb) {
@@ -340,6 +343,23 @@ tdks_status tdks_create(const tdks_mesh_desc* m, const tdks_system_desc* s, void
   std::vector<float> tabbf(tab.size());
   for (size_t k = 0; k < tab.size(); ++k) tabbf[k] = round_bf16(tabf[k]);
   if ((st = upload(c, &c->d_tabbf, tabbf)) != TDKS_OK) return fail(st);
+  {
+    // fixed-point tables: W^1/2 B and its transpose folded in extended precision
+    std::vector<long double> Bt(P1 * P1), f(cs_size(P1));
+    for (int q = 0; q < P1; ++q)
+      for (int i = 0; i < P1; ++i) Bt[i * P1 + q] = t.Bw[q * P1 + i];
+    for (const std::vector<long double>* m : {&t.Bw, &Bt}) {
+      std::fill(f.begin(), f.end(), 0.0L);
+      fold_centrosymmetric(m->data(), P1, f.data());
+      for (long double x : f) c->fx_c.push_back(llrintl(ldexpl(x, 63)));
+    }
+    std::vector<double> fk(cs_size(P1));
+    fold_centrosymmetric(t.Kw.data(), P1, fk.data());
+    if ((st = upload(c, &c->d_fxK, fk)) != TDKS_OK) return fail(st);
+    c->fx.c = c->fx_c.data();
+    c->fx.dK = c->d_fxK;
+    c->fx.kinf = t.kw_inf;
+  }
   if ((st = upload(c, &c->d_occ, c->occ)) != TDKS_OK) return fail(st);
   if ((st = upload(c, &c->d_R, c->R)) != TDKS_OK) return fail(st);
   if ((st = upload(c, &c->d_Z, c->Z)) != TDKS_OK) return fail(st);

@@ -32,18 +32,6 @@ using namespace tdks;
 
 namespace {
 
-template <int P1>
-struct Cfg {
-  static constexpr int P2 = P1 * P1;
-  static constexpr int P3 = P2 * P1;
-  static constexpr int E = (256 / P2) < 1 ? 1 : (256 / P2);   // elements per CTA
-};
-
-// Byte offset of the cp.async prefetch buffer (16-byte entries) in dynamic shared
-// memory: the end of the element lines rounded up to 16 bytes.  With float lines
-// that end is only 8-byte aligned for odd P1 (E * 2 * P1^3 * 4 bytes).
-__host__ __device__ constexpr size_t pf_offset(size_t lines_end) { return (lines_end + 15) & ~size_t(15); }
-
 // ---------------------------------------------------------------------------
 // Hbar psibar, complex, contraction type T (double or float)
 //
@@ -225,24 +213,6 @@ __device__ __forceinline__ void hbar_elem_body(const Geom& g, const T* sB, const
     __syncthreads();
   }
 }
-
-// Shared-memory layout of one element's lines in the split body: entry (a, b, c) at
-// c * PS + b * LS + a, the Gauss-space copy S2 at P1 * PS, the next element ES entries on.
-// The strides are padded (chosen by counting shared-memory wavefronts of the x-, y- and
-// z-line accesses of 32-thread warps that straddle elements, for 4- and 8-byte entries)
-// so that the line loads and stores of a warp fall into distinct banks as far as the
-// P1 x P1 thread planes allow: at p = 7 the wavefronts per request fall from 4.3 to 1.3,
-// at p = 6 from 1.8 to 1.6.
-template <int P1, typename T>
-struct SplitLayout {
-  static constexpr bool kF = sizeof(T) == 4;
-  static constexpr int LS = P1 == 8 || P1 == 9 ? 9 : P1;
-  static constexpr int PS = P1 == 5 ? 25 : P1 == 6 ? 39 : P1 == 7 ? (kF ? 56 : 52) : P1 == 8 ? 72
-                          : P1 == 9 ? (kF ? 81 : 89) : P1 * P1;
-  static constexpr int ES = P1 == 5 ? 253 : P1 == 6 ? (kF ? 484 : 468) : P1 == 7 ? (kF ? 785 : 737)
-                          : P1 == 8 ? 1152 : P1 == 9 ? (kF ? 1465 : 1617) : 2 * P1 * P1 * P1;
-  static_assert(PS >= P1 * LS && ES >= 2 * P1 * PS, "padded layout holds two element cubes");
-};
 
 // Split form of the element body for the double-float contractions: Hbar is real, so
 // the real and imaginary parts pass through the element one after the other.  Each
@@ -605,12 +575,14 @@ __device__ __forceinline__ int node_elems(int I, int p, int n, int* e, int* loc)
 // contributions in a fixed order and applies the Loewdin scale.  With `lanczos`
 // the three-term update w = Hbar q_j - alpha_j q_j - beta_{j-1} q_{j-1} is fused
 // (ca = alpha_j s_j, cb = beta_{j-1} s_{j-1}) and the sum of |w|^2 over the rows
-// r0, r0 + rstride, ... handled here is returned.  The degree is a compile-time
+// r0, r0 + rstride, ... handled here is returned.  FP64 element results are those of V_j
+// (the fixed-point kernel leaves the scale out): qs = s_j scales them here, 1 otherwise.
+// The degree is a compile-time
 // constant: the node -> (element, local index) split is a multiply-shift.
 template <int P1, typename T>
 __device__ __forceinline__ double assemble_rows(const Geom& g, const Cx<T>* __restrict__ evo,
                                                 const double2* qj, const double2* qm,
-                                                double2* out, double ca, double cb, int lanczos,
+                                                double2* out, double qs, double ca, double cb, int lanczos,
                                                 int accumulate, int r0, int rstride) {
   constexpr int p = P1 - 1, P2 = P1 * P1, P3 = P2 * P1;
   constexpr bool kF32 = std::is_same<T, float>::value;
@@ -639,7 +611,7 @@ __device__ __forceinline__ double assemble_rows(const Geom& g, const Cx<T>* __re
       for (int ky = 0; ky < 2; ++ky)
         if (kz < nz && ky < ny)
           base[kz * ny + ky] = (long long)g.nx * (ey[ky] + (long long)g.ny * ez[kz]) * P3 + bz[kz] * P2 + by[ky] * P1;
-    const double syz = g.s[1][J] * g.s[2][K];
+    const double syz = g.s[1][J] * g.s[2][K] * qs;
     const float syzf = g.sf[1][J] * g.sf[2][K];
     const long long rowbase = (long long)g.nix * (r);
     for (int I = tI + 1; I <= g.nix; I += tstep) {
@@ -717,10 +689,11 @@ template <int P1, typename T>
 __global__ void __launch_bounds__(128) k_assemble(Geom g, const Cx<T>* __restrict__ ev, ApplyArgs a) {
   __shared__ double red[4];
   const int o = blockIdx.y;
-  double ca = 0.0, cb = 0.0;
+  double ca = 0.0, cb = 0.0, qs = 1.0;
   if (a.kry) {
     const KryOrb& K = a.kry[o];
     if (K.status != KRY_ACTIVE) return;
+    if (std::is_same<T, double>::value) qs = K.s[a.kj];
     if (a.lanczos) {
       ca = K.alpha[a.kj] * K.s[a.kj];
       cb = a.kj > 0 ? K.beta[a.kj - 1] * K.s[a.kj - 1] : 0.0;
@@ -731,7 +704,7 @@ __global__ void __launch_bounds__(128) k_assemble(Geom g, const Cx<T>* __restric
   const double2* qj = a.in_base + (long long)o * a.in_stride;
   const double2* qm = a.vm_base ? a.vm_base + (long long)o * a.vm_stride : nullptr;
   double2* out = a.out_base + (long long)o * a.out_stride;
-  const double acc = assemble_rows<P1, T>(g, evo, qj, qm, out, ca, cb, a.lanczos, a.accumulate,
+  const double acc = assemble_rows<P1, T>(g, evo, qj, qm, out, qs, ca, cb, a.lanczos, a.accumulate,
                                           blockIdx.x, gridDim.x);
   if (a.npart) {
     const double s = block_sum(acc, red);
@@ -859,78 +832,6 @@ __global__ void k_diag_add(long long n, int n_orb, const double* __restrict__ vn
 // current basis vector V_j (j = K.k): the exponential's start vector for j = 0
 // (input or, after a sub-step, output), the workspace otherwise.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ const double2* bvec(const BSys& S, const KryOrb& K, int o, int j) {
-  if (j == 0) return (K.nsub == 0 ? S.in : S.out) + (long long)o * S.n_int;
-  return S.Vw + ((long long)o * S.kmax + (j - 1)) * S.n_int;
-}
-
-template <int P1, typename T>
-__global__ void __launch_bounds__(256, 2) k_hbar_batch(const BSys* __restrict__ sys,
-                                                    const BItem* __restrict__ items, int n_items,
-                                                    const T* __restrict__ tab, int* __restrict__ qctr) {
-  constexpr int P3 = Cfg<P1>::P3;
-  constexpr int CS = 2 * (P1 / 2) * (P1 / 2) + 2 * (P1 / 2) + 1;
-  typedef Cx<T> V;
-  extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ double red[8];
-  T* sB = reinterpret_cast<T*>(smem);
-  T* sBT = sB + CS;
-  T* sK = sBT + CS;
-  T* sw = sK + CS;
-  const size_t off = ((3 * CS + P1) * sizeof(T) + 15) & ~size_t(15);
-  V* S1 = reinterpret_cast<V*>(smem + off) + (size_t)threadIdx.y * 2 * P3;
-  V* S2 = S1 + P3;
-  const int tid = threadIdx.x + blockDim.x * threadIdx.y;
-  const int nthr = blockDim.x * blockDim.y;
-  for (int i = tid; i < 3 * CS; i += nthr) sB[i] = tab[tab_off_csB(P1) + i];
-  for (int i = tid; i < P1; i += nthr) sw[i] = tab[tab_off_w(P1) + i];
-  __syncthreads();
-  // the current item's system descriptor is staged in shared memory: its fields are
-  // re-read where used instead of occupying registers across the element body
-  // items are taken from a shared ticket counter (zeroed before every launch), so
-  // CTAs that draw items of finished orbitals move on at once and the grid stays
-  // balanced whatever the mix of active orbitals
-  __shared__ BSys sS;
-  __shared__ BItem sW;
-  __shared__ int sIt;
-  for (;;) {
-    __syncthreads();
-    if (tid == 0) {
-      const int it = atomicAdd(qctr, 1);
-      sIt = it;
-      if (it < n_items) sW = items[it];
-    }
-    __syncthreads();
-    if (sIt >= n_items) break;
-    for (int i = tid; i < (int)(sizeof(BSys) / 8); i += nthr)
-      reinterpret_cast<long long*>(&sS)[i] = reinterpret_cast<const long long*>(&sys[sW.sys])[i];
-    __syncthreads();
-    const BItem w = sW;
-    const BSys& S = sS;
-    const Geom& g = S.g;
-    const long long eidx = (long long)w.eblk * blockDim.y + threadIdx.y;
-    auto orb = [&](int o, const double2*& in, double& sc) -> bool {
-      const KryOrb& K = S.kry[o];
-      if (K.status != KRY_ACTIVE) return false;
-      const int j = K.k;
-      in = bvec(S, K, o, j);
-      sc = K.s[j];
-      return true;
-    };
-    {   // an item none of whose orbitals is active is skipped before the element set-up
-      bool any = false;
-      for (int o = w.o0; o < w.o1 && !any; ++o) {
-        const double2* in_o;
-        double sc_o;
-        any = orb(o, in_o, sc_o);
-      }
-      if (!any) continue;
-    }
-    hbar_elem_body<P1, T>(g, sB, sBT, sK, sw, S1, S2, red, S.vks, eidx, w.o0, w.o1, orb,
-                          static_cast<Cx<T>*>(S.ev), S.apart, S.n_eblk, w.eblk);
-  }
-}
-
 // Batched element results are kept at the orbital stride of 16-byte entries for every
 // contraction type, so that under TDKS_MIXED FP32 and double-float orbitals share the
 // buffer: entries of Cx<T> per orbital = n_elem P1^3 * omul<T>.
@@ -1041,7 +942,8 @@ __global__ void __launch_bounds__(128) k_bassemble(const BSys* __restrict__ sys,
   double2* out = S.Vw + ((long long)w.o * S.kmax + j) * S.n_int;
   const Cx<T>* evo = static_cast<const Cx<T>*>(S.ev) +
                      (long long)w.o * S.n_elem * (P1 * P1 * P1) * batch_omul<T>();
-  const double acc = assemble_rows<P1, T>(S.g, evo, qj, qm, out, ca, cb, 1, 0, w.rblk, S.n_rblk);
+  const double qs = std::is_same<T, double>::value ? K.s[j] : 1.0;
+  const double acc = assemble_rows<P1, T>(S.g, evo, qj, qm, out, qs, ca, cb, 1, 0, w.rblk, S.n_rblk);
   const double sum = block_sum(acc, red);
   if (threadIdx.x == 0) S.npart[(long long)w.o * S.n_rblk + w.rblk] = sum;
 }
@@ -1570,6 +1472,7 @@ template <int P1, typename T, bool kBF = false>
 tdks_status hbar_t(tdks_ctx* c, const ApplyArgs& a) {
   constexpr int P2 = Cfg<P1>::P2, P3 = Cfg<P1>::P3, E = Cfg<P1>::E;
   constexpr int CS = 2 * (P1 / 2) * (P1 / 2) + 2 * (P1 / 2) + 1;
+  constexpr bool kFx = std::is_same<T, double>::value;       // fixed-point element kernel (hbar_fx.cu)
   constexpr bool kSplit = std::is_same<T, Df>::value || (std::is_same<T, float>::value && !kBF);
   constexpr size_t elem = kSplit ? (size_t)SplitLayout<P1, T>::ES * sizeof(T) : 2 * P3 * sizeof(Cx<T>);
   const size_t lines_end = (((3 * CS + P1) * sizeof(T) + 15) & ~size_t(15)) + (size_t)E * elem;
@@ -1586,7 +1489,7 @@ tdks_status hbar_t(tdks_ctx* c, const ApplyArgs& a) {
       if (study)
         TDKS_CU(c, cudaFuncSetAttribute(k_hbar_split<P1, T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)smem));
-  } else {
+  } else if constexpr (!kFx) {
     TDKS_CU(c, set_smem(k_hbar<P1, T, kBF>, smem));
   }
   const size_t need = (size_t)a.n_orb * c->n_elem * P3 * sizeof(Cx<T>);
@@ -1601,16 +1504,20 @@ tdks_status hbar_t(tdks_ctx* c, const ApplyArgs& a) {
     c->evec_bytes = need;
   }
   Cx<T>* ev = static_cast<Cx<T>*>(c->d_evec);
-  const int bpe = elem_blocks_t<P1>(c);
+  // fixed point: fewer elements per CTA while the launch would leave SMs idle (the smallest
+  // meshes are bound by the latency of one CTA, not by the work)
+  int E_l = E;
+  if constexpr (kFx)
+    while (E_l > 1 && ((c->n_elem + E_l - 1) / E_l) * a.n_orb < 2 * 152) E_l = (E_l + 1) / 2;
+  const int bpe = (int)((c->n_elem + E_l - 1) / E_l);
   // orbitals per CTA: V and geometry are reused across them; keep >= 8 CTAs per SM
   // (about four waves at two CTAs per SM, so the last partial wave costs little)
   int opc = 1;
   while (opc < a.n_orb && (long long)bpe * ((a.n_orb + 2 * opc - 1) / (2 * opc)) >= 8 * 152) opc *= 2;
   if (c->opc_force > 0) opc = c->opc_force < a.n_orb ? c->opc_force : a.n_orb;
   const int ochunks = (a.n_orb + opc - 1) / opc;
-  const T* tab = std::is_same<T, double>::value ? (const T*)c->d_tab
-                 : std::is_same<T, float>::value ? (const T*)(kBF ? c->d_tabbf : c->d_tabf)
-                                                 : (const T*)c->d_tabdf;
+  [[maybe_unused]] const T* tab =
+      std::is_same<T, float>::value ? (const T*)(kBF ? c->d_tabbf : c->d_tabf) : (const T*)c->d_tabdf;
   const Geom g = tdks_geom(c);
   if (c->kb) TDKS_TRY(kb_project(c, a));
   if constexpr (kStudyOk) {
@@ -1621,6 +1528,8 @@ tdks_status hbar_t(tdks_ctx* c, const ApplyArgs& a) {
       k_hbar_split<P1, T><<<dim3(bpe, ochunks), dim3(P2, E), smem, c->stream>>>(g, tab, c->d_vks, a, opc, ev, 0u);
   } else if constexpr (kSplit)
     k_hbar_split<P1, T><<<dim3(bpe, ochunks), dim3(P2, E), smem, c->stream>>>(g, tab, c->d_vks, a, opc, ev, 0u);
+  else if constexpr (kFx)
+    TDKS_CU(c, launch_hbar_fx(P1, g, c->fx, c->d_vks, a, E_l, bpe, opc, reinterpret_cast<double2*>(ev), c->stream));
   else
     k_hbar<P1, T, kBF><<<dim3(bpe, ochunks), dim3(P2, E), smem, c->stream>>>(g, tab, c->d_vks, a, opc, ev);
   if (a.lanczos && a.kry && a.part) {
@@ -1856,44 +1765,17 @@ tdks_status launch_density(tdks_ctx* c, const double2* psi, int n_orb, double* r
 // ---- batched apply launchers ------------------------------------------------
 template <int P1, typename T>
 static size_t hbar_batch_smem_t(int E) {
-  constexpr int P3 = Cfg<P1>::P3;
   constexpr int CS = 2 * (P1 / 2) * (P1 / 2) + 2 * (P1 / 2) + 1;
-  constexpr bool kSplit = !std::is_same<T, double>::value;
-  constexpr size_t elem = kSplit ? (size_t)SplitLayout<P1, T>::ES * sizeof(T) : 2 * P3 * sizeof(Cx<T>);
-  const size_t lines_end = (((3 * CS + P1) * sizeof(T) + 15) & ~size_t(15)) + (size_t)E * elem;
-  return kSplit ? pf_offset(lines_end) + (size_t)E * Cfg<P1>::P2 * P1 * sizeof(double2)   // + prefetch buffer
-                : lines_end;
-}
-
-template <int P1>
-static size_t hbar_batch_smem_p(int prec, int E) {
-  if (prec == TDKS_FP32) return hbar_batch_smem_t<P1, float>(E);
-  if (prec == TDKS_DF64) return hbar_batch_smem_t<P1, Df>(E);
-  return hbar_batch_smem_t<P1, double>(E);
-}
-
-size_t hbar_batch_smem(int P1, int prec, int E) {
-  switch (P1) {
-    case 2: return hbar_batch_smem_p<2>(prec, E);
-    case 3: return hbar_batch_smem_p<3>(prec, E);
-    case 4: return hbar_batch_smem_p<4>(prec, E);
-    case 5: return hbar_batch_smem_p<5>(prec, E);
-    case 6: return hbar_batch_smem_p<6>(prec, E);
-    case 7: return hbar_batch_smem_p<7>(prec, E);
-    case 8: return hbar_batch_smem_p<8>(prec, E);
-    case 9: return hbar_batch_smem_p<9>(prec, E);
-    default: return 0;
-  }
+  const size_t lines_end =
+      (((3 * CS + P1) * sizeof(T) + 15) & ~size_t(15)) + (size_t)E * SplitLayout<P1, T>::ES * sizeof(T);
+  return pf_offset(lines_end) + (size_t)E * Cfg<P1>::P2 * P1 * sizeof(double2);   // + prefetch buffer
 }
 
 template <int P1, typename T>
 static cudaError_t hbar_batch_launch_t(const BSys* sys, const BItem* items, int n_items, int E,
                                        int grid, const void* tab, int* qctr, cudaStream_t st, int* occ) {
   const size_t smem = hbar_batch_smem_t<P1, T>(E);
-  // split body for double-float (see k_hbar_split), complex body otherwise
-  void (*kern)(const BSys*, const BItem*, int, const T*, int*);
-  if constexpr (!std::is_same<T, double>::value) kern = k_hbar_batch_split<P1, T>;
-  else kern = k_hbar_batch<P1, T>;
+  const auto kern = k_hbar_batch_split<P1, T>;
   // the kernel also holds ~330 B of static shared memory: opt in for any large size
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -1908,13 +1790,16 @@ static cudaError_t hbar_batch_p(int prec, const BSys* sys, const BItem* items, i
                                 int grid, const void* tab, int* qctr, cudaStream_t st, int* occ) {
   if (E < 1 || Cfg<P1>::P2 * E > 256) return cudaErrorInvalidValue;
   if (prec == TDKS_FP32) return hbar_batch_launch_t<P1, float>(sys, items, n_items, E, grid, tab, qctr, st, occ);
-  if (prec == TDKS_DF64) return hbar_batch_launch_t<P1, Df>(sys, items, n_items, E, grid, tab, qctr, st, occ);
-  return hbar_batch_launch_t<P1, double>(sys, items, n_items, E, grid, tab, qctr, st, occ);
+  return hbar_batch_launch_t<P1, Df>(sys, items, n_items, E, grid, tab, qctr, st, occ);
 }
+
+// tab: the device table of the contraction type; FP64: the tdks::FxHost (host)
 
 static cudaError_t hbar_batch_dispatch(int P1, int prec, const BSys* sys, const BItem* items,
                                        int n_items, int E, int grid, const void* tab, int* qctr,
                                        cudaStream_t st, int* occ) {
+  if (prec == TDKS_FP64)
+    return launch_hbar_batch_fx(P1, static_cast<const FxHost*>(tab), sys, items, n_items, E, grid, qctr, st, occ);
   switch (P1) {
     case 2: return hbar_batch_p<2>(prec, sys, items, n_items, E, grid, tab, qctr, st, occ);
     case 3: return hbar_batch_p<3>(prec, sys, items, n_items, E, grid, tab, qctr, st, occ);

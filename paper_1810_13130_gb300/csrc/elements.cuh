@@ -388,4 +388,42 @@ __device__ __forceinline__ T block_sum_t(T v, T* red) {
   return s;
 }
 
+// ---- launch shape and layouts shared by the element kernels ---------------------
+template <int P1>
+struct Cfg {
+  static constexpr int P2 = P1 * P1;
+  static constexpr int P3 = P2 * P1;
+  static constexpr int E = (256 / P2) < 1 ? 1 : (256 / P2);   // elements per CTA
+};
+
+// Byte offset of the cp.async prefetch buffer (16-byte entries) in dynamic shared
+// memory: the end of the element lines rounded up to 16 bytes.  With float lines
+// that end is only 8-byte aligned for odd P1 (E * 2 * P1^3 * 4 bytes).
+__host__ __device__ constexpr size_t pf_offset(size_t lines_end) { return (lines_end + 15) & ~size_t(15); }
+
+// Shared-memory layout of one element's lines in the split body: entry (a, b, c) at
+// c * PS + b * LS + a, the Gauss-space copy S2 at P1 * PS, the next element ES entries on.
+// The strides are padded (chosen by counting shared-memory wavefronts of the x-, y- and
+// z-line accesses of 32-thread warps that straddle elements, for 4- and 8-byte entries)
+// so that the line loads and stores of a warp fall into distinct banks as far as the
+// P1 x P1 thread planes allow: at p = 7 the wavefronts per request fall from 4.3 to 1.3,
+// at p = 6 from 1.8 to 1.6.
+template <int P1, typename T>
+struct SplitLayout {
+  static constexpr bool kF = sizeof(T) == 4;
+  static constexpr int LS = P1 == 8 || P1 == 9 ? 9 : P1;
+  static constexpr int PS = P1 == 5 ? 25 : P1 == 6 ? 39 : P1 == 7 ? (kF ? 56 : 52) : P1 == 8 ? 72
+                          : P1 == 9 ? (kF ? 81 : 89) : P1 * P1;
+  static constexpr int ES = P1 == 5 ? 253 : P1 == 6 ? (kF ? 484 : 468) : P1 == 7 ? (kF ? 785 : 737)
+                          : P1 == 8 ? 1152 : P1 == 9 ? (kF ? 1465 : 1617) : 2 * P1 * P1 * P1;
+  static_assert(PS >= P1 * LS && ES >= 2 * P1 * PS, "padded layout holds two element cubes");
+};
+
+// Krylov vector V_j of an orbital of a batched system: the exponential's start vector for
+// j = 0 (input or, after a sub-step, output), the workspace otherwise
+__device__ __forceinline__ const double2* bvec(const BSys& S, const KryOrb& K, int o, int j) {
+  if (j == 0) return (K.nsub == 0 ? S.in : S.out) + (long long)o * S.n_int;
+  return S.Vw + ((long long)o * S.kmax + (j - 1)) * S.n_int;
+}
+
 }  // namespace tdks

@@ -1,0 +1,182 @@
+// Fixed-point contractions with a float tail: the element operator in integer arithmetic.
+//
+// GB300 runs 2 FP64 operations per clock and SM; its integer pipe multiplies 32 x 32 bits
+// into 64 sixteen times as fast, its FP32 pipe is 64 times as fast.  So a contraction is
+// carried out in 55-bit integers with an FP32 tail below them: faster than the FP64 pipe
+// and more accurate.  All values of one element and orbital share a power of two:
+//   value x = (V + f) 2^E,    V a 64-bit integer, |V| < 2^55, f a float of a few units;
+//   coefficient c = C 2^-63,  C = h 2^32 + l, |c| < 1, l signed.
+// With V = vh 2^32 + vl (vl signed; taken from V + 2^31, whose high word is vh)
+//   C V 2^-64 = h vh + (h vl + l vh) 2^-32 + (l 2^-32)(vl 2^-32),
+// half the product: every contraction halves the unit's exponent count by one (E grows by
+// 1), which keeps h in 32 bits.  A dot product sums h vh and mid = sum (h vl + l vh)
+// exactly in 64 bits (three wide multiply-adds per term); the integer part is
+// sum h vh + (mid >> 32), rounded to nearest.  What is left goes to the tail in FP32: the
+// fraction of mid 2^-32, sum (c / 2) f and the low products, each to about 2^-21 of a
+// unit, so a result is good to some 2^-75 of the element's largest value.  Measured on the
+// CPU against 80-bit arithmetic the whole element operator is off by 4.7e-17 .. 9.7e-17
+// relative in the 2-norm (p = 2..8, smooth and random vectors: little more than the
+// rounding of the result), the FP64 contractions by 2.4e-16 .. 1.2e-15.
+//
+// Range: with row sums sum |c| = R, |sum h vl| <= R 2^62 and |sum l vh| <= 5 2^31 2^(56 - 32)
+// R^2, so |mid| < 2^63 for R <= 1.54, the largest row sum (the transposed interpolation of
+// p = 2); the integer parts keep |V| < 2^55 / 2 * R.
+#pragma once
+
+#include <cuda_runtime.h>
+
+namespace tdks {
+
+struct FxC {      // coefficient c 2^63 = h 2^32 + l, and c / 2, l 2^-32 as floats
+  int h, l;
+  float c, cl;
+};
+struct FxL {      // the limbs alone
+  int h, l;
+};
+
+constexpr int kFxBits = 55;   // |V| < 2^55 on input
+
+// c 2^63 -> limbs (|c| < 1)
+__host__ __device__ __forceinline__ FxC fx_coef(long long c) {
+  const long long h = (c >> 32) + ((c >> 31) & 1);
+  const int l = (int)(unsigned)c;
+  return FxC{(int)h, l, (float)c * 0x1p-64f, (float)l * 0x1p-32f};
+}
+
+__host__ __device__ __forceinline__ float fx_bits_float(unsigned b) {
+#ifdef __CUDA_ARCH__
+  return __uint_as_float(b);
+#else
+  float f;
+  __builtin_memcpy(&f, &b, 4);
+  return f;
+#endif
+}
+// 1 + w 2^-32, cut to 23 bits
+__host__ __device__ __forceinline__ float fx_frac1(unsigned w) { return fx_bits_float((w >> 9) + 0x3f800000u); }
+
+// operand: V = h 2^32 + l (l signed), its tail f, and g = 1.5 + l 2^-32
+struct FxV {
+  int h, l;
+  float f, g;
+};
+constexpr long long kFxHalf = 1ll << 31;
+// from V + 2^31
+__host__ __device__ __forceinline__ FxV fx_operand(long long vb, float f) {
+  const unsigned w = (unsigned)vb;
+  return FxV{(int)(vb >> 32), (int)(w ^ 0x80000000u), f, fx_frac1(w)};
+}
+// a b + c; as one instruction also where b is known to be non-negative (the compiler would
+// extend such an operand without sign and multiply 64 x 64 bits)
+__host__ __device__ __forceinline__ long long fx_mad(int a, int b, long long c) {
+#ifdef __CUDA_ARCH__
+  long long d;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
+  return d;
+#else
+  return (long long)a * (long long)b + c;
+#endif
+}
+
+// A dot product: term() for every term, close(), then top() for every term.  The tail
+// constant k of a row is -1.5 (1 + sum of its cl): operands bring g = 1.5 + l 2^-32, the
+// fraction of mid comes as 1 + fraction, and mid starts at one half.
+struct FxDot {
+  long long mid = kFxHalf, hi = 0;
+  float f = 0.0f;
+  __host__ __device__ __forceinline__ void term(FxC c, const FxV& x) {
+    mid = fx_mad(c.l, x.h, fx_mad(c.h, x.l, mid));
+    f = fmaf(c.cl, x.g, fmaf(c.c, x.f, f));
+  }
+  __host__ __device__ __forceinline__ void close(float k) {
+    hi = mid >> 32;
+    f += fx_frac1((unsigned)mid) + k;
+  }
+  __host__ __device__ __forceinline__ void top(FxC c, const FxV& x) { hi = fx_mad(c.h, x.h, hi); }
+};
+
+// Folded operator: coefficients in the layout of tdks_internal.h (CS of them), tail
+// constants of the even, odd and middle rows (KS).
+template <int N>
+struct FxOp {
+  static constexpr int h = N / 2, CS = 2 * h * h + 2 * h + 1, KS = 2 * h + 1;
+};
+
+// M (v, f) / 2 for a centrosymmetric N x N operator; c(i), k(i) its coefficients and tail
+// constants; out(q, V, F) takes output q as soon as it is formed (all inputs have been
+// read by then, so it may overwrite them in place).
+template <int N, class CF, class KF, class OF>
+__host__ __device__ __forceinline__ void fx_apply(CF c, KF k, const long long (&v)[N], const float (&f)[N], OF out) {
+  constexpr int h = N / 2;
+  constexpr int hh = h > 0 ? h : 1;
+  FxV e[hh], o[hh], m{0, 0, 0.0f, 0.0f};
+#pragma unroll
+  for (int i = 0; i < h; ++i) {
+    e[i] = fx_operand(v[i] + v[N - 1 - i] + kFxHalf, f[i] + f[N - 1 - i]);
+    o[i] = fx_operand(v[i] - v[N - 1 - i] + kFxHalf, f[i] - f[N - 1 - i]);
+  }
+  if (N & 1) m = fx_operand(v[h] + kFxHalf, f[h]);
+#pragma unroll
+  for (int q = 0; q < h; ++q) {
+    FxDot a, b;
+#pragma unroll
+    for (int i = 0; i < h; ++i) {
+      a.term(c(q * h + i), e[i]);
+      b.term(c(h * h + q * h + i), o[i]);
+    }
+    if (N & 1) a.term(c(2 * h * h + q), m);
+    a.close(k(q));
+    b.close(k(h + q));
+#pragma unroll
+    for (int i = 0; i < h; ++i) {
+      a.top(c(q * h + i), e[i]);
+      b.top(c(h * h + q * h + i), o[i]);
+    }
+    if (N & 1) a.top(c(2 * h * h + q), m);
+    out(q, a.hi + b.hi, a.f + b.f);
+    out(N - 1 - q, a.hi - b.hi, a.f - b.f);
+  }
+  if (N & 1) {
+    FxDot a;
+#pragma unroll
+    for (int i = 0; i < h; ++i) a.term(c(2 * h * h + h + i), e[i]);
+    a.term(c(2 * h * h + 2 * h), m);
+    a.close(k(2 * h));
+#pragma unroll
+    for (int i = 0; i < h; ++i) a.top(c(2 * h * h + h + i), e[i]);
+    a.top(c(2 * h * h + 2 * h), m);
+    out(h, a.hi, a.f);
+  }
+}
+
+// Tail constant i (ke, ko, km order) of the folded rows whose cl are given by c(i).
+template <int N, class CF>
+__host__ __device__ __forceinline__ float fx_tail_const(CF c, int i) {
+  constexpr int h = N / 2;
+  float s = 0.0f;
+  if (i < h) {
+    for (int j = 0; j < h; ++j) s += c(i * h + j).cl;
+    if (N & 1) s += c(2 * h * h + i).cl;
+  } else if (i < 2 * h) {
+    for (int j = 0; j < h; ++j) s += c(h * h + (i - h) * h + j).cl;
+  } else {
+    for (int j = 0; j < h; ++j) s += c(2 * h * h + h + j).cl;
+    s += c(2 * h * h + 2 * h).cl;
+  }
+  return -1.5f - 1.5f * s;
+}
+
+// y -> V at the block exponent eb (biased exponent of the block's largest |y|, in
+// [64, 2046]): |V| < 2^kFxBits.  Bits below one unit are cut off (sign-magnitude); subnormal
+// y give 0.
+__host__ __device__ __forceinline__ long long fx_from_bits(unsigned hw, unsigned lw, int eb) {
+  const int e = (int)((hw >> 20) & 0x7ffu);
+  unsigned long long m = ((unsigned long long)((hw & 0xfffffu) | 0x100000u) << 32) | lw;
+  int d = eb - e;
+  d = (e == 0 || d > 63) ? 63 : d;
+  m = (m << (kFxBits - 53)) >> d;
+  return (hw & 0x80000000u) ? -(long long)m : (long long)m;
+}
+
+}  // namespace tdks

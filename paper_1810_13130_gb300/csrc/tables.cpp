@@ -155,6 +155,23 @@ Tables1D tdks_build_tables(int p, int nq) {
       for (int m = 0; m < nq; ++m) s += Dg[m * nq + a] * om[m] * Dg[m * nq + b];
       t.Kq[a * nq + b] = (double)s;
     }
+  // the same operators with the Gauss weights split evenly (hbar_fx.cu)
+  t.Bw.resize(nq * P1);
+  t.Kw.resize(nq * nq);
+  ld kinf = 0.0L;
+  for (int a = 0; a < nq; ++a) {
+    ld row = 0.0L;
+    for (int i = 0; i < P1; ++i) t.Bw[a * P1 + i] = sqrtl(om[a]) * B[a * P1 + i];
+    for (int b = 0; b < nq; ++b) {
+      ld s = 0.0L;
+      for (int m = 0; m < nq; ++m) s += Dg[m * nq + a] * om[m] * Dg[m * nq + b];
+      s /= sqrtl(om[a] * om[b]);
+      t.Kw[a * nq + b] = (double)s;
+      row += fabsl(s);
+    }
+    kinf = row > kinf ? row : kinf;
+  }
+  t.kw_inf = (double)kinf;
   t.K1.resize(P1 * P1);
   t.Mg.resize(P1 * P1);
   for (int i = 0; i < P1; ++i)

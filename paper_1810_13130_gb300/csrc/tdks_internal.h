@@ -69,6 +69,15 @@ struct Geom {
   const double* wq;            // Gauss weights on [-1, 1] (P1)
 };
 
+namespace tdks {
+// Fixed-point tables of a degree (fixed.cuh), units of 2^-63.
+struct FxHost {
+  const long long* c = nullptr; // folded B' = W^1/2 B, then B'^T (2 * cs_size entries)
+  const double* dK = nullptr;   // device: folded K' = W^-1/2 Kq W^-1/2 (cs_size doubles)
+  double kinf = 0.0;            // largest row sum of |K'|
+};
+}  // namespace tdks
+
 struct tdks_ctx {
   // mesh
   int nx = 0, ny = 0, nz = 0, p = 0, P1 = 0, nq = 0;
@@ -94,6 +103,8 @@ struct tdks_ctx {
   float* d_tabf = nullptr;     // float copy
   float* d_tabdf = nullptr;    // double-float copy (hi, lo pairs)
   float* d_tabbf = nullptr;    // float copy rounded to bfloat16 (BF16-operand mode)
+  std::vector<long long> fx_c; // fixed-point tables (FxHost::c)
+  double* d_fxK = nullptr;     // and the folded K'
   double* d_occ = nullptr;
   double* d_R = nullptr;
   double* d_Z = nullptr;
@@ -131,6 +142,7 @@ struct tdks_ctx {
   int device_loop = 1;          // Lanczos iterations of a sub-step as one CUDA graph (krylov.cu)
   void* kgraph = nullptr;       // its cached graphs
   double mixed_relax = 1e8;     // TDKS_MIXED: FP32 contractions once every estimate <= relax * tol
+  tdks::FxHost fx;              // fixed-point tables of the element kernel (hbar_fx.cu)
   unsigned f32_stages = 0;      // per-stage precision study of the double-float apply (diagnostics)
   double2* d_ro_part = nullptr; // its partial dots [n_orb][TDKS_KMAX][chunks]
   double2* d_ro_h = nullptr;    // its projections [n_orb][TDKS_KMAX]
@@ -166,6 +178,9 @@ struct Tables1D {
   std::vector<double> B, D;        // [nq][P1] Lagrange values / derivatives at Gauss points
   std::vector<double> Kq;          // [nq][nq] Dg^T diag(omega) Dg on Gauss-point Lagrange basis
   std::vector<double> K1, Mg;      // [P1][P1] D^T W D and B^T W B
+  std::vector<long double> Bw;     // [nq][P1] W^1/2 B
+  std::vector<double> Kw;          // [nq][nq] W^-1/2 Kq W^-1/2
+  double kw_inf = 0.0;             // largest row sum of |Kw|
 };
 Tables1D tdks_build_tables(int p, int nq);
 // fdm.cpp: generalized eigenpairs (1-D stiffness, 1-D Gauss mass) of one axis
@@ -221,6 +236,10 @@ struct ApplyArgs {
   int accumulate;             // out += result instead of out = result (plain apply only)
 };
 tdks_status launch_hbar_apply(tdks_ctx* c, const ApplyArgs& a, int prec);
+// hbar_fx.cu: element results of the FP64 and double-float applications, E elements per
+// CTA (bpe CTAs) and opc orbitals per CTA; results and alpha as described there
+cudaError_t launch_hbar_fx(int P1, const Geom& g, const tdks::FxHost& h, const double* vks, const ApplyArgs& a,
+                           int E, int bpe, int opc, double2* ev, cudaStream_t st);
 tdks_status launch_stiffness(tdks_ctx* c, const double* in, double* out, double* part,
                              const CgState* cg);
 tdks_status launch_load_vector(tdks_ctx* c, const double* f_q, double* out, double scale,
@@ -324,11 +343,12 @@ struct BOrb { int sys, o; };               // one orbital of one system
 struct BKbItem { int sys, o, p, pad; };    // nonlocal projection: projector p of orbital o
 
 // elements.cu
-size_t hbar_batch_smem(int P1, int prec, int E);
 cudaError_t hbar_batch_occupancy(int P1, int prec, int E, int* blocks_per_sm);
 // qctr: the launch's work ticket counter, zero at launch
 cudaError_t launch_hbar_batch(int P1, int prec, const BSys* sys, const BItem* items, int n_items,
                               int E, int grid, const void* tab, int* qctr, cudaStream_t st);
+cudaError_t launch_hbar_batch_fx(int P1, const tdks::FxHost* h, const BSys* sys, const BItem* items, int n_items,
+                                 int E, int grid, int* qctr, cudaStream_t st, int* occ);
 cudaError_t launch_balpha(const BSys* sys, const BOrb* orbs, int n_orbs, cudaStream_t st);
 // rows: (system, orbital, row block) items of systems of degree P1 - 1 only
 cudaError_t launch_bassemble(int P1, int prec, const BSys* sys, const BRow* rows, int n_rows,
