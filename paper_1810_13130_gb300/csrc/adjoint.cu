@@ -250,7 +250,6 @@ tdks_status hxc_adjoint(tdks_ctx* c, AdjState* A, const double* rho, const doubl
   const size_t nf = (size_t)(c->n_elem * c->nq3);
   const long long n = c->n_int;
   if (c->hartree) {
-    TDKS_CU(c, cudaMemsetAsync(A->ny, 0, n * sizeof(double), c->stream));
     TDKS_TRY(launch_load_vector(c, g_h, A->ny, 1.0, 0));     // (B^T)^(x)3 g_h, assembled
     TDKS_CU(c, cudaMemsetAsync(A->nz, 0, n * sizeof(double), c->stream));
     TDKS_TRY(run_cg_solve(c, A->ny, A->nz, nullptr));

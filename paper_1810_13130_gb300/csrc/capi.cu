@@ -96,7 +96,7 @@ void free_ctx(tdks_ctx* c) {
   cudaFree(c->d_b);
   cudaFree(c->d_r);
   cudaFree(c->d_pv);
-  cudaFree(c->d_Ap);
+  cudaFree(c->d_sev);
   cudaFree(c->d_cg);
   for (int w = 0; w < 2; ++w) {
     cudaFree(c->d_Vw[w]);
@@ -329,6 +329,7 @@ tdks_status tdks_create(const tdks_mesh_desc* m, const tdks_system_desc* s, void
     // GLL-collocation variant: GLL weights and the folded 1-D stiffness K1 = D^T W D
     std::memcpy(&tab[tab_off_wl(P1)], t.w.data(), P1 * sizeof(double));
     fold_centrosymmetric(t.K1.data(), P1, &tab[tab_off_csK1(P1)]);
+    fold_centrosymmetric(t.Mg.data(), P1, &tab[tab_off_csMg(P1)]);
   }
   std::vector<float> tabf(tab.begin(), tab.end());
   std::vector<float> tabdf(2 * tab.size());
@@ -369,13 +370,14 @@ tdks_status tdks_create(const tdks_mesh_desc* m, const tdks_system_desc* s, void
     if ((st = dalloc(c, f, nf)) != TDKS_OK) return fail(st);
     if (cudaMemset(*f, 0, nf * sizeof(double)) != cudaSuccess) return fail(TDKS_ERR_CUDA);
   }
-  double** vecs[] = {&c->d_phi, &c->d_b, &c->d_r, &c->d_pv, &c->d_Ap};
+  double** vecs[] = {&c->d_phi, &c->d_b, &c->d_r, &c->d_pv};
   for (double** f : vecs) {
     if ((st = dalloc(c, f, (size_t)c->n_int)) != TDKS_OK) return fail(st);
     if (cudaMemset(*f, 0, c->n_int * sizeof(double)) != cudaSuccess) return fail(TDKS_ERR_CUDA);
   }
+  if ((st = dalloc(c, &c->d_sev, nf)) != TDKS_OK) return fail(st);
   if ((st = dalloc(c, &c->d_cg, 1)) != TDKS_OK) return fail(st);
-  const int bpc = hbar_blocks_per_color(c);
+  const int bpc = hbar_blocks(c);
   c->part_stride = std::max<int64_t>(2048, 8 * (int64_t)bpc);
   if ((st = dalloc(c, &c->d_part, (size_t)(2 * (c->n_orb + 2) * c->part_stride + 8192))) != TDKS_OK)
     return fail(st);

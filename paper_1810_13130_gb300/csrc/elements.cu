@@ -18,9 +18,8 @@
 // cx' = hy hz / (2 hx), factored as Mg_x (cy' K1_y Mg_z + cz' Mg_y K1_z) + cx' K1_x Mg_y Mg_z:
 // 7 contractions per element.
 //
-// Assembly: elements are processed in 8 parity colours (one launch each); two
-// elements of one colour never share a node, so the scatter is a plain
-// read-modify-write and the summation order is fixed (deterministic results).
+// Assembly: every kernel writes element results and a gather sums each node's (at most
+// eight) contributions in a fixed order (deterministic, no atomics).
 #include <cuda_bf16.h>
 
 #include <cstdio>
@@ -949,121 +948,107 @@ __global__ void __launch_bounds__(128) k_bassemble(const BSys* __restrict__ sys,
 }
 
 // ---------------------------------------------------------------------------
-// Poisson stiffness K u (real, FP64), nodal 7-contraction form
+// Poisson stiffness K u (real, FP64), nodal 7-contraction form with folded operators:
+// element results only, assembled by k_gather.  Contractions along x, y, then z, so that
+// the results end in the layout of the gathered input (thread = z-column): coalesced
+// stores, and the partials of u . K u come from the thread's own registers.
+//
+// All elements in one launch and one gather replace eight colour launches that scattered
+// into the result: on small meshes each launch took the latency of one CTA (18 us at
+// p = 4, 6^3 elements: 144 us an application; with two elements per CTA, see elems_per_cta,
+// and the gather 12 us).
 // ---------------------------------------------------------------------------
 template <int P1>
 __global__ void __launch_bounds__(256) k_stiff(Geom g, const double* __restrict__ tab,
-                                               const double* __restrict__ in,
-                                               double* __restrict__ out, double* part,
-                                               int part_off, const CgState* cg, int color) {
+                                               const double* __restrict__ in, double* __restrict__ ev,
+                                               double* part, const CgState* cg) {
   if (cg && cg->done) return;
   constexpr int P2 = Cfg<P1>::P2, P3 = Cfg<P1>::P3;
+  constexpr int CS = 2 * (P1 / 2) * (P1 / 2) + 2 * (P1 / 2) + 1;
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ double red[8];
   double* sK1 = reinterpret_cast<double*>(smem);
-  double* sMg = sK1 + P2;
-  double* S1 = sMg + P2 + (size_t)threadIdx.y * 4 * P3;
+  double* sMg = sK1 + CS;
+  double* S1 = sMg + CS + (size_t)threadIdx.y * 2 * P3;
   double* S2 = S1 + P3;
-  double* S3 = S2 + P3;
-  double* S4 = S3 + P3;
   const int tid = threadIdx.x + blockDim.x * threadIdx.y;
   const int nthr = blockDim.x * blockDim.y;
-  for (int i = tid; i < P2; i += nthr) {
-    sK1[i] = tab[tab_off_K1(P1) + i];
-    sMg[i] = tab[tab_off_Mg(P1) + i];
+  for (int i = tid; i < CS; i += nthr) {
+    sK1[i] = tab[tab_off_csK1(P1) + i];
+    sMg[i] = tab[tab_off_csMg(P1) + i];
   }
-  const int ta = threadIdx.x % P1, tb = threadIdx.x / P1;
+  const int u = threadIdx.x % P1, v = threadIdx.x / P1;
   int ex = 0, ey = 0, ez = 0;
-  const bool valid = color_elem(g, color, (long long)blockIdx.x * blockDim.y + threadIdx.y, ex, ey, ez);
-  __syncthreads();
+  const long long eidx = (long long)blockIdx.x * blockDim.y + threadIdx.y;
+  const bool valid = plain_elem(g, eidx, ex, ey, ez);
   double cx = 0, cy = 0, cz = 0;
   if (valid) {
     const double hx = g.brk[0][ex + 1] - g.brk[0][ex];
     const double hy = g.brk[1][ey + 1] - g.brk[1][ey];
     const double hz = g.brk[2][ez + 1] - g.brk[2][ez];
-    cx = hy * hz / (2.0 * hx);
-    cy = hx * hz / (2.0 * hy);
-    cz = hx * hy / (2.0 * hz);
+    cx = 0.5 * hy * hz * g.ih[0][ex];
+    cy = 0.5 * hx * hz * g.ih[1][ey];
+    cz = 0.5 * hx * hy * g.ih[2][ez];
   }
-  const int I = ex * g.p + ta, Jn = ey * g.p + tb;
+  const int I = ex * g.p + u, Jn = ey * g.p + v;
   const bool inIJ = valid && I >= 1 && I <= g.nix && Jn >= 1 && Jn <= g.niy;
   const long long base = inIJ ? (long long)(I - 1) + (long long)g.nix * (Jn - 1) : 0;
   const long long plane = (long long)g.nix * g.niy;
-  double u[P1];
+  double w[P1], m[P1], k[P1], t[P1];
 #pragma unroll
   for (int c = 0; c < P1; ++c) {
     const int K = ez * g.p + c;
-    u[c] = (inIJ && K >= 1 && K <= g.niz) ? in[base + plane * (K - 1)] : 0.0;
+    w[c] = (inIJ && K >= 1 && K <= g.niz) ? in[base + plane * (K - 1)] : 0.0;
   }
-  // z: Mg_z u and K1_z u
+  store_line(w, S1 + v * P1 + u, P2);
+  __syncthreads();
+  // x-lines (y = u, z = v): Mg u and K1 u
+  load_line(t, S1 + v * P2 + u * P1, 1);
+  cs_apply<P1>(sMg, t, m);
+  cs_apply<P1>(sK1, t, k);
+  store_line(m, S1 + v * P2 + u * P1, 1);
+  store_line(k, S2 + v * P2 + u * P1, 1);
+  __syncthreads();
+  // y-lines (x = u, z = v): A = Mg Mg u;  C = cx Mg K1_x u + cy K1_y Mg_x u
   {
-    double m1[P1], k1[P1];
+    double A[P1], B[P1];
+    load_line(t, S1 + v * P2 + u, P1);
+    cs_apply<P1>(sMg, t, A);
+    cs_apply<P1>(sK1, t, B);
+    load_line(t, S2 + v * P2 + u, P1);
+    cs_apply<P1>(sMg, t, m);
 #pragma unroll
-    for (int c = 0; c < P1; ++c) {
-      m1[c] = 0.0;
-      k1[c] = 0.0;
-    }
-#pragma unroll
-    for (int c = 0; c < P1; ++c)
-#pragma unroll
-      for (int cc = 0; cc < P1; ++cc) {
-        m1[cc] = fma(sMg[cc * P1 + c], u[c], m1[cc]);
-        k1[cc] = fma(sK1[cc * P1 + c], u[c], k1[cc]);
-      }
-#pragma unroll
-    for (int c = 0; c < P1; ++c) {
-      S1[c * P2 + tb * P1 + ta] = m1[c];
-      S2[c * P2 + tb * P1 + ta] = k1[c];
-    }
+    for (int q = 0; q < P1; ++q) B[q] = fma(cx, m[q], cy * B[q]);
+    store_line(A, S1 + v * P2 + u, P1);
+    store_line(B, S2 + v * P2 + u, P1);
   }
   __syncthreads();
-  // y: thread (a = ta, b' = tb)
-#pragma unroll
-  for (int c = 0; c < P1; ++c) {
-    double A = 0.0, Bv = 0.0, Cv = 0.0;
-#pragma unroll
-    for (int b = 0; b < P1; ++b) {
-      const double s1 = S1[c * P2 + b * P1 + ta];
-      A = fma(sMg[tb * P1 + b], s1, A);
-      Bv = fma(sK1[tb * P1 + b], s1, Bv);
-      Cv = fma(sMg[tb * P1 + b], S2[c * P2 + b * P1 + ta], Cv);
-    }
-    S3[c * P2 + tb * P1 + ta] = A;
-    S4[c * P2 + tb * P1 + ta] = cy * Bv + cz * Cv;
-  }
-  __syncthreads();
+  // z-lines (x = u, y = v): y = Mg C + cz K1 A
+  load_line(t, S1 + v * P1 + u, P2);
+  cs_apply<P1>(sK1, t, k);
+  load_line(t, S2 + v * P1 + u, P2);
+  cs_apply<P1>(sMg, t, m);
   double ppart = 0.0;
 #pragma unroll
   for (int c = 0; c < P1; ++c) {
-    double m = 0.0, k = 0.0;
-#pragma unroll
-    for (int a2 = 0; a2 < P1; ++a2) {
-      m = fma(sMg[ta * P1 + a2], S4[c * P2 + tb * P1 + a2], m);
-      k = fma(sK1[ta * P1 + a2], S3[c * P2 + tb * P1 + a2], k);
-    }
-    const double y = m + cx * k;
-    const int K = ez * g.p + c;
-    if (inIJ && K >= 1 && K <= g.niz) {
-      const long long idx = base + plane * (K - 1);
-      out[idx] += y;
-      ppart = fma(u[c], y, ppart);
-    }
+    m[c] = fma(cz, k[c], m[c]);
+    ppart = fma(w[c], m[c], ppart);     // w is 0 on the boundary
   }
+  if (valid) store_line(m, ev + eidx * P3 + v * P1 + u, P2);
   if (part) {
     const double s = block_sum(ppart, red);
-    if (tid == 0) part[part_off + blockIdx.x] = s;
+    if (tid == 0) part[blockIdx.x] = s;
   }
 }
 
 // ---------------------------------------------------------------------------
-// Load vector out += (B^T)^(x)3 (J W f_q) (real), Eq. 19 right-hand side:
-// x-lines of the Gauss-point field, then y, then z, scatter of the z-column.
+// Load vector (B^T)^(x)3 (J W f_q) (real), Eq. 19 right-hand side: x-lines of the
+// Gauss-point field, then y, then z; element results, assembled by k_gather.
 // ---------------------------------------------------------------------------
 template <int P1>
 __global__ void __launch_bounds__(256) k_load(Geom g, const double* __restrict__ tab,
-                                              const double* __restrict__ fq,
-                                              double* __restrict__ out, double scale, int color,
-                                              int weighted) {
+                                              const double* __restrict__ fq, double* __restrict__ ev,
+                                              double scale, int weighted) {
   constexpr int P2 = Cfg<P1>::P2, P3 = Cfg<P1>::P3;
   constexpr int CS = 2 * (P1 / 2) * (P1 / 2) + 2 * (P1 / 2) + 1;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -1077,7 +1062,8 @@ __global__ void __launch_bounds__(256) k_load(Geom g, const double* __restrict__
   for (int i = tid; i < P1; i += nthr) sw[i] = tab[tab_off_w(P1) + i];
   const int u = threadIdx.x % P1, v = threadIdx.x / P1;
   int ex = 0, ey = 0, ez = 0;
-  const bool valid = color_elem(g, color, (long long)blockIdx.x * blockDim.y + threadIdx.y, ex, ey, ez);
+  const long long eidx = (long long)blockIdx.x * blockDim.y + threadIdx.y;
+  const bool valid = plain_elem(g, eidx, ex, ey, ez);
   __syncthreads();
   double col[P1], t[P1];
 #pragma unroll
@@ -1087,8 +1073,7 @@ __global__ void __launch_bounds__(256) k_load(Geom g, const double* __restrict__
     const double hy = g.brk[1][ey + 1] - g.brk[1][ey];
     const double hz = g.brk[2][ez + 1] - g.brk[2][ez];
     const double Jw = weighted ? 0.125 * hx * hy * hz * scale * sw[u] * sw[v] : scale;
-    const long long e = ex + (long long)g.nx * (ey + (long long)g.ny * ez);
-    const double* fp = fq + e * P3 + v * P2 + u * P1;      // x-line (qy = u, qz = v)
+    const double* fp = fq + eidx * P3 + v * P2 + u * P1;      // x-line (qy = u, qz = v)
 #pragma unroll
     for (int q = 0; q < P1; ++q) col[q] = fp[q] * Jw * (weighted ? sw[q] : 1.0);
   }
@@ -1101,14 +1086,64 @@ __global__ void __launch_bounds__(256) k_load(Geom g, const double* __restrict__
   __syncthreads();
   load_line(col, S2 + v * P1 + u, P2);                    // z-line (a = u, b = v)
   cs_apply<P1>(sBT, col, t);
-  const int I = ex * g.p + u, Jn = ey * g.p + v;
-  const bool inIJ = valid && I >= 1 && I <= g.nix && Jn >= 1 && Jn <= g.niy;
-  const long long base = inIJ ? (long long)(I - 1) + (long long)g.nix * (Jn - 1) : 0;
-  const long long plane = (long long)g.nix * g.niy;
-#pragma unroll
-  for (int c = 0; c < P1; ++c) {
-    const int K = ez * g.p + c;
-    if (inIJ && K >= 1 && K <= g.niz) out[base + plane * (K - 1)] += t[c];
+  if (valid) store_line(t, ev + eidx * P3 + v * P1 + u, P2);
+}
+
+// Assembly of real element results by gathering, each interior node summing its (at most
+// 8) contributions in a fixed order (z, y, x), with the vector work of the CG that follows
+// fused in (kGatherInit, kGatherUpdate: the assembled vector itself is not stored):
+//   kGatherSum     out = sum
+//   kGatherInit    r = b - sum; partials of b . b and r . r
+//   kGatherUpdate  alpha = rz / p . Kp;  x += alpha p;  r -= alpha sum;  partials of r . r
+enum { kGatherSum = 0, kGatherInit = 1, kGatherUpdate = 2 };
+template <int P1, int kMode>
+__global__ void __launch_bounds__(256) k_gather(Geom g, const double* __restrict__ ev, long long n, GatherArgs a) {
+  if (kMode == kGatherUpdate && a.cg->done) return;
+  constexpr int p = P1 - 1, P2 = P1 * P1, P3 = P2 * P1;
+  __shared__ double red[8];
+  double alpha = 0.0, s0 = 0.0, s1 = 0.0;
+  if (kMode == kGatherUpdate) {
+    double v = 0.0;
+    for (int k = threadIdx.x; k < a.n_pAp; k += blockDim.x) v += a.pAp[k];
+    v = block_sum(v, red);
+    __shared__ double tot;
+    if (threadIdx.x == 0) tot = v;
+    __syncthreads();
+    alpha = a.cg->alpha / tot;      // CgState::alpha carries the current r . z here
+  }
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const unsigned iu = (unsigned)i, row = iu / (unsigned)g.nix;   // n < 2^32: the fields of a larger mesh do not fit the device
+    const int I = (int)(iu - row * g.nix) + 1, J = (int)(row % (unsigned)g.niy) + 1, K = (int)(row / (unsigned)g.niy) + 1;
+    int ex[2], ax[2], ey[2], ay[2], ez[2], az[2];
+    const int nx = node_elems(I, p, g.nx, ex, ax), ny = node_elems(J, p, g.ny, ey, ay), nz = node_elems(K, p, g.nz, ez, az);
+    double sum = 0.0;
+    for (int kz = 0; kz < nz; ++kz)
+      for (int ky = 0; ky < ny; ++ky) {
+        const long long eb = (long long)g.nx * (ey[ky] + (long long)g.ny * ez[kz]);
+        const int lb = az[kz] * P2 + ay[ky] * P1;
+        for (int kx = 0; kx < nx; ++kx) sum += ev[(eb + ex[kx]) * P3 + lb + ax[kx]];
+      }
+    if (kMode == kGatherSum) {
+      a.out[i] = sum;
+    } else if (kMode == kGatherInit) {
+      const double bi = a.b[i], ri = bi - sum;
+      a.r[i] = ri;
+      s0 = fma(bi, bi, s0);
+      s1 = fma(ri, ri, s1);
+    } else {
+      a.x[i] = fma(alpha, a.p[i], a.x[i]);
+      const double ri = fma(-alpha, sum, a.r[i]);
+      a.r[i] = ri;
+      s0 = fma(ri, ri, s0);
+    }
+  }
+  if (kMode != kGatherSum) {
+    const double t0 = block_sum(s0, red);
+    if (threadIdx.x == 0) a.part[blockIdx.x] = t0;
+    if (kMode == kGatherInit) {
+      const double t1 = block_sum(s1, red);
+      if (threadIdx.x == 0) a.part[gridDim.x + blockIdx.x] = t1;
+    }
   }
 }
 
@@ -1448,15 +1483,6 @@ __global__ void __launch_bounds__(256) k_cross(Geom g, const double* __restrict_
 // ---------------------------------------------------------------------------
 // launch helpers
 // ---------------------------------------------------------------------------
-long long color_max(const tdks_ctx* c) {
-  return (long long)((c->nx + 1) / 2) * ((c->ny + 1) / 2) * ((c->nz + 1) / 2);
-}
-
-template <int P1>
-int blocks_per_color_t(const tdks_ctx* c) {
-  return (int)((color_max(c) + Cfg<P1>::E - 1) / Cfg<P1>::E);
-}
-
 template <typename K>
 cudaError_t set_smem(K kernel, size_t bytes) {
   if (bytes <= 48 * 1024) return cudaSuccess;
@@ -1545,34 +1571,60 @@ tdks_status hbar_t(tdks_ctx* c, const ApplyArgs& a) {
   return TDKS_OK;
 }
 
+// Elements per CTA of the real element kernels: the full tile once that fills the SMs,
+// fewer on small meshes, where a launch takes as long as one CTA's FP64 work (p = 4, 6^3
+// elements: 18 us with ten elements per CTA, 8 with two)
 template <int P1>
-tdks_status stiff_t(tdks_ctx* c, const double* in, double* out, double* part, const CgState* cg) {
-  constexpr int P2 = Cfg<P1>::P2, P3 = Cfg<P1>::P3, E = Cfg<P1>::E;
-  const size_t smem = (2 * P2 + (size_t)E * 4 * P3) * sizeof(double);
+int elems_per_cta(const tdks_ctx* c) {
+  int E = Cfg<P1>::E;
+  while (E > 1 && (c->n_elem + E - 1) / E < 2 * 152) E = (E + 1) / 2;
+  return E;
+}
+
+template <int P1>
+int stiff_blocks_t(const tdks_ctx* c) {
+  const int E = elems_per_cta<P1>(c);
+  return (int)((c->n_elem + E - 1) / E);
+}
+
+template <int P1>
+tdks_status stiff_t(tdks_ctx* c, const double* in, double* part, const CgState* cg) {
+  constexpr int P2 = Cfg<P1>::P2, P3 = Cfg<P1>::P3;
+  constexpr int CS = 2 * (P1 / 2) * (P1 / 2) + 2 * (P1 / 2) + 1;
+  const int E = elems_per_cta<P1>(c);
+  const size_t smem = (2 * CS + (size_t)E * 2 * P3) * sizeof(double);
   TDKS_CU(c, set_smem(k_stiff<P1>, smem));
-  const int bpc = blocks_per_color_t<P1>(c);
-  dim3 block(P2, E), grid(bpc);
+  k_stiff<P1><<<stiff_blocks_t<P1>(c), dim3(P2, E), smem, c->stream>>>(tdks_geom(c), c->d_tab, in, c->d_sev, part, cg);
+  c->n_launch += 1;
+  TDKS_CU(c, cudaGetLastError());
+  return TDKS_OK;
+}
+
+template <int P1>
+tdks_status gather_t(tdks_ctx* c, const GatherArgs& a, int mode, int nb) {
   const Geom g = tdks_geom(c);
-  for (int color = 0; color < 8; ++color)
-    k_stiff<P1><<<grid, block, smem, c->stream>>>(g, c->d_tab, in, out, part, color * bpc, cg, color);
-  c->n_launch += 8;
+  if (mode == kGatherInit) k_gather<P1, kGatherInit><<<nb, 256, 0, c->stream>>>(g, c->d_sev, c->n_int, a);
+  else if (mode == kGatherUpdate) k_gather<P1, kGatherUpdate><<<nb, 256, 0, c->stream>>>(g, c->d_sev, c->n_int, a);
+  else k_gather<P1, kGatherSum><<<nb, 256, 0, c->stream>>>(g, c->d_sev, c->n_int, a);
+  c->n_launch += 1;
   TDKS_CU(c, cudaGetLastError());
   return TDKS_OK;
 }
 
 template <int P1>
 tdks_status load_t(tdks_ctx* c, const double* fq, double* out, double scale, int weighted) {
-  constexpr int P2 = Cfg<P1>::P2, P3 = Cfg<P1>::P3, E = Cfg<P1>::E;
+  constexpr int P2 = Cfg<P1>::P2, P3 = Cfg<P1>::P3;
   constexpr int CS = 2 * (P1 / 2) * (P1 / 2) + 2 * (P1 / 2) + 1;
+  const int E = elems_per_cta<P1>(c);
   const size_t smem = (CS + P1 + (size_t)E * 2 * P3) * sizeof(double);
   TDKS_CU(c, set_smem(k_load<P1>, smem));
-  dim3 block(P2, E), grid(blocks_per_color_t<P1>(c));
-  const Geom g = tdks_geom(c);
-  for (int color = 0; color < 8; ++color)
-    k_load<P1><<<grid, block, smem, c->stream>>>(g, c->d_tab, fq, out, scale, color, weighted);
-  c->n_launch += 8;
+  k_load<P1><<<stiff_blocks_t<P1>(c), dim3(P2, E), smem, c->stream>>>(tdks_geom(c), c->d_tab, fq, c->d_sev, scale,
+                                                                     weighted);
+  c->n_launch += 1;
   TDKS_CU(c, cudaGetLastError());
-  return TDKS_OK;
+  GatherArgs a{};
+  a.out = out;
+  return gather_t<P1>(c, a, kGatherSum, gather_blocks(c));
 }
 
 template <int P1>
@@ -1682,7 +1734,7 @@ tdks_status ensure_evec(tdks_ctx* c, int n_orb) {
   return TDKS_OK;
 }
 
-int hbar_blocks_per_color(const tdks_ctx* c) {
+int hbar_blocks(const tdks_ctx* c) {
   int b = 0;
   switch (c->P1) {
     case 2: b = elem_blocks_t<2>(c); break;
@@ -1695,13 +1747,18 @@ int hbar_blocks_per_color(const tdks_ctx* c) {
     case 9: b = elem_blocks_t<9>(c); break;
     default: break;
   }
-  const int bs = stiff_blocks_per_color(c);
+  const int bs = stiff_blocks(c);
   return b > bs ? b : bs;
 }
 
-int stiff_blocks_per_color(const tdks_ctx* c) {
-  TDKS_DISPATCH(c->P1, blocks_per_color_t<P1>(c));
+int stiff_blocks(const tdks_ctx* c) {
+  TDKS_DISPATCH(c->P1, stiff_blocks_t<P1>(c));
   return 0;
+}
+
+int gather_blocks(const tdks_ctx* c) {
+  const long long b = (c->n_int + 255) / 256;
+  return (int)(b < 608 ? b : 608);
 }
 
 int assemble_blocks(const tdks_ctx* c, int n_orb) {
@@ -1727,9 +1784,13 @@ tdks_status launch_hbar_apply(tdks_ctx* c, const ApplyArgs& a, int prec) {
   return tdks_fail(c, TDKS_ERR_ARG, "unsupported degree");
 }
 
-tdks_status launch_stiffness(tdks_ctx* c, const double* in, double* out, double* part,
-                             const CgState* cg) {
-  TDKS_DISPATCH(c->P1, (stiff_t<P1>(c, in, out, part, cg)));
+tdks_status launch_stiffness(tdks_ctx* c, const double* in, double* part, const CgState* cg) {
+  TDKS_DISPATCH(c->P1, (stiff_t<P1>(c, in, part, cg)));
+  return tdks_fail(c, TDKS_ERR_ARG, "unsupported degree");
+}
+
+tdks_status launch_gather(tdks_ctx* c, const GatherArgs& a, int mode) {
+  TDKS_DISPATCH(c->P1, (gather_t<P1>(c, a, mode, gather_blocks(c))));
   return tdks_fail(c, TDKS_ERR_ARG, "unsupported degree");
 }
 

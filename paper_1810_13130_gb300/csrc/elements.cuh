@@ -286,25 +286,6 @@ __device__ __forceinline__ void store_line(const V (&r)[N], V* dst, int stride) 
   for (int i = 0; i < N; ++i) dst[i * stride] = r[i];
 }
 
-// Element of a parity colour: colour bits (cx, cy, cz) select ex = cx + 2 gx etc.
-// Elements of one colour share no node, so a launch can read-modify-write its
-// nodes without atomics; eight launches cover the mesh in a fixed order.
-__device__ __forceinline__ bool color_elem(const Geom& g, int color, long long gidx, int& ex,
-                                           int& ey, int& ez) {
-  const int cx = color & 1, cy = (color >> 1) & 1, cz = (color >> 2) & 1;
-  const int ncx = (g.nx - cx + 1) >> 1, ncy = (g.ny - cy + 1) >> 1, ncz = (g.nz - cz + 1) >> 1;
-  const long long tot = (long long)ncx * ncy * ncz;
-  if (gidx < 0 || gidx >= tot) return false;
-  const int gx = (int)(gidx % ncx);
-  const long long r = gidx / ncx;
-  const int gy = (int)(r % ncy);
-  const int gz = (int)(r / ncy);
-  ex = cx + 2 * gx;
-  ey = cy + 2 * gy;
-  ez = cz + 2 * gz;
-  return true;
-}
-
 __device__ __forceinline__ bool plain_elem(const Geom& g, long long gidx, int& ex, int& ey,
                                            int& ez) {
   const long long tot = (long long)g.nx * g.ny * g.nz;

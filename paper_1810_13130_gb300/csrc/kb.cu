@@ -459,7 +459,6 @@ extern "C" tdks_status tdks_set_kb(tdks_ctx* c, int n_atoms, const double* R, do
       k_kb_fields<<<nbq, kThreads, 0, c->stream>>>(g, eta, c->P1, nq, R[3 * I], R[3 * I + 1], R[3 * I + 2], m,
                                                    a, b, cl[l], chi, udu);
       k_kb_wsum<<<nbq, kThreads, 0, c->stream>>>(g, w, c->P1, nq, udu, part);
-      cudaMemsetAsync(col, 0, n * sizeof(double), c->stream);
       tdks_status st = launch_load_vector(c, chi, col, 1.0, 1);
       if (st != TDKS_OK) {
         cleanup();

@@ -1148,7 +1148,7 @@ tdks_status run_expm_ws(tdks_ctx* c, int w, const double2* in, double2* out, int
   if (kmax < 1 || kmax > TDKS_KMAX) return tdks_fail(c, TDKS_ERR_ARG, "k_max must be in [1, 128]");
   if (n_orb < 1 || n_orb > c->n_orb) return tdks_fail(c, TDKS_ERR_ARG, "n_orb out of range");
   const long long n = c->n_int;
-  const int bpc = hbar_blocks_per_color(c);
+  const int bpc = hbar_blocks(c);
   TDKS_TRY(ensure_part(c, n_orb, 8 * (int64_t)bpc));
   TDKS_TRY(ensure_krylov(c, w, n_orb, kmax));
   if (c->lanczos_reorth) TDKS_TRY(ensure_reorth(c));

@@ -75,24 +75,6 @@ __global__ void k_invdiag(long long n, int nix, int niy, const double* kx, const
   }
 }
 
-// r = b - Ap; partials of b.b and r.r
-__global__ void k_cg_init(long long n, const double* b, const double* Ap, double* r, double* part) {
-  __shared__ double red[2 * kThreads / 32];
-  double bb = 0.0, rr = 0.0;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x) {
-    const double ri = b[i] - Ap[i];
-    r[i] = ri;
-    bb = fma(b[i], b[i], bb);
-    rr = fma(ri, ri, rr);
-  }
-  block_sum2(bb, rr, red);
-  if (threadIdx.x == 0) {
-    part[blockIdx.x] = bb;
-    part[gridDim.x + blockIdx.x] = rr;
-  }
-}
-
 __global__ void k_cg_init_fin(const double* part, int nb, double tol, CgState* cg) {
   const double bb = sum_fixed(part, nb);
   const double rr = sum_fixed(part + nb, nb);
@@ -131,47 +113,17 @@ __global__ void k_dot_part(long long n, const double* r, const double* z, double
   if (threadIdx.x == 0) part[blockIdx.x] = a;
 }
 
-// rz_new = r.z; beta = rz_new / rz (unused for the first direction)
-__global__ void k_cg_fin_rz(const double* part, int nb, CgState* cg) {
+// rz_new = r.z, beta = rz_new / rz, p = z + beta p (p = z for the first direction).  Every
+// block sums the partials; rz is moved on by k_cg_fin_rr, when no block reads it any more.
+__global__ void k_cg_dir(long long n, const double* part, int nb, const double* z, double* p, CgState* cg) {
   if (cg->done) return;
   const double rz = sum_fixed(part, nb);
-  if (threadIdx.x == 0) {
-    cg->alpha = cg->first ? 0.0 : rz / cg->rz;
-    cg->rz = rz;
-  }
-}
-
-// p = z + beta p  (p = z for the first direction)
-__global__ void k_cg_dir(long long n, const double* z, double* p, const CgState* cg) {
-  if (cg->done) return;
-  const double beta = cg->alpha;
   const bool first = cg->first != 0;
+  const double beta = first ? 0.0 : rz / cg->rz;
+  if (blockIdx.x == 0 && threadIdx.x == 0) cg->alpha = rz;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x)
     p[i] = first ? z[i] : fma(beta, p[i], z[i]);
-}
-
-__global__ void k_cg_clear_first(CgState* cg) {
-  if (!cg->done) cg->first = 0;
-}
-
-// alpha = rz / p.Kp;  x += alpha p;  r -= alpha Ap;  partial r.r
-__global__ void k_cg_update(long long n, const double* pAp_part, int npart, double* x, double* r,
-                            const double* p, const double* Ap, double* part, const CgState* cg) {
-  if (cg->done) return;
-  __shared__ double red[2 * kThreads / 32];
-  const double pAp = sum_fixed(pAp_part, npart);
-  const double alpha = cg->rz / pAp;
-  double rr = 0.0, dummy = 0.0;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x) {
-    x[i] = fma(alpha, p[i], x[i]);
-    const double ri = fma(-alpha, Ap[i], r[i]);
-    r[i] = ri;
-    rr = fma(ri, ri, rr);
-  }
-  block_sum2(rr, dummy, red);
-  if (threadIdx.x == 0) part[blockIdx.x] = rr;
 }
 
 __global__ void k_cg_fin_rr(const double* part, int nb, double tol, int maxit, CgState* cg) {
@@ -179,6 +131,8 @@ __global__ void k_cg_fin_rr(const double* part, int nb, double tol, int maxit, C
   const double rr = sum_fixed(part, nb);
   if (threadIdx.x == 0) {
     cg->rr = rr;
+    cg->rz = cg->alpha;
+    cg->first = 0;
     cg->iters += 1;
     if (!isfinite(rr)) {
       cg->failed = 1;
@@ -203,11 +157,15 @@ struct Gemm {
   int M, N, K;
 };
 
-constexpr int GT = 64;   // output tile
 constexpr int GK = 16;   // depth tile
 
+// GT x GT output tile, 16 x 16 threads of (GT / 16)^2 outputs.  The product is bound by the
+// FP64 pipe whatever the tile, so the tile only decides how much of the work is padding and
+// how it spreads over the SMs (gemm_tile).
+template <int GT>
 __global__ void __launch_bounds__(256) k_gemm(Gemm g, const CgState* cg) {
   if (cg && cg->done) return;
+  constexpr int R = GT / 16;
   __shared__ double As[GK][GT + 1];
   __shared__ double Bs[GK][GT + 1];
   const int tid = threadIdx.x;
@@ -216,11 +174,11 @@ __global__ void __launch_bounds__(256) k_gemm(Gemm g, const CgState* cg) {
   const int m0 = blockIdx.y * GT, n0 = blockIdx.x * GT;
   const double* A = g.A + b * g.sAb;
   const double* B = g.B + b * g.sBb;
-  double acc[4][4];
+  double acc[R][R];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < R; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
+    for (int j = 0; j < R; ++j) acc[i][j] = 0.0;
   const bool a_k_fast = (g.sAk == 1);
   const bool b_n_fast = (g.sBn == 1);
   for (int k0 = 0; k0 < g.K; k0 += GK) {
@@ -251,26 +209,26 @@ __global__ void __launch_bounds__(256) k_gemm(Gemm g, const CgState* cg) {
     __syncthreads();
 #pragma unroll
     for (int kk = 0; kk < GK; ++kk) {
-      double a[4], bb[4];
+      double a[R], bb[R];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
+      for (int i = 0; i < R; ++i) a[i] = As[kk][ty * R + i];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) bb[j] = Bs[kk][tx * 4 + j];
+      for (int j = 0; j < R; ++j) bb[j] = Bs[kk][tx * R + j];
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < R; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], bb[j], acc[i][j]);
+        for (int j = 0; j < R; ++j) acc[i][j] = fma(a[i], bb[j], acc[i][j]);
     }
     __syncthreads();
   }
   double* C = g.C + b * g.sCb;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const long long gm = m0 + ty * 4 + i;
+  for (int i = 0; i < R; ++i) {
+    const long long gm = m0 + ty * R + i;
     if (gm >= g.M) continue;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const long long gn = n0 + tx * 4 + j;
+    for (int j = 0; j < R; ++j) {
+      const long long gn = n0 + tx * R + j;
       if (gn < g.N) C[gm * g.sCm + gn * g.sCn] = acc[i][j];
     }
   }
@@ -293,8 +251,10 @@ __device__ __forceinline__ void gemm_dfa(float& hi, float& err, Df a, Df b) {
   hi = s;
 }
 
+template <int GT>
 __global__ void __launch_bounds__(256) k_gemm_df(Gemm g, const CgState* cg) {
   if (cg && cg->done) return;
+  constexpr int R = GT / 16;
   __shared__ Df As[GK][GT + 1];
   __shared__ Df Bs[GK][GT + 1];
   const int tid = threadIdx.x;
@@ -303,11 +263,11 @@ __global__ void __launch_bounds__(256) k_gemm_df(Gemm g, const CgState* cg) {
   const int m0 = blockIdx.y * GT, n0 = blockIdx.x * GT;
   const double* A = g.A + b * g.sAb;
   const double* B = g.B + b * g.sBb;
-  float hi[4][4], er[4][4];
+  float hi[R][R], er[R][R];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < R; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
+    for (int j = 0; j < R; ++j) {
       hi[i][j] = 0.0f;
       er[i][j] = 0.0f;
     }
@@ -341,26 +301,26 @@ __global__ void __launch_bounds__(256) k_gemm_df(Gemm g, const CgState* cg) {
     __syncthreads();
 #pragma unroll 4
     for (int kk = 0; kk < GK; ++kk) {
-      Df a[4], bb[4];
+      Df a[R], bb[R];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
+      for (int i = 0; i < R; ++i) a[i] = As[kk][ty * R + i];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) bb[j] = Bs[kk][tx * 4 + j];
+      for (int j = 0; j < R; ++j) bb[j] = Bs[kk][tx * R + j];
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < R; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) gemm_dfa(hi[i][j], er[i][j], a[i], bb[j]);
+        for (int j = 0; j < R; ++j) gemm_dfa(hi[i][j], er[i][j], a[i], bb[j]);
     }
     __syncthreads();
   }
   double* C = g.C + b * g.sCb;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const long long gm = m0 + ty * 4 + i;
+  for (int i = 0; i < R; ++i) {
+    const long long gm = m0 + ty * R + i;
     if (gm >= g.M) continue;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const long long gn = n0 + tx * 4 + j;
+    for (int j = 0; j < R; ++j) {
+      const long long gn = n0 + tx * R + j;
       if (gn < g.N) {
         const Df r = tdks::df_norm(hi[i][j], er[i][j]);
         C[gm * g.sCm + gn * g.sCn] = (double)r.hi + (double)r.lo;
@@ -387,6 +347,24 @@ int grid_for(long long n) {
   return (int)(b < kBlocks ? (b < 1 ? 1 : b) : kBlocks);
 }
 
+// Output tile of an M x N product (batch b): the least work of the busiest SM, counted in
+// outputs of whole tiles (152 SMs); the larger tile on a tie (fewer shared-memory loads).
+// 95 x 9025 (p = 6, 16^3 elements): 64 pads 95 to 128, 32 to 96: 134 -> 104 us a product;
+// 23 x 529 (p = 4, 6^3): 9 CTAs of 64 against 68 of 16: 18.5 -> 4 us.
+int gemm_tile(long long M, long long N, long long b) {
+  int best = 64;
+  long long cost = -1;
+  for (int t : {64, 32, 16}) {
+    const long long ctas = ((M + t - 1) / t) * ((N + t - 1) / t) * b;
+    const long long c = ((ctas + 151) / 152) * t * t;
+    if (cost < 0 || c < cost) {
+      cost = c;
+      best = t;
+    }
+  }
+  return best;
+}
+
 // out = transform of `in` along `axis` with S (n_a x n_a, row-major [i][mode]):
 // forward out[.., mode, ..] = sum_i S[i][mode] in[.., i, ..]; backward uses S^T.
 void axis_gemm(tdks_ctx* c, int axis, bool forward, const double* in, double* out,
@@ -395,7 +373,7 @@ void axis_gemm(tdks_ctx* c, int axis, bool forward, const double* in, double* ou
   const double* S = c->d_fdmS[axis];
   const long long na = c->Ni[axis];
   Gemm g{};
-  dim3 grid;
+  long long batch = 1;
   if (axis == 0) {
     // rows (j,k): C[row][mode] = sum_i V[row][i] S[i][mode]
     g.A = in;
@@ -413,7 +391,6 @@ void axis_gemm(tdks_ctx* c, int axis, bool forward, const double* in, double* ou
     g.M = (int)(ny * nz);
     g.N = (int)nx;
     g.K = (int)nx;
-    grid = dim3((g.N + GT - 1) / GT, (g.M + GT - 1) / GT, 1);
   } else if (axis == 1) {
     // per z-slab: C[mode][i] = sum_j S[j][mode] V[j][i]
     g.A = S;
@@ -431,7 +408,7 @@ void axis_gemm(tdks_ctx* c, int axis, bool forward, const double* in, double* ou
     g.M = (int)ny;
     g.N = (int)nx;
     g.K = (int)ny;
-    grid = dim3((g.N + GT - 1) / GT, (g.M + GT - 1) / GT, (unsigned)nz);
+    batch = nz;
   } else {
     // C[mode][(i,j)] = sum_k S[k][mode] V[k][(i,j)]
     g.A = S;
@@ -449,12 +426,12 @@ void axis_gemm(tdks_ctx* c, int axis, bool forward, const double* in, double* ou
     g.M = (int)nz;
     g.N = (int)(nx * ny);
     g.K = (int)nz;
-    grid = dim3((g.N + GT - 1) / GT, (g.M + GT - 1) / GT, 1);
   }
-  if (df)
-    k_gemm_df<<<grid, 256, 0, c->stream>>>(g, cg);
-  else
-    k_gemm<<<grid, 256, 0, c->stream>>>(g, cg);
+  const int t = gemm_tile(g.M, g.N, batch);
+  const dim3 grid((g.N + t - 1) / t, (g.M + t - 1) / t, (unsigned)batch);
+  const auto go = [&](auto* kernel) { kernel<<<grid, 256, 0, c->stream>>>(g, cg); };
+  if (df) go(t == 64 ? k_gemm_df<64> : t == 32 ? k_gemm_df<32> : k_gemm_df<16>);
+  else go(t == 64 ? k_gemm<64> : t == 32 ? k_gemm<32> : k_gemm<16>);
 }
 
 // z = S D^-1 S^T r  (exact inverse of the separable stiffness)
@@ -531,52 +508,65 @@ tdks_status poisson_setup(tdks_ctx* c, const Tables1D& t) {
   return TDKS_OK;
 }
 
+// One iteration of the CG above, and its start: z = P^-1 r; rz = r.z; p = z + beta p;
+// alpha = rz / p.Kp; x += alpha p; r -= alpha Kp.  Three launches besides the preconditioner:
+// K p element by element, the gather with the vector updates, the stopping test.
+static tdks_status cg_start(tdks_ctx* c, const double* b, const double* x, double* part_vec) {
+  TDKS_TRY(launch_stiffness(c, x, nullptr, nullptr));
+  GatherArgs a{};
+  a.b = b;
+  a.r = c->d_r;
+  a.part = part_vec;
+  TDKS_TRY(launch_gather(c, a, 1));
+  k_cg_init_fin<<<1, kThreads, 0, c->stream>>>(part_vec, gather_blocks(c), c->cg_tol, c->d_cg);
+  c->n_launch += 1;
+  TDKS_CU(c, cudaGetLastError());
+  return TDKS_OK;
+}
+
+static tdks_status cg_iteration(tdks_ctx* c, double* x, double* part_pAp, double* part_vec, bool fdm, bool df) {
+  const long long n = c->n_int;
+  const int nb = grid_for(n);
+  CgState* cg = c->d_cg;
+  if (fdm) {
+    fdm_apply(c, c->d_r, c->d_z, cg, df);
+  } else {
+    k_jacobi<<<nb, kThreads, 0, c->stream>>>(n, c->d_r, c->d_invdiag, c->d_z, cg);
+    c->n_launch += 1;
+  }
+  k_dot_part<<<nb, kThreads, 0, c->stream>>>(n, c->d_r, c->d_z, part_vec, cg);
+  k_cg_dir<<<nb, kThreads, 0, c->stream>>>(n, part_vec, nb, c->d_z, c->d_pv, cg);
+  TDKS_TRY(launch_stiffness(c, c->d_pv, part_pAp, cg));
+  GatherArgs a{};
+  a.r = c->d_r;
+  a.x = x;
+  a.p = c->d_pv;
+  a.pAp = part_pAp;
+  a.n_pAp = stiff_blocks(c);
+  a.part = part_vec;
+  a.cg = cg;
+  TDKS_TRY(launch_gather(c, a, 2));
+  k_cg_fin_rr<<<1, kThreads, 0, c->stream>>>(part_vec, gather_blocks(c), c->cg_tol, c->cg_maxit, cg);
+  c->n_launch += 3;
+  TDKS_CU(c, cudaGetLastError());
+  return TDKS_OK;
+}
+
 // Solve K x = b by the preconditioned CG above; x holds the initial guess.
 tdks_status run_cg_solve(tdks_ctx* c, const double* b, double* x, int* iters, bool df) {
   const long long n = c->n_int;
-  const int nb = grid_for(n);
-  const int sbpc = stiff_blocks_per_color(c);
   const bool fdm = (c->cg_precond == 0 && c->fdm_ok);
-  double* part_pAp = c->d_part;                       // 8 * sbpc
-  double* part_vec = c->d_part + 8 * (int64_t)sbpc;   // 2 * nb
-  CgState* cg = c->d_cg;
-  // r = b - K x0
-  TDKS_CU(c, cudaMemsetAsync(c->d_Ap, 0, n * sizeof(double), c->stream));
-  TDKS_TRY(launch_stiffness(c, x, c->d_Ap, nullptr, nullptr));
-  k_cg_init<<<nb, kThreads, 0, c->stream>>>(n, b, c->d_Ap, c->d_r, part_vec);
-  k_cg_init_fin<<<1, kThreads, 0, c->stream>>>(part_vec, nb, c->cg_tol, cg);
-  c->n_launch += 2;
-  // z = P^-1 r; rz = r.z; p = z (first direction) or z + beta p
-  auto precondition = [&]() {
-    if (fdm) {
-      fdm_apply(c, c->d_r, c->d_z, cg, df);
-    } else {
-      k_jacobi<<<nb, kThreads, 0, c->stream>>>(n, c->d_r, c->d_invdiag, c->d_z, cg);
-      c->n_launch += 1;
-    }
-    k_dot_part<<<nb, kThreads, 0, c->stream>>>(n, c->d_r, c->d_z, part_vec, cg);
-    k_cg_fin_rz<<<1, kThreads, 0, c->stream>>>(part_vec, nb, cg);
-    k_cg_dir<<<nb, kThreads, 0, c->stream>>>(n, c->d_z, c->d_pv, cg);
-    k_cg_clear_first<<<1, 1, 0, c->stream>>>(cg);
-    c->n_launch += 4;
-  };
-  precondition();
-  TDKS_CU(c, cudaGetLastError());
+  double* part_pAp = c->d_part;                          // stiff_blocks
+  double* part_vec = c->d_part + stiff_blocks(c);        // 2 * grid
+  TDKS_TRY(cg_start(c, b, x, part_vec));
   int it = 0, next_poll = 1;
   CgState host{};
   while (true) {
     while (it < next_poll) {
-      TDKS_CU(c, cudaMemsetAsync(c->d_Ap, 0, n * sizeof(double), c->stream));
-      TDKS_TRY(launch_stiffness(c, c->d_pv, c->d_Ap, part_pAp, cg));
-      k_cg_update<<<nb, kThreads, 0, c->stream>>>(n, part_pAp, 8 * sbpc, x, c->d_r, c->d_pv,
-                                                  c->d_Ap, part_vec, cg);
-      k_cg_fin_rr<<<1, kThreads, 0, c->stream>>>(part_vec, nb, c->cg_tol, c->cg_maxit, cg);
-      c->n_launch += 2;
-      precondition();
+      TDKS_TRY(cg_iteration(c, x, part_pAp, part_vec, fdm, df));
       ++it;
     }
-    TDKS_CU(c, cudaGetLastError());
-    TDKS_CU(c, cudaMemcpyAsync(&host, cg, sizeof(CgState), cudaMemcpyDeviceToHost, c->stream));
+    TDKS_CU(c, cudaMemcpyAsync(&host, c->d_cg, sizeof(CgState), cudaMemcpyDeviceToHost, c->stream));
     TDKS_CU(c, cudaStreamSynchronize(c->stream));
     if (host.done) break;
     if (it > c->cg_maxit + 32) break;
@@ -595,9 +585,7 @@ tdks_status run_cg_solve(tdks_ctx* c, const double* b, double* x, int* iters, bo
 }
 
 tdks_status run_hartree(tdks_ctx* c, const double* rho_q, double* vh_q, int* iters, bool df) {
-  const long long n = c->n_int;
   // b = 4 pi c
-  TDKS_CU(c, cudaMemsetAsync(c->d_b, 0, n * sizeof(double), c->stream));
   TDKS_TRY(launch_load_vector(c, rho_q, c->d_b, 4.0 * M_PI));
   TDKS_TRY(run_cg_solve(c, c->d_b, c->d_phi, iters, df));
   TDKS_TRY(launch_interp(c, c->d_phi, vh_q));
@@ -612,40 +600,16 @@ tdks_status run_hartree(tdks_ctx* c, const double* rho_q, double* vh_q, int* ite
 tdks_status cg_solve_graph(tdks_ctx* c, const double* b, double* x, int n_iter, int* err, bool df) {
   if (!(c->cg_precond == 0 && c->fdm_ok))
     return tdks_fail(c, TDKS_ERR_ARG, "graph CG needs the fast-diagonalization preconditioner");
-  const long long n = c->n_int;
-  const int nb = grid_for(n);
-  const int sbpc = stiff_blocks_per_color(c);
   double* part_pAp = c->d_part;
-  double* part_vec = c->d_part + 8 * (int64_t)sbpc;
-  CgState* cg = c->d_cg;
-  TDKS_CU(c, cudaMemsetAsync(c->d_Ap, 0, n * sizeof(double), c->stream));
-  TDKS_TRY(launch_stiffness(c, x, c->d_Ap, nullptr, nullptr));
-  k_cg_init<<<nb, kThreads, 0, c->stream>>>(n, b, c->d_Ap, c->d_r, part_vec);
-  k_cg_init_fin<<<1, kThreads, 0, c->stream>>>(part_vec, nb, c->cg_tol, cg);
-  auto precondition = [&]() {
-    fdm_apply(c, c->d_r, c->d_z, cg, df);
-    k_dot_part<<<nb, kThreads, 0, c->stream>>>(n, c->d_r, c->d_z, part_vec, cg);
-    k_cg_fin_rz<<<1, kThreads, 0, c->stream>>>(part_vec, nb, cg);
-    k_cg_dir<<<nb, kThreads, 0, c->stream>>>(n, c->d_z, c->d_pv, cg);
-    k_cg_clear_first<<<1, 1, 0, c->stream>>>(cg);
-  };
-  precondition();
-  for (int it = 0; it < n_iter; ++it) {
-    TDKS_CU(c, cudaMemsetAsync(c->d_Ap, 0, n * sizeof(double), c->stream));
-    TDKS_TRY(launch_stiffness(c, c->d_pv, c->d_Ap, part_pAp, cg));
-    k_cg_update<<<nb, kThreads, 0, c->stream>>>(n, part_pAp, 8 * sbpc, x, c->d_r, c->d_pv, c->d_Ap,
-                                                part_vec, cg);
-    k_cg_fin_rr<<<1, kThreads, 0, c->stream>>>(part_vec, nb, c->cg_tol, c->cg_maxit, cg);
-    precondition();
-  }
-  k_cg_graph_end<<<nb, kThreads, 0, c->stream>>>(n, x, cg, err);
+  double* part_vec = c->d_part + stiff_blocks(c);
+  TDKS_TRY(cg_start(c, b, x, part_vec));
+  for (int it = 0; it < n_iter; ++it) TDKS_TRY(cg_iteration(c, x, part_pAp, part_vec, true, df));
+  k_cg_graph_end<<<grid_for(c->n_int), kThreads, 0, c->stream>>>(c->n_int, x, c->d_cg, err);
   TDKS_CU(c, cudaGetLastError());
   return TDKS_OK;
 }
 
 tdks_status hartree_graph(tdks_ctx* c, const double* rho_q, double* vh_q, int n_iter, int* err, bool df) {
-  const long long n = c->n_int;
-  TDKS_CU(c, cudaMemsetAsync(c->d_b, 0, n * sizeof(double), c->stream));
   TDKS_TRY(launch_load_vector(c, rho_q, c->d_b, 4.0 * M_PI));
   TDKS_TRY(cg_solve_graph(c, c->d_b, c->d_phi, n_iter, err, df));
   TDKS_TRY(launch_interp(c, c->d_phi, vh_q));

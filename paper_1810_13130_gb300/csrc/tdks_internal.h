@@ -48,9 +48,9 @@ enum { KRY_ACTIVE = 0, KRY_CONVERGED = 1, KRY_SUBSTEP = 2, KRY_DONE = 3, KRY_FAI
 // CG state, resident in device memory.
 struct CgState {
   double bb;        // ||b||^2
-  double rz;        // r.z of the current iterate
+  double rz;        // r.z of the previous residual
   double rr;        // ||r||^2
-  double alpha;     // CG step length; carries beta between the last two kernels
+  double alpha;     // r.z of the current residual, while rz still holds the previous one
   int iters;
   int done;         // 1 when converged
   int failed;
@@ -112,7 +112,8 @@ struct tdks_ctx {
   double *d_vks = nullptr, *d_vnuc = nullptr, *d_vhxc1 = nullptr, *d_vhxc2 = nullptr;
   double *d_vtmp = nullptr, *d_rho = nullptr, *d_vh = nullptr;
   // Poisson
-  double *d_phi = nullptr, *d_b = nullptr, *d_r = nullptr, *d_pv = nullptr, *d_Ap = nullptr;
+  double *d_phi = nullptr, *d_b = nullptr, *d_r = nullptr, *d_pv = nullptr;
+  double* d_sev = nullptr;     // element results of the stiffness and load kernels [n_elem][P1^3]
   CgState* d_cg = nullptr;
   double cg_tol = 1e-12;
   int cg_maxit = 5000;
@@ -213,7 +214,8 @@ TDKS_HD inline int tab_off_csBT(int P1) { return tab_off_csB(P1) + cs_size(P1); 
 TDKS_HD inline int tab_off_csK(int P1) { return tab_off_csBT(P1) + cs_size(P1); }
 TDKS_HD inline int tab_off_wl(int P1) { return tab_off_csK(P1) + cs_size(P1); }   // GLL weights
 TDKS_HD inline int tab_off_csK1(int P1) { return tab_off_wl(P1) + P1; }            // folded K1
-TDKS_HD inline int tab_size(int P1) { return tab_off_csK1(P1) + cs_size(P1); }
+TDKS_HD inline int tab_off_csMg(int P1) { return tab_off_csK1(P1) + cs_size(P1); } // folded Mg
+TDKS_HD inline int tab_size(int P1) { return tab_off_csMg(P1) + cs_size(P1); }
 
 // ---------------------------------------------------------------- launchers
 // element kernels (elements.cu)
@@ -240,8 +242,21 @@ tdks_status launch_hbar_apply(tdks_ctx* c, const ApplyArgs& a, int prec);
 // CTA (bpe CTAs) and opc orbitals per CTA; results and alpha as described there
 cudaError_t launch_hbar_fx(int P1, const Geom& g, const tdks::FxHost& h, const double* vks, const ApplyArgs& a,
                            int E, int bpe, int opc, double2* ev, cudaStream_t st);
-tdks_status launch_stiffness(tdks_ctx* c, const double* in, double* out, double* part,
-                             const CgState* cg);
+// element results of K in (c->d_sev), per-CTA partials of in . K in (stiff_blocks of them)
+tdks_status launch_stiffness(tdks_ctx* c, const double* in, double* part, const CgState* cg);
+// gather of the element results in c->d_sev with fused CG vector work (modes in elements.cu)
+struct GatherArgs {
+  double* out;                 // mode 0: assembled vector
+  const double* b;             // mode 1: right-hand side
+  double *r, *x;               // modes 1, 2: residual; mode 2: solution
+  const double* p;             // mode 2: direction
+  const double* pAp;           // mode 2: partials of p . K p
+  int n_pAp;
+  double* part;                // modes 1, 2: partial sums (gather_blocks, twice in mode 1)
+  const CgState* cg;
+};
+tdks_status launch_gather(tdks_ctx* c, const GatherArgs& a, int mode);
+int gather_blocks(const tdks_ctx* c);
 tdks_status launch_load_vector(tdks_ctx* c, const double* f_q, double* out, double scale,
                                int weighted = 1);
 tdks_status launch_interp(tdks_ctx* c, const double* nodal, double* f_q, double scale = 1.0,
@@ -257,9 +272,9 @@ tdks_status launch_cross(tdks_ctx* c, const double2* mu, const double2* phi, int
 // any other value: FP64 throughout
 tdks_status launch_density(tdks_ctx* c, const double2* psi, int n_orb, double* rho_q,
                            int prec = TDKS_FP64);
-int hbar_blocks_per_color(const tdks_ctx* c);
+int hbar_blocks(const tdks_ctx* c);
 int assemble_blocks(const tdks_ctx* c, int n_orb);   // partial-sum count of the fused update
-int stiff_blocks_per_color(const tdks_ctx* c);
+int stiff_blocks(const tdks_ctx* c);
 
 // magnus step with optional recording of the intermediates (capi.cu)
 tdks_status magnus_step_impl(tdks_ctx* c, double2* psi, int n_orb, double dt, const double Eq[3],
