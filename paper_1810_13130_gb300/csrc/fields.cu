@@ -204,22 +204,25 @@ __global__ void k_dipole_part(Geom g, const double* eta, const double* w, int P1
   }
 }
 
+// one warp per component, a fixed order
+__device__ __forceinline__ double warp_sum_parts(const double* part, int nb) {
+  const int lane = threadIdx.x & 31;
+  double v = 0.0;
+  for (int k = lane; k < nb; k += 32) v += part[(threadIdx.x >> 5) * nb + k];
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+  return v;
+}
+
 __global__ void k_sum_parts3(const double* part, int nb, double* out) {
-  if (threadIdx.x < 3) {
-    double s = 0.0;
-    for (int k = 0; k < nb; ++k) s += part[threadIdx.x * nb + k];
-    out[threadIdx.x] = s;
-  }
+  const double s = warp_sum_parts(part, nb);
+  if ((threadIdx.x & 31) == 0) out[threadIdx.x >> 5] = s;
 }
 
 // d = sum of the partials, written to base + (*step) * stride (step counter on the device)
 __global__ void k_sum_parts3_at(const double* part, int nb, double* base, const int* step,
                                 int64_t stride) {
-  if (threadIdx.x < 3) {
-    double s = 0.0;
-    for (int k = 0; k < nb; ++k) s += part[threadIdx.x * nb + k];
-    base[(long long)(*step) * stride + threadIdx.x] = s;
-  }
+  const double s = warp_sum_parts(part, nb);
+  if ((threadIdx.x & 31) == 0) base[(long long)(*step) * stride + (threadIdx.x >> 5)] = s;
 }
 
 __global__ void k_counter_add(int* counter, int inc) {
@@ -309,7 +312,7 @@ tdks_status run_dipole(tdks_ctx* c, const double* rho, double d[3], int weighted
   k_dipole_part<<<nb, kVecThreads, 0, c->stream>>>(tdks_geom(c), c->d_tab + tab_off_eta(c->P1),
                                                    c->d_tab + tab_off_w(c->P1), c->P1, n, rho, part,
                                                    weighted);
-  k_sum_parts3<<<1, 32, 0, c->stream>>>(part, nb, out);
+  k_sum_parts3<<<1, 96, 0, c->stream>>>(part, nb, out);
   c->n_launch += 2;
   TDKS_CU(c, cudaGetLastError());
   TDKS_CU(c, cudaMemcpyAsync(c->h_red, out, 3 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
@@ -335,7 +338,7 @@ tdks_status dipole_graph(tdks_ctx* c, const double* rho, double* base, const int
   double* part = c->d_part;
   k_dipole_part<<<nb, kVecThreads, 0, c->stream>>>(tdks_geom(c), c->d_tab + tab_off_eta(c->P1),
                                                    c->d_tab + tab_off_w(c->P1), c->P1, n, rho, part, 1);
-  k_sum_parts3_at<<<1, 32, 0, c->stream>>>(part, nb, base, step, step_stride);
+  k_sum_parts3_at<<<1, 96, 0, c->stream>>>(part, nb, base, step, step_stride);
   c->n_launch += 2;
   TDKS_CU(c, cudaGetLastError());
   return TDKS_OK;

@@ -123,8 +123,6 @@ __global__ void k_kry_start(KryOrb* kry, const double* part, int64_t pstride, in
 struct ChebWork {
   double J[kBessMax + 1];
   double a[TDKS_KMAX], b[TDKS_KMAX];
-  double at[TDKS_KMAX], bt[TDKS_KMAX];   // 2 (a - c)/R and 2 b/R
-  double v0[TDKS_KMAX], v1[TDKS_KMAX], v2[TDKS_KMAX];
   double yr[TDKS_KMAX], yi[TDKS_KMAX];
   double scal[4];
 };
@@ -136,6 +134,66 @@ __device__ __forceinline__ double warp_min(double v) {
 __device__ __forceinline__ double warp_max(double v) {
   for (int off = 16; off > 0; off >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, off));
   return v;
+}
+
+// sum_n (2 - delta_n0) (-i)^n J_n T_n(X) e_1 for X = (T - c) / R by the three-term recurrence,
+// RB consecutive rows per lane (row lane RB + r), everything in registers: a row's
+// neighbours are in the same lane or come by one shuffle each way.  The four phases of
+// (-i)^n are unrolled.  What bounds it is the latency of one term (the shuffles and three
+// dependent FP64 multiply-adds); the shared-memory form with four row blocks whatever m
+// took 0.45 us a term, this one 0.1.
+template <int RB>
+__device__ __forceinline__ void cheb_rows(int m, int N, double c, double invR, ChebWork& W, double cs, double sn) {
+  const int lane = threadIdx.x & 31;
+  double at[RB], bl[RB], br[RB], vp[RB], vc[RB], re[RB], im[RB];
+#pragma unroll
+  for (int r = 0; r < RB; ++r) {
+    const int i = lane * RB + r;
+    const bool in = i < m;
+    at[r] = in ? 2.0 * invR * (W.a[i] - c) : 0.0;              // 2 X, by diagonals
+    bl[r] = in && i > 0 ? 2.0 * invR * W.b[i - 1] : 0.0;
+    br[r] = i < m - 1 ? 2.0 * invR * W.b[i] : 0.0;
+    vp[r] = i == 0 ? 1.0 : 0.0;                                // T_0 e_1
+    vc[r] = i == 0 ? 0.5 * at[r] : (i == 1 ? 0.5 * bl[r] : 0.0);   // T_1 e_1
+    re[r] = W.J[0] * vp[r];
+    im[r] = -W.J[1] * vc[r];
+  }
+  // T_n from vc = T_{n-1}, vp = T_{n-2} into vp
+  auto step = [&](double* p, const double* q) {
+    const double left = __shfl_up_sync(0xffffffffu, q[RB - 1], 1);      // lane 0: its bl is 0
+    const double right = __shfl_down_sync(0xffffffffu, q[0], 1);        // lane 31: its last br is 0
+#pragma unroll
+    for (int r = 0; r < RB; ++r) {
+      double t = fma(at[r], q[r], -p[r]);
+      t = fma(bl[r], r > 0 ? q[r > 0 ? r - 1 : 0] : left, t);
+      p[r] = fma(br[r], r < RB - 1 ? q[r < RB - 1 ? r + 1 : 0] : right, t);
+    }
+  };
+  auto add = [&](double* acc, double cf, const double* v) {
+#pragma unroll
+    for (int r = 0; r < RB; ++r) acc[r] = fma(cf, v[r], acc[r]);
+  };
+  // W.J[n] is 0 for N < n <= N + 3
+  for (int n = 2; n <= N; n += 4) {
+    const double j0 = W.J[n], j1 = W.J[n + 1], j2 = W.J[n + 2], j3 = W.J[n + 3];
+    step(vp, vc);
+    add(re, -j0, vp);      // (-i)^2
+    step(vc, vp);
+    add(im, j1, vc);       // (-i)^3 = i
+    step(vp, vc);
+    add(re, j2, vp);
+    step(vc, vp);
+    add(im, -j3, vc);
+  }
+#pragma unroll
+  for (int r = 0; r < RB; ++r) {
+    const int i = lane * RB + r;
+    if (i < m) {           // times e^{-i tau c} = cs - i sn
+      W.yr[i] = re[r] * cs + im[r] * sn;
+      W.yi[i] = im[r] * cs - re[r] * sn;
+    }
+  }
+  __syncwarp();
 }
 
 // y = exp(-i tau T) e_1 into W.yr/W.yi[0..m-1] (T from W.a, W.b); false if the
@@ -175,132 +233,91 @@ __device__ bool cheb_exp(int m, double tau, ChebWork& W, KryOrb* C = nullptr) {
     hi += wd;
   }
   const double c = 0.5 * (hi + lo);
-  const double R = 0.5 * (hi - lo);
-  double sn, cs;
-  sincos(tau * c, &sn, &cs);
-  const double z = tau * R;
-  if (!(R > 1e-300) || !(z > 1e-280)) {
-    for (int i = lane; i < m; i += 32) {
-      W.yr[i] = (i == 0) ? cs : 0.0;
-      W.yi[i] = (i == 0) ? -sn : 0.0;
-    }
-    __syncwarp();
-    return true;
-  }
-  const int N = reuse ? C->cN : (int)ceil(z + 14.0 * cbrt(z) + 25.0);
-  if (N > kBessMax) return false;
+  double sn, cs, invR;
+  int N;
   if (reuse) {
-    for (int k = lane; k <= N; k += 32) W.J[k] = C->cJ[k];
+    N = C->cN;
+    sn = C->csn;
+    cs = C->ccs;
+    invR = C->cinvR;
+    for (int k = lane; k <= N + 3; k += 32) W.J[k] = k <= N ? C->cJ[k] : 0.0;
     __syncwarp();
   } else {
+    const double R = 0.5 * (hi - lo);
+    sincos(tau * c, &sn, &cs);
+    const double z = tau * R;
+    if (!(R > 1e-300) || !(z > 1e-280)) {
+      for (int i = lane; i < m; i += 32) {
+        W.yr[i] = (i == 0) ? cs : 0.0;
+        W.yi[i] = (i == 0) ? -sn : 0.0;
+      }
+      __syncwarp();
+      return true;
+    }
+    invR = 1.0 / R;
+    // |J_n(z)| < 1e-18 beyond z + 12.5 z^(1/3) for large z (Airy) and well before this for small z
+    const int N0 = (int)ceil(z + 14.0 * cbrt(z) + 10.0);
+    if (N0 + 15 > kBessMax) return false;
     if (lane == 0) {
       // Miller: b_{n-1} = (2n/z) b_n - b_{n+1} from n = M down to 1.  The factor is
       // n (2/z) with n carried as a double (exact), and the overflow test reads the
       // exponent bits, so the FP64 pipe sees two instructions per step.
-      const int M = N + 20;
+      const int M = N0 + 15;
       const double two_inv_z = 2.0 * (1.0 / z);
       double bn1 = 0.0, bn = 1e-280, nd = (double)M, Stail = 0.0;
       for (int n = M; n >= 1; --n, nd -= 1.0) {
         const double bm = (nd * two_inv_z) * bn - bn1;
         const int idx = n - 1;
-        if (idx <= N) W.J[idx] = bm;
-        else if ((idx & 1) == 0) Stail += 2.0 * bm;   // even terms past N enter the sum only
+        if (idx <= N0) W.J[idx] = bm;
+        else if ((idx & 1) == 0) Stail += 2.0 * bm;   // even terms past N0 enter the sum only
         bn1 = bn;
         bn = bm;
         if ((((unsigned long long)__double_as_longlong(bn) >> 52) & 0x7ffull) > 1853ull) {   // |bn| > 2^830
           bn *= 1e-250;
           bn1 *= 1e-250;
           Stail *= 1e-250;
-          for (int k = idx; k <= N && k <= M; ++k) W.J[k] *= 1e-250;
+          for (int k = idx; k <= N0 && k <= M; ++k) W.J[k] *= 1e-250;
         }
       }
       W.scal[0] = Stail;
     }
     __syncwarp();
     // normalization J_0 + 2 sum_{k >= 1} J_2k = 1 (the sum in a fixed order), then J_n
-    // for n >= 1 stored doubled: the expansion uses 2 J_n
-    {
-      double sp = 0.0;
-      for (int k = 2 + 2 * lane; k <= N; k += 64) sp += W.J[k];
-      for (int off = 16; off > 0; off >>= 1) sp += __shfl_down_sync(0xffffffffu, sp, off);
-      const double S = W.J[0] + 2.0 * __shfl_sync(0xffffffffu, sp, 0) + W.scal[0];
-      const double inv = 1.0 / S;
-      __syncwarp();
-      for (int k = lane; k <= N; k += 32) W.J[k] *= (k == 0 ? inv : 2.0 * inv);
+    // for n >= 1 stored doubled: the expansion uses 2 J_n.  Terms past the last one above
+    // 1e-18 are dropped (they decay faster than geometrically).
+    double sp = 0.0;
+    for (int k = 2 + 2 * lane; k <= N0; k += 64) sp += W.J[k];
+    for (int off = 16; off > 0; off >>= 1) sp += __shfl_down_sync(0xffffffffu, sp, off);
+    const double S = W.J[0] + 2.0 * __shfl_sync(0xffffffffu, sp, 0) + W.scal[0];
+    const double inv = 1.0 / S;
+    __syncwarp();
+    int last = 1;
+    for (int k = lane; k <= N0; k += 32) {
+      const double jk = W.J[k] * (k == 0 ? inv : 2.0 * inv);
+      W.J[k] = jk;
+      if (fabs(jk) > 1e-18) last = max(last, k);
     }
+    N = __reduce_max_sync(0xffffffffu, last);
+    __syncwarp();
+    for (int k = N + 1 + lane; k <= N + 3; k += 32) W.J[k] = 0.0;
+    __syncwarp();
     if (C && N <= kChebCache) {
-      __syncwarp();
       for (int k = lane; k <= N; k += 32) C->cJ[k] = W.J[k];
       if (lane == 0) {
         C->clo = lo;
         C->chi = hi;
         C->ctau = tau;
+        C->csn = sn;
+        C->ccs = cs;
+        C->cinvR = invR;
         C->cN = N;
         C->cv = 1;
       }
     }
   }
-  const double invR = 1.0 / R;
-  const double two_invR = 2.0 * invR;
-  // scaled tridiagonal of X = (T - c)/R, doubled: the recurrence v_n = 2 X v_{n-1} - v_{n-2}
-  for (int i = lane; i < m; i += 32) {
-    W.at[i] = two_invR * (W.a[i] - c);
-    W.bt[i] = (i < m - 1) ? two_invR * W.b[i] : 0.0;
-  }
-  // v0 = e_1, v1 = X e_1
-  for (int i = lane; i < m; i += 32) {
-    W.v0[i] = (i == 0) ? 1.0 : 0.0;
-    double t = (i == 0) ? (W.a[0] - c) : 0.0;
-    if (i == 1) t = W.b[0];
-    W.v1[i] = t * invR;
-  }
-  __syncwarp();
-  double accr[TDKS_KMAX / 32], acci[TDKS_KMAX / 32];
-  for (int r = 0; r < TDKS_KMAX / 32; ++r) {
-    const int i = lane + 32 * r;
-    accr[r] = (i < m) ? W.J[0] * W.v0[i] : 0.0;
-    acci[r] = (i < m) ? -W.J[1] * W.v1[i] : 0.0;
-  }
-  double* vp = W.v0;
-  double* vc = W.v1;
-  double* vn = W.v2;
-  for (int n = 2; n <= N; ++n) {
-    for (int r = 0; r < TDKS_KMAX / 32; ++r) {
-      const int i = lane + 32 * r;
-      if (i < m) {
-        double t = fma(W.at[i], vc[i], -vp[i]);
-        if (i > 0) t = fma(W.bt[i - 1], vc[i - 1], t);
-        if (i < m - 1) t = fma(W.bt[i], vc[i + 1], t);
-        vn[i] = t;
-      }
-    }
-    __syncwarp();
-    // (-i)^n 2 J_n T_n: real part for even n, imaginary for odd, signs by n mod 4
-    const double cf = W.J[n];
-    const int ph = n & 3;
-    const double sg = (ph == 0 || ph == 3) ? cf : -cf;
-    for (int r = 0; r < TDKS_KMAX / 32; ++r) {
-      const int i = lane + 32 * r;
-      if (i < m) {
-        if (ph & 1) acci[r] = fma(sg, vn[i], acci[r]);
-        else accr[r] = fma(sg, vn[i], accr[r]);
-      }
-    }
-    double* t = vp;
-    vp = vc;
-    vc = vn;
-    vn = t;
-    __syncwarp();
-  }
-  for (int r = 0; r < TDKS_KMAX / 32; ++r) {
-    const int i = lane + 32 * r;
-    if (i < m) {
-      // multiply by e^{-i tau c} = cs - i sn
-      W.yr[i] = accr[r] * cs + acci[r] * sn;
-      W.yi[i] = acci[r] * cs - accr[r] * sn;
-    }
-  }
-  __syncwarp();
+  if (m <= 32) cheb_rows<1>(m, N, c, invR, W, cs, sn);
+  else if (m <= 64) cheb_rows<2>(m, N, c, invR, W, cs, sn);
+  else cheb_rows<4>(m, N, c, invR, W, cs, sn);
   return true;
 }
 
@@ -353,10 +370,11 @@ __device__ void kry_decide(KryOrb& K, int j, int kmax, double tol, double beta, 
       }
     }
   }
-  for (int i = lane; i < m; i += 32) {
-    K.yre[i] = W.yr[i];
-    K.yim[i] = W.yi[i];
-  }
+  if (decision != 0)   // the coefficients are read by the recombination only
+    for (int i = lane; i < m; i += 32) {
+      K.yre[i] = W.yr[i];
+      K.yim[i] = W.yi[i];
+    }
   if (lane == 0) {
     K.applies += 1;
     K.beta[j] = beta;
@@ -377,18 +395,27 @@ __device__ void kry_decide(KryOrb& K, int j, int kmax, double tol, double beta, 
   }
 }
 
-__global__ void k_kry_exp(int j, int kmax, double tol, KryOrb* kry, const double* npart,
-                          int64_t npstride, int nb, const double* xpart, int nx) {
+// kExpThreads threads sum the partials, the first warp goes on alone
+constexpr int kExpThreads = 128;
+__device__ __forceinline__ double exp_sum(double v, double* red) {
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  return (red[0] + red[1]) + (red[2] + red[3]);
+}
+
+__global__ void __launch_bounds__(kExpThreads) k_kry_exp(int j, int kmax, double tol, KryOrb* kry, const double* npart,
+                                                         int64_t npstride, int nb, const double* xpart, int nx) {
   __shared__ ChebWork W;
+  __shared__ double red[kExpThreads / 32];
   const int o = blockIdx.x;
-  const int lane = threadIdx.x;
   KryOrb& K = kry[o];
   if (K.status != KRY_ACTIVE) return;
   double v = 0.0;
-  for (int k = lane; k < nb; k += 32) v += npart[(long long)o * npstride + k];
-  for (int k = lane; k < nx; k += 32) v += xpart[(long long)o * nx + k];   // nonlocal correction
-  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-  kry_decide(K, j, kmax, tol, sqrt(v), W);
+  for (int k = threadIdx.x; k < nb; k += kExpThreads) v += npart[(long long)o * npstride + k];
+  for (int k = threadIdx.x; k < nx; k += kExpThreads) v += xpart[(long long)o * nx + k];   // nonlocal correction
+  v = exp_sum(v, red);
+  if (threadIdx.x < 32) kry_decide(K, j, kmax, tol, sqrt(v), W);
 }
 
 // out = ||psi|| sum_j y_j s_j V_j
@@ -650,21 +677,21 @@ __global__ void k_bkry_start(const BSys* __restrict__ sys, const BOrb* __restric
 }
 
 // beta_j, small exponential and decision: one warp per orbital, j = K.k
-__global__ void k_bkry_exp(const BSys* __restrict__ sys, const BOrb* __restrict__ orbs, double tol,
-                           double theta) {
+__global__ void __launch_bounds__(kExpThreads) k_bkry_exp(const BSys* __restrict__ sys,
+                                                          const BOrb* __restrict__ orbs, double tol, double theta) {
   __shared__ ChebWork W;
+  __shared__ double red[kExpThreads / 32];
   const BOrb b = orbs[blockIdx.x];
   const BSys& S = sys[b.sys];
   KryOrb& K = S.kry[b.o];
   if (K.status != KRY_ACTIVE) return;
-  const int lane = threadIdx.x;
   const double* np = S.npart + (long long)b.o * S.n_rblk;
   double v = 0.0;
-  for (int k = lane; k < S.n_rblk; k += 32) v += np[k];
-  for (int k = lane; k < S.kb_nblk; k += 32) v += S.kb_part[(long long)b.o * S.kb_nblk + k];   // nonlocal
-  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  for (int k = threadIdx.x; k < S.n_rblk; k += kExpThreads) v += np[k];
+  for (int k = threadIdx.x; k < S.kb_nblk; k += kExpThreads) v += S.kb_part[(long long)b.o * S.kb_nblk + k];   // nonlocal
+  v = exp_sum(v, red);
   const int j = K.k;
-  kry_decide(K, j, S.kmax, tol, sqrt(v), W, theta);
+  if (threadIdx.x < 32) kry_decide(K, j, S.kmax, tol, sqrt(v), W, theta);
 }
 
 // out = ||psi|| sum_j y_j s_j V_j of converged / sub-stepped orbitals, one block per chunk
@@ -935,9 +962,9 @@ static tdks_status iteration_kernels(tdks_ctx* c, KryOrb* kry, const double2* cu
     }
     // ||w||^2 after the passes (the assembly's and the nonlocal partials are stale)
     k_norm_part<<<dim3(nb, n_orb), kThreads, 0, c->stream>>>(VW + (int64_t)j * n, wsorb, n, kry, npart, ps);
-    k_kry_exp<<<n_orb, 32, 0, c->stream>>>(j, kmax, tol, kry, npart, ps, nb, nullptr, 0);
+    k_kry_exp<<<n_orb, kExpThreads, 0, c->stream>>>(j, kmax, tol, kry, npart, ps, nb, nullptr, 0);
   } else {
-    k_kry_exp<<<n_orb, 32, 0, c->stream>>>(j, kmax, tol, kry, npart, ps, nasm, kb_norm_parts(c),
+    k_kry_exp<<<n_orb, kExpThreads, 0, c->stream>>>(j, kmax, tol, kry, npart, ps, nasm, kb_norm_parts(c),
                                            kb_norm_blocks(c));
   }
   TDKS_CU(c, cudaGetLastError());
@@ -1312,7 +1339,7 @@ cudaError_t launch_bkry_prepare(const BSys* sys, const BOrb* orbs, int n, const 
 
 cudaError_t launch_bkry_exp(const BSys* sys, const BOrb* orbs, int n, double tol, double theta,
                             cudaStream_t st) {
-  k_bkry_exp<<<n, 32, 0, st>>>(sys, orbs, tol, theta);
+  k_bkry_exp<<<n, kExpThreads, 0, st>>>(sys, orbs, tol, theta);
   return cudaGetLastError();
 }
 

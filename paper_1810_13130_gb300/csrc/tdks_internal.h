@@ -39,6 +39,7 @@ struct KryOrb {
   // coefficients cJ[0..cN]; valid for any later T whose Gershgorin interval lies inside
   // [clo, chi] (cv = 0: empty)
   double clo, chi, ctau;
+  double csn, ccs, cinvR;      // sin and cos of ctau times the middle, 1 / half-width
   int cN, cv;
   double cJ[kChebCache + 1];
 };
