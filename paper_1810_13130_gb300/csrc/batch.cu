@@ -231,11 +231,11 @@ tdks_status build_kb_lists(tdks_batch* b) {
   std::vector<BRow> rows;
   for (int s = 0; s < b->n_sys; ++s) {
     if (!b->h_full[s].kb) continue;
-    int nblk = 0, nproj = 0;
-    kb_view(b->ctx[s], nullptr, &nblk, &nproj);
+    int nblk = 0, nchunk = 0;
+    kb_view(b->ctx[s], nullptr, &nblk, &nchunk);
     for (int o = 0; o < b->n_orb[s]; ++o) {
       orbs.push_back(BOrb{s, o});
-      for (int p = 0; p < nproj; ++p) items.push_back(BKbItem{s, o, p, 0});
+      for (int k = 0; k < nchunk; ++k) items.push_back(BKbItem{s, o, k, 0});
       for (int r = 0; r < nblk; ++r) rows.push_back(BRow{s, o, r, 0});
     }
   }

@@ -13,8 +13,9 @@
 // column's largest (the projectors are Gaussian; the dropped part is far below the
 // Lanczos tolerance), dense inside the box.
 //
-// Apply: C[o][p] = Pbar_p^T psi_o (one block per projector and orbital, fixed-order
-// reduction), then a gather over the nodes covered by any box:
+// Apply: C[o][p] = Pbar_p^T psi_o (one block per chunk of an atom's box and orbital for all
+// of the atom's projectors, partials summed in a fixed order), then a gather over the nodes
+// covered by any box:
 //   y_j = sum over the boxes holding j of sum_p Pbar_p[j] C[o][p] / h_p.
 // In a Lanczos step alpha_j gains sum_p |C[o][p]|^2 / h_p, and the gather adds y to the
 // updated vector w and writes the partials of |w + y|^2 - |w|^2, which the Krylov
@@ -29,13 +30,19 @@
 namespace {
 
 constexpr int kThreads = 256;
+constexpr int kFinThreads = 128;
 constexpr double kDropRel = 1e-16;
 
 struct KbGroup {          // one atom: box of interior nodes and its projector columns
   int I0, J0, K0, nI, nJ, nK;
   int n_pg;               // projectors of the atom
   int p0;                 // first projector index
-  long long val_off;      // values [n_pg][box] start in the value array
+  long long val_off;      // values [box][n_pg] start in the value array
+};
+
+constexpr int kChunk = 2048;   // box nodes per projection block (8 a thread)
+struct KbChunk {          // box nodes [l0, min(l0 + kChunk, box)) of group g
+  int g, l0;
 };
 
 struct KbEntry {          // one (group, local box index) that covers a node
@@ -117,95 +124,164 @@ __device__ __forceinline__ long long box_global(const KbGroup& G, int nix, int n
   return (long long)(G.I0 + i) + (long long)nix * ((G.J0 + j) + (long long)niy * (G.K0 + k));
 }
 
-// sc * sum_box Pbar_p[l] x[j(l)] by one block (fixed-order reduction), written by thread 0
-__device__ __forceinline__ void kb_project_block(const KbGroup* __restrict__ grp, const int* __restrict__ pg,
+// Partial projections of one chunk of a box, all projectors of its atom at once:
+// dst[s] = sum_l Pbar_s[l] x[j(l)], s < NPG (fixed order).  One block per projector over the
+// whole box left most SMs idle and read the vector four times (119 us for 16 projectors and
+// 8 orbitals at p = 6, 8^3 elements); bound by the FP64 pipe now.  The 2 NPG sums are reduced
+// over the warp by exchanging halves: 9 additions instead of 40.
+template <int NPG>
+__device__ __forceinline__ void kb_project_chunk(const KbGroup* __restrict__ grp, const KbChunk c,
                                                  const double* __restrict__ vals, int nix, int niy,
-                                                 const double2* x, double sc, int p, double2* dst) {
-  __shared__ double red[2][kThreads / 32];
-  const KbGroup G = grp[pg[p]];
-  const int slot = p - G.p0;
-  const long long box = (long long)G.nI * G.nJ * G.nK;
-  const double* v = vals + G.val_off + slot * box;
-  double re = 0.0, im = 0.0;
-  for (long long l = threadIdx.x; l < box; l += blockDim.x) {
-    const double2 a = x[box_global(G, nix, niy, l)];
-    re = fma(v[l], a.x, re);
-    im = fma(v[l], a.y, im);
+                                                 const double2* __restrict__ x, double2* dst) {
+  __shared__ double red[kThreads / 32][2 * NPG];
+  const KbGroup G = grp[c.g];
+  const int box = G.nI * G.nJ * G.nK, l1 = min(c.l0 + kChunk, box);
+  double a[2 * NPG];
+#pragma unroll
+  for (int k = 0; k < 2 * NPG; ++k) a[k] = 0.0;
+  for (int l = c.l0 + threadIdx.x; l < l1; l += kThreads) {
+    const double2 v = x[box_global(G, nix, niy, l)];
+    const double* q = vals + G.val_off + (long long)l * NPG;
+    double f[NPG];
+    if constexpr (NPG == 4) {
+      const double2 q0 = reinterpret_cast<const double2*>(q)[0], q1 = reinterpret_cast<const double2*>(q)[1];
+      f[0] = q0.x, f[1] = q0.y, f[2] = q1.x, f[3] = q1.y;
+    } else {
+      f[0] = q[0];
+    }
+#pragma unroll
+    for (int k = 0; k < NPG; ++k) {
+      a[2 * k] = fma(f[k], v.x, a[2 * k]);
+      a[2 * k + 1] = fma(f[k], v.y, a[2 * k + 1]);
+    }
   }
-  for (int off = 16; off > 0; off >>= 1) {
-    re += __shfl_down_sync(0xffffffffu, re, off);
-    im += __shfl_down_sync(0xffffffffu, im, off);
+  // after step b (n values left) a lane holds those whose index bits match its lane bits
+  const int lane = threadIdx.x & 31;
+  int n = 2 * NPG, off = 1, which = 0;
+#pragma unroll
+  for (int b = 0; b < 5; ++b, off <<= 1) {
+    if (n > 1) {
+      n >>= 1;
+      const bool up = lane & off;
+      which |= up ? n : 0;
+#pragma unroll
+      for (int k = 0; k < NPG; ++k)
+        if (k < n) {
+          const double send = up ? a[k] : a[k + n], keep = up ? a[k + n] : a[k];
+          a[k] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+        }
+    } else {
+      a[0] += __shfl_xor_sync(0xffffffffu, a[0], off);
+    }
   }
-  if ((threadIdx.x & 31) == 0) {
-    red[0][threadIdx.x >> 5] = re;
-    red[1][threadIdx.x >> 5] = im;
-  }
+  if (lane < 2 * NPG) red[threadIdx.x >> 5][which] = a[0];
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double sr = 0.0, si = 0.0;
-    for (int k = 0; k < kThreads / 32; ++k) {
-      sr += red[0][k];
-      si += red[1][k];
+  if (threadIdx.x < 2 * NPG) {
+    double t = 0.0;
+    for (int k = 0; k < kThreads / 32; ++k) t += red[k][threadIdx.x];
+    reinterpret_cast<double*>(dst)[threadIdx.x] = t;
+  }
+}
+
+// P[o][chunk][s]: partial projections of the orbitals in the recurrence (of V_j, unscaled)
+template <int NPG>
+__global__ void __launch_bounds__(kThreads) k_kb_project(const KbGroup* __restrict__ grp,
+                                                         const KbChunk* __restrict__ chunks,
+                                                         const double* __restrict__ vals, int nix, int niy,
+                                                         const double2* in, int64_t in_stride, const KryOrb* kry,
+                                                         double2* P) {
+  const int o = blockIdx.y;
+  if (kry && kry[o].status != KRY_ACTIVE) return;
+  kb_project_chunk<NPG>(grp, chunks[blockIdx.x], vals, nix, niy, in + (long long)o * in_stride,
+                        P + ((long long)o * gridDim.x + blockIdx.x) * NPG);
+}
+
+// C_p / h_p of one orbital from its chunk partials (C_p = sc sum), and sum_p |C_p|^2 / h_p
+// (valid in thread 0), by one block
+__device__ __forceinline__ double kb_finish(const int* __restrict__ pg, const int* __restrict__ goff, int npg,
+                                            const double2* P, double sc, const double* __restrict__ invh, int n_proj,
+                                            double2* CD) {
+  __shared__ double red[kFinThreads / 32];
+  double acc = 0.0;
+  const int sub = threadIdx.x & 3;          // four threads sum the chunks of one projector
+  for (int p0 = 0; p0 < n_proj; p0 += kFinThreads / 4) {
+    const int p = p0 + (threadIdx.x >> 2);
+    double re = 0.0, im = 0.0;
+    if (p < n_proj) {
+      const int g = pg[p], c1 = goff[g + 1];
+#pragma unroll 4
+      for (int c = goff[g] + sub; c < c1; c += 4) {
+        const double2 v = P[(long long)c * npg + p % npg];
+        re += v.x;
+        im += v.y;
+      }
     }
-    *dst = make_double2(sc * sr, sc * si);
-  }
-}
-
-// C[o][p] = sc_o sum_box Pbar_p[l] in_o[j(l)]; sc_o = s_kj of the orbital's Lanczos
-// state (0 and no work for orbitals out of the recurrence) or 1
-__global__ void k_kb_project(const KbGroup* __restrict__ grp, const int* __restrict__ pg,
-                             const double* __restrict__ vals, int nix, int niy, const double2* in,
-                             int64_t in_stride, const KryOrb* kry, int kj, double2* C, int n_proj) {
-  const int p = blockIdx.x, o = blockIdx.y;
-  double sc = 1.0;
-  if (kry) {
-    if (kry[o].status != KRY_ACTIVE) {
-      if (threadIdx.x == 0) C[(long long)o * n_proj + p] = make_double2(0.0, 0.0);
-      return;
+    for (int off = 1; off < 4; off <<= 1) {
+      re += __shfl_xor_sync(0xffffffffu, re, off);
+      im += __shfl_xor_sync(0xffffffffu, im, off);
     }
-    sc = kry[o].s[kj];
+    if (p < n_proj && sub == 0) {
+      re *= sc;
+      im *= sc;
+      const double w = invh[p];
+      CD[p] = make_double2(w * re, w * im);
+      acc = fma(w, re * re + im * im, acc);
+    }
   }
-  kb_project_block(grp, pg, vals, nix, niy, in + (long long)o * in_stride, sc, p, &C[(long long)o * n_proj + p]);
+  for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  return (red[0] + red[1]) + (red[2] + red[3]);
 }
 
-// alpha_j += sum_p |C[o][p]|^2 / h_p (after the element partials were summed)
-__global__ void k_kb_alpha(KryOrb* kry, int kj, const double2* C, const double* invh, int n_proj,
-                           int n_orb) {
-  const int o = blockIdx.x * blockDim.x + threadIdx.x;
-  if (o >= n_orb) return;
-  if (kry[o].status != KRY_ACTIVE) return;
-  double s = 0.0;
-  for (int p = 0; p < n_proj; ++p) {
-    const double2 c = C[(long long)o * n_proj + p];
-    s = fma(invh[p], c.x * c.x + c.y * c.y, s);
-  }
-  kry[o].alpha[kj] += s;
+// CD[o][p] = C / h; in a Lanczos step alpha_j += sum_p |C|^2 / h (after the element partials
+// were summed); C = s_j P in the recurrence
+__global__ void __launch_bounds__(kFinThreads) k_kb_finish(const int* __restrict__ pg, const int* __restrict__ goff,
+                                                           int npg, int n_chunks, const double2* P,
+                                                           const double* __restrict__ invh, int n_proj, KryOrb* kry,
+                                                           int kj, int lanczos, double2* CD) {
+  const int o = blockIdx.x;
+  if (kry && kry[o].status != KRY_ACTIVE) return;
+  const double s = kb_finish(pg, goff, npg, P + (long long)o * n_chunks * npg, kry ? kry[o].s[kj] : 1.0, invh, n_proj,
+                             CD + (long long)o * n_proj);
+  if (lanczos && threadIdx.x == 0) kry[o].alpha[kj] += s;
 }
 
-// w_j += y_j = sum_entries sum_slots Pbar C / h over the covered nodes t = t0, t0 + dt, ...;
-// returns the sum of |w + y|^2 - |w|^2 over them
+// w_j += y_j = sum_entries sum_slots Pbar CD over the covered nodes t = t0, t0 + dt, ...;
+// returns the sum of |w + y|^2 - |w|^2 over them.  (Several orbitals per thread, to read a
+// node's values once, is slower: fewer loads in flight; 8 orbitals on 8^3 elements at p = 6:
+// 70 us with one or two, 74 with four; one orbital at p = 4: 7.7, 11, 18 us.)
+template <int NPG>
 __device__ __forceinline__ double kb_add_nodes(const KbGroup* __restrict__ grp, const double* __restrict__ vals,
                                                const long long* __restrict__ tnode, const int* __restrict__ toff,
-                                               const KbEntry* __restrict__ tent, long long n_t, const double2* Co,
-                                               const double* __restrict__ invh, double2* w, long long t0,
+                                               const KbEntry* __restrict__ tent, long long n_t,
+                                               const double2* __restrict__ CD, double2* w, long long t0,
                                                long long dt) {
   double acc = 0.0;
   for (long long t = t0; t < n_t; t += dt) {
     double yr = 0.0, yi = 0.0;
-    for (int e = toff[t]; e < toff[t + 1]; ++e) {
+    const int e1 = toff[t + 1];
+    for (int e = toff[t]; e < e1; ++e) {
       const KbEntry E = tent[e];
-      const KbGroup G = grp[E.g];
-      const long long box = (long long)G.nI * G.nJ * G.nK;
-      for (int s = 0; s < G.n_pg; ++s) {
-        const int p = G.p0 + s;
-        const double f = vals[G.val_off + s * box + E.l] * invh[p];
-        yr = fma(f, Co[p].x, yr);
-        yi = fma(f, Co[p].y, yi);
+      const int p0 = grp[E.g].p0;
+      const double* q = vals + grp[E.g].val_off + (long long)E.l * NPG;
+      double f[NPG];
+      if constexpr (NPG == 4) {
+        const double2 q0 = reinterpret_cast<const double2*>(q)[0], q1 = reinterpret_cast<const double2*>(q)[1];
+        f[0] = q0.x, f[1] = q0.y, f[2] = q1.x, f[3] = q1.y;
+      } else {
+        f[0] = q[0];
+      }
+#pragma unroll
+      for (int s = 0; s < NPG; ++s) {
+        const double2 c = CD[p0 + s];
+        yr = fma(f[s], c.x, yr);
+        yi = fma(f[s], c.y, yi);
       }
     }
     const long long j = tnode[t];
     double2 v = w[j];
-    acc += 2.0 * (v.x * yr + v.y * yi) + yr * yr + yi * yi;
+    acc = fma(yr, fma(2.0, v.x, yr), fma(yi, fma(2.0, v.y, yi), acc));
     v.x += yr;
     v.y += yi;
     w[j] = v;
@@ -228,17 +304,19 @@ __device__ __forceinline__ void kb_block_sum(double acc, double* dst) {
 
 // out_j (+)= y_j over the covered nodes; in a Lanczos step the partials of
 // |w + y|^2 - |w|^2 go to part[o][block]
-__global__ void k_kb_add(const KbGroup* __restrict__ grp, const double* __restrict__ vals,
-                         const long long* __restrict__ tnode, const int* __restrict__ toff,
-                         const KbEntry* __restrict__ tent, long long n_t, const double2* C,
-                         const double* __restrict__ invh, int n_proj, double2* out,
-                         int64_t out_stride, const KryOrb* kry, double* part, int64_t part_stride) {
+template <int NPG>
+__global__ void __launch_bounds__(kThreads) k_kb_add(const KbGroup* __restrict__ grp, const double* __restrict__ vals,
+                                                     const long long* __restrict__ tnode,
+                                                     const int* __restrict__ toff, const KbEntry* __restrict__ tent,
+                                                     long long n_t, const double2* CD, int n_proj, double2* out,
+                                                     int64_t out_stride, const KryOrb* kry, double* part,
+                                                     int64_t part_stride) {
   const int o = blockIdx.y;
   if (kry && kry[o].status != KRY_ACTIVE) return;
-  const double acc = kb_add_nodes(grp, vals, tnode, toff, tent, n_t, C + (long long)o * n_proj, invh,
-                                  out + (long long)o * out_stride,
-                                  blockIdx.x * (long long)blockDim.x + threadIdx.x,
-                                  (long long)gridDim.x * blockDim.x);
+  const double acc = kb_add_nodes<NPG>(grp, vals, tnode, toff, tent, n_t, CD + (long long)o * n_proj,
+                                       out + (long long)o * out_stride,
+                                       blockIdx.x * (long long)blockDim.x + threadIdx.x,
+                                       (long long)gridDim.x * blockDim.x);
   if (part) kb_block_sum(acc, &part[(long long)o * part_stride + blockIdx.x]);
 }
 
@@ -248,14 +326,17 @@ __global__ void k_kb_add(const KbGroup* __restrict__ grp, const double* __restri
 struct KbView {
   const KbGroup* grp;
   const int* pg;
+  const int* goff;         // first chunk of each group (n_grp + 1)
+  const KbChunk* chunks;
   const double* vals;
   const double* invh;
   const long long* tnode;
   const int* toff;
   const KbEntry* tent;
-  double2* C;             // [n_orb][n_proj]
+  double2* P;             // [n_orb][n_chunks][npg] partial projections
+  double2* CD;            // [n_orb][n_proj] C / h
   long long n_t;
-  int n_proj, n_blocks, nix, niy;
+  int n_proj, n_chunks, npg, n_blocks, nix, niy;
 };
 
 namespace {
@@ -268,46 +349,43 @@ __device__ __forceinline__ const double2* kb_bcur(const BSys& S, const KryOrb& K
   return S.Vw + ((long long)o * S.kmax + (K.k - 1)) * S.n_int;
 }
 
-__global__ void k_bkb_project(const BSys* __restrict__ sys, const BKbItem* __restrict__ items) {
+__global__ void __launch_bounds__(kThreads) k_bkb_project(const BSys* __restrict__ sys,
+                                                          const BKbItem* __restrict__ items) {
   const BKbItem it = items[blockIdx.x];
   const BSys& S = sys[it.sys];
   const KbView& V = *S.kb;
   const KryOrb& K = S.kry[it.o];
-  double2* dst = &V.C[(long long)it.o * V.n_proj + it.p];
-  if (K.status != KRY_ACTIVE) {
-    if (threadIdx.x == 0) *dst = make_double2(0.0, 0.0);
-    return;
-  }
-  kb_project_block(V.grp, V.pg, V.vals, V.nix, V.niy, kb_bcur(S, K, it.o), K.s[K.k], it.p, dst);
+  if (K.status != KRY_ACTIVE) return;
+  const double2* x = kb_bcur(S, K, it.o);
+  double2* dst = V.P + ((long long)it.o * V.n_chunks + it.chunk) * V.npg;
+  if (V.npg == 4) kb_project_chunk<4>(V.grp, V.chunks[it.chunk], V.vals, V.nix, V.niy, x, dst);
+  else kb_project_chunk<1>(V.grp, V.chunks[it.chunk], V.vals, V.nix, V.niy, x, dst);
 }
 
-__global__ void k_bkb_alpha(const BSys* __restrict__ sys, const BOrb* __restrict__ orbs, int n) {
-  const int g = blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= n) return;
-  const BOrb b = orbs[g];
+__global__ void __launch_bounds__(kFinThreads) k_bkb_finish(const BSys* __restrict__ sys,
+                                                            const BOrb* __restrict__ orbs) {
+  const BOrb b = orbs[blockIdx.x];
   const BSys& S = sys[b.sys];
   KryOrb& K = S.kry[b.o];
   if (K.status != KRY_ACTIVE) return;
   const KbView& V = *S.kb;
-  double s = 0.0;
-  for (int p = 0; p < V.n_proj; ++p) {
-    const double2 c = V.C[(long long)b.o * V.n_proj + p];
-    s = fma(V.invh[p], c.x * c.x + c.y * c.y, s);
-  }
-  K.alpha[K.k] += s;
+  const double s = kb_finish(V.pg, V.goff, V.npg, V.P + (long long)b.o * V.n_chunks * V.npg, K.s[K.k], V.invh, V.n_proj,
+                             V.CD + (long long)b.o * V.n_proj);
+  if (threadIdx.x == 0) K.alpha[K.k] += s;
 }
 
 // one block per (system, orbital, node block): y into the assembly's output V_{j+1}
-__global__ void k_bkb_add(const BSys* __restrict__ sys, const BRow* __restrict__ rows) {
+__global__ void __launch_bounds__(kThreads) k_bkb_add(const BSys* __restrict__ sys, const BRow* __restrict__ rows) {
   const BRow r = rows[blockIdx.x];
   const BSys& S = sys[r.sys];
   const KryOrb& K = S.kry[r.o];
   if (K.status != KRY_ACTIVE) return;
   const KbView& V = *S.kb;
   double2* w = S.Vw + ((long long)r.o * S.kmax + K.k) * S.n_int;
-  const double acc = kb_add_nodes(V.grp, V.vals, V.tnode, V.toff, V.tent, V.n_t, V.C + (long long)r.o * V.n_proj,
-                                  V.invh, w, r.rblk * (long long)blockDim.x + threadIdx.x,
-                                  (long long)S.kb_nblk * blockDim.x);
+  const double2* CD = V.CD + (long long)r.o * V.n_proj;
+  const long long t0 = r.rblk * (long long)blockDim.x + threadIdx.x, dt = (long long)S.kb_nblk * blockDim.x;
+  const double acc = V.npg == 4 ? kb_add_nodes<4>(V.grp, V.vals, V.tnode, V.toff, V.tent, V.n_t, CD, w, t0, dt)
+                                : kb_add_nodes<1>(V.grp, V.vals, V.tnode, V.toff, V.tent, V.n_t, CD, w, t0, dt);
   kb_block_sum(acc, &S.kb_part[(long long)r.o * S.kb_nblk + r.rblk]);
 }
 
@@ -319,7 +397,8 @@ int grid_for(long long n, int cap) {
 }  // namespace
 
 struct KbState {
-  int n_proj = 0, n_grp = 0, n_blocks = 0;
+  int n_proj = 0, n_grp = 0, n_blocks = 0, n_chunks = 0, npg = 1;
+  int c_orb = 0;                // orbitals the projections are sized for
   long long n_t = 0, n_vals = 0;
   KbGroup* d_grp = nullptr;
   int* d_pg = nullptr;
@@ -328,7 +407,10 @@ struct KbState {
   long long* d_tnode = nullptr;
   int* d_toff = nullptr;
   KbEntry* d_tent = nullptr;
-  double2* d_C = nullptr;
+  int* d_goff = nullptr;
+  KbChunk* d_chunks = nullptr;
+  double2* d_P = nullptr;       // partial projections [c_orb][n_chunks][npg]
+  double2* d_CD = nullptr;      // C / h [c_orb][n_proj]
   double* d_part = nullptr;     // [n_orb][n_blocks] partials of the Lanczos correction
   KbView* d_view = nullptr;     // device view for the batched engine (made on first use)
   std::vector<double> h;
@@ -337,8 +419,8 @@ struct KbState {
 void kb_free(tdks_ctx* c) {
   if (!c || !c->kb) return;
   KbState* k = static_cast<KbState*>(c->kb);
-  void* ptrs[] = {k->d_grp, k->d_pg, k->d_vals, k->d_invh, k->d_tnode, k->d_toff, k->d_tent, k->d_C, k->d_part,
-                  k->d_view};
+  void* ptrs[] = {k->d_grp, k->d_pg, k->d_vals, k->d_invh, k->d_tnode, k->d_toff, k->d_tent, k->d_P, k->d_CD,
+                  k->d_goff, k->d_chunks, k->d_part, k->d_view};
   for (void* p : ptrs) cudaFree(p);
   delete k;
   c->kb = nullptr;
@@ -352,12 +434,13 @@ const double* kb_norm_parts(const tdks_ctx* c) {
   return c->kb ? static_cast<const KbState*>(c->kb)->d_part : nullptr;
 }
 
-const KbView* kb_view(tdks_ctx* c, double** part, int* n_blocks, int* n_proj) {
+const KbView* kb_view(tdks_ctx* c, double** part, int* n_blocks, int* n_chunks) {
   KbState* k = c ? static_cast<KbState*>(c->kb) : nullptr;
   if (!k) return nullptr;
   if (!k->d_view) {
-    const KbView v{k->d_grp, k->d_pg, k->d_vals, k->d_invh, k->d_tnode, k->d_toff, k->d_tent, k->d_C,
-                   k->n_t, k->n_proj, k->n_blocks, c->Ni[0], c->Ni[1]};
+    const KbView v{k->d_grp,  k->d_pg,   k->d_goff,   k->d_chunks, k->d_vals,   k->d_invh,   k->d_tnode,
+                   k->d_toff, k->d_tent, k->d_P,      k->d_CD,     k->n_t,      k->n_proj,   k->n_chunks,
+                   k->npg,    k->n_blocks, c->Ni[0],  c->Ni[1]};
     if (cudaMalloc((void**)&k->d_view, sizeof(KbView)) != cudaSuccess ||
         cudaMemcpy(k->d_view, &v, sizeof(v), cudaMemcpyHostToDevice) != cudaSuccess) {
       cudaGetLastError();
@@ -368,7 +451,7 @@ const KbView* kb_view(tdks_ctx* c, double** part, int* n_blocks, int* n_proj) {
   }
   if (part) *part = k->d_part;
   if (n_blocks) *n_blocks = k->n_t > 0 ? k->n_blocks : 0;
-  if (n_proj) *n_proj = k->n_proj;
+  if (n_chunks) *n_chunks = k->n_chunks;
   return k->d_view;
 }
 
@@ -380,7 +463,7 @@ cudaError_t launch_bkb_project(const BSys* sys, const BKbItem* items, int n_item
 
 cudaError_t launch_bkb_alpha(const BSys* sys, const BOrb* orbs, int n_orbs, cudaStream_t st) {
   if (n_orbs < 1) return cudaSuccess;
-  k_bkb_alpha<<<(n_orbs + 63) / 64, 64, 0, st>>>(sys, orbs, n_orbs);
+  k_bkb_finish<<<n_orbs, kFinThreads, 0, st>>>(sys, orbs);
   return cudaGetLastError();
 }
 
@@ -393,18 +476,41 @@ cudaError_t launch_bkb_add(const BSys* sys, const BRow* rows, int n_rows, cudaSt
 tdks_status kb_project(tdks_ctx* c, const ApplyArgs& a) {
   KbState* k = static_cast<KbState*>(c->kb);
   if (!k) return TDKS_OK;
-  k_kb_project<<<dim3(k->n_proj, a.n_orb), kThreads, 0, c->stream>>>(
-      k->d_grp, k->d_pg, k->d_vals, c->Ni[0], c->Ni[1], a.in_base, a.in_stride, a.kry, a.kj, k->d_C,
-      k->n_proj);
+  if (a.n_orb > k->c_orb) {   // a plain application of more vectors than the system's orbitals
+    cudaFree(k->d_P);
+    cudaFree(k->d_CD);
+    k->d_P = k->d_CD = nullptr;
+    k->c_orb = 0;
+    if (cudaMalloc(&k->d_P, ((size_t)a.n_orb * k->n_chunks * k->npg + 1) * sizeof(double2)) != cudaSuccess ||
+        cudaMalloc(&k->d_CD, (size_t)a.n_orb * k->n_proj * sizeof(double2)) != cudaSuccess) {
+      cudaGetLastError();
+      return tdks_fail(c, TDKS_ERR_NOMEM, "projections");
+    }
+    k->c_orb = a.n_orb;
+    kgraph_free(c);           // captured Lanczos loops hold the old buffers
+    cudaFree(k->d_view);      // as does the batched view
+    k->d_view = nullptr;
+  }
+  if (k->n_chunks > 0) {
+    const dim3 grid(k->n_chunks, a.n_orb);
+    if (k->npg == 4)
+      k_kb_project<4><<<grid, kThreads, 0, c->stream>>>(k->d_grp, k->d_chunks, k->d_vals, c->Ni[0], c->Ni[1], a.in_base,
+                                                        a.in_stride, a.kry, k->d_P);
+    else
+      k_kb_project<1><<<grid, kThreads, 0, c->stream>>>(k->d_grp, k->d_chunks, k->d_vals, c->Ni[0], c->Ni[1], a.in_base,
+                                                        a.in_stride, a.kry, k->d_P);
+  }
   c->n_launch += 1;
   TDKS_CU(c, cudaGetLastError());
-  return TDKS_OK;
+  // (with a Lanczos step kb_alpha does this once alpha has been summed)
+  return a.lanczos && a.kry && a.part ? TDKS_OK : kb_alpha(c, a);
 }
 
 tdks_status kb_alpha(tdks_ctx* c, const ApplyArgs& a) {
   KbState* k = static_cast<KbState*>(c->kb);
-  if (!k || !a.kry) return TDKS_OK;
-  k_kb_alpha<<<(a.n_orb + 63) / 64, 64, 0, c->stream>>>(a.kry, a.kj, k->d_C, k->d_invh, k->n_proj, a.n_orb);
+  if (!k) return TDKS_OK;
+  k_kb_finish<<<a.n_orb, kFinThreads, 0, c->stream>>>(k->d_pg, k->d_goff, k->npg, k->n_chunks, k->d_P, k->d_invh,
+                                                      k->n_proj, a.kry, a.kj, a.lanczos && a.kry && a.part, k->d_CD);
   c->n_launch += 1;
   TDKS_CU(c, cudaGetLastError());
   return TDKS_OK;
@@ -414,9 +520,15 @@ tdks_status kb_add(tdks_ctx* c, const ApplyArgs& a) {
   KbState* k = static_cast<KbState*>(c->kb);
   if (!k || k->n_t == 0) return TDKS_OK;
   const bool lz = a.lanczos && a.kry;
-  k_kb_add<<<dim3(k->n_blocks, a.n_orb), kThreads, 0, c->stream>>>(
-      k->d_grp, k->d_vals, k->d_tnode, k->d_toff, k->d_tent, k->n_t, k->d_C, k->d_invh, k->n_proj,
-      a.out_base, a.out_stride, a.kry, lz ? k->d_part : nullptr, k->n_blocks);
+  const dim3 grid(k->n_blocks, a.n_orb);
+  if (k->npg == 4)
+    k_kb_add<4><<<grid, kThreads, 0, c->stream>>>(k->d_grp, k->d_vals, k->d_tnode, k->d_toff, k->d_tent, k->n_t,
+                                                  k->d_CD, k->n_proj, a.out_base, a.out_stride, a.kry,
+                                                  lz ? k->d_part : nullptr, k->n_blocks);
+  else
+    k_kb_add<1><<<grid, kThreads, 0, c->stream>>>(k->d_grp, k->d_vals, k->d_tnode, k->d_toff, k->d_tent, k->n_t,
+                                                  k->d_CD, k->n_proj, a.out_base, a.out_stride, a.kry,
+                                                  lz ? k->d_part : nullptr, k->n_blocks);
   c->n_launch += 1;
   TDKS_CU(c, cudaGetLastError());
   return TDKS_OK;
@@ -486,7 +598,8 @@ extern "C" tdks_status tdks_set_kb(tdks_ctx* c, int n_atoms, const double* R, do
   // boxes: per atom, the interior-index box outside which every entry of its columns
   // is below kDropRel of that column's largest magnitude
   std::vector<KbGroup> grp(n_atoms);
-  std::vector<int> pg(n_proj);
+  std::vector<int> pg(n_proj), goff(n_atoms + 1, 0);
+  std::vector<KbChunk> chunks;
   std::vector<double> vals;
   for (int I = 0; I < n_atoms; ++I) {
     int lo[3] = {nix, niy, niz}, hi[3] = {-1, -1, -1};
@@ -521,14 +634,15 @@ extern "C" tdks_status tdks_set_kb(tdks_ctx* c, int n_atoms, const double* R, do
     G.p0 = I * npa;
     G.val_off = (long long)vals.size();
     const long long box = (long long)G.nI * G.nJ * G.nK;
-    for (int m = 0; m < npa; ++m) {
-      pg[I * npa + m] = I;
-      const std::vector<double>& v = cols[I * npa + m];
-      for (long long l = 0; l < box; ++l) {
-        const int i = (int)(l % G.nI), jj = (int)((l / G.nI) % G.nJ), kk = (int)(l / ((long long)G.nI * G.nJ));
-        vals.push_back(v[(G.I0 + i) + (long long)nix * ((G.J0 + jj) + (long long)niy * (G.K0 + kk))]);
-      }
+    for (int m = 0; m < npa; ++m) pg[I * npa + m] = I;
+    for (long long l = 0; l < box; ++l) {
+      const int i = (int)(l % G.nI), jj = (int)((l / G.nI) % G.nJ), kk = (int)(l / ((long long)G.nI * G.nJ));
+      const long long node = (G.I0 + i) + (long long)nix * ((G.J0 + jj) + (long long)niy * (G.K0 + kk));
+      for (int m = 0; m < npa; ++m) vals.push_back(cols[I * npa + m][node]);
     }
+    goff[I] = (int)chunks.size();
+    for (long long l0 = 0; l0 < box; l0 += kChunk) chunks.push_back(KbChunk{I, (int)l0});
+    goff[I + 1] = (int)chunks.size();
     grp[I] = G;
   }
   // covered nodes (ascending) and the (atom, local index) entries of each
@@ -562,6 +676,9 @@ extern "C" tdks_status tdks_set_kb(tdks_ctx* c, int n_atoms, const double* R, do
   KbState* k = new KbState();
   k->n_proj = n_proj;
   k->n_grp = n_atoms;
+  k->npg = npa;
+  k->n_chunks = (int)chunks.size();
+  k->c_orb = c->n_orb;
   k->n_t = (long long)tnode.size();
   k->n_vals = (long long)vals.size();
   k->n_blocks = grid_for(std::max<long long>(k->n_t, 1), 512);
@@ -576,7 +693,9 @@ extern "C" tdks_status tdks_set_kb(tdks_ctx* c, int n_atoms, const double* R, do
   };
   if (!up(&k->d_grp, grp) || !up(&k->d_pg, pg) || !up(&k->d_vals, vals) || !up(&k->d_invh, invh) ||
       !up(&k->d_tnode, tnode) || !up(&k->d_toff, toff) || !up(&k->d_tent, tent) ||
-      cudaMalloc(&k->d_C, (size_t)c->n_orb * n_proj * sizeof(double2)) != cudaSuccess ||
+      !up(&k->d_goff, goff) || !up(&k->d_chunks, chunks) ||
+      cudaMalloc(&k->d_P, ((size_t)c->n_orb * k->n_chunks * npa + 1) * sizeof(double2)) != cudaSuccess ||
+      cudaMalloc(&k->d_CD, (size_t)c->n_orb * n_proj * sizeof(double2)) != cudaSuccess ||
       cudaMalloc(&k->d_part, (size_t)c->n_orb * k->n_blocks * sizeof(double)) != cudaSuccess) {
     cudaGetLastError();
     kb_free(c);

@@ -356,7 +356,7 @@ static_assert(sizeof(BSys) % 8 == 0, "BSys is copied as 64-bit words");
 struct BItem { int sys, eblk, o0, o1; };   // apply: E elements of block eblk, orbitals [o0, o1)
 struct BRow { int sys, o, rblk, pad; };    // one row block of one orbital
 struct BOrb { int sys, o; };               // one orbital of one system
-struct BKbItem { int sys, o, p, pad; };    // nonlocal projection: projector p of orbital o
+struct BKbItem { int sys, o, chunk, pad; };   // nonlocal projection: one box chunk of orbital o
 
 // elements.cu
 cudaError_t hbar_batch_occupancy(int P1, int prec, int E, int* blocks_per_sm);
@@ -386,11 +386,11 @@ cudaError_t launch_bloop_control(cudaGraphConditionalHandle h, const BSys* sys, 
                                  int n_orbs, int* iter, int cap, int* err, int* qctr, int n_q,
                                  cudaStream_t st);
 // kb.cu, batched nonlocal term: the device view of c's projectors (nullptr without
-// them; owned by the context), its partial buffer [n_orb][*n_blocks] and projector count
-const KbView* kb_view(tdks_ctx* c, double** part, int* n_blocks, int* n_proj);
-// C of every item's (orbital, projector) from the orbital's current Krylov vector
+// them; owned by the context), its partial buffer [n_orb][*n_blocks] and chunk count
+const KbView* kb_view(tdks_ctx* c, double** part, int* n_blocks, int* n_chunks);
+// partial projections of every item's (orbital, chunk) from the orbital's current Krylov vector
 cudaError_t launch_bkb_project(const BSys* sys, const BKbItem* items, int n_items, cudaStream_t st);
-// alpha_j += sum_p |C_p|^2 / h_p of every listed orbital (after launch_balpha)
+// C from the partials; alpha_j += sum_p |C_p|^2 / h_p of every listed orbital (after launch_balpha)
 cudaError_t launch_bkb_alpha(const BSys* sys, const BOrb* orbs, int n_orbs, cudaStream_t st);
 // w += y over the covered nodes of block rows[i].rblk, partials to kb_part (after the assembly)
 cudaError_t launch_bkb_add(const BSys* sys, const BRow* rows, int n_rows, cudaStream_t st);
@@ -415,8 +415,8 @@ cudaError_t launch_counter_add(int* counter, int inc, cudaStream_t st);
 
 // kb.cu: nonlocal Kleinman-Bylander term, hooked into the Hbar application
 void kb_free(tdks_ctx* c);
-tdks_status kb_project(tdks_ctx* c, const ApplyArgs& a);   // C = Pbar^T (s_j) in
-tdks_status kb_alpha(tdks_ctx* c, const ApplyArgs& a);     // alpha_j += sum |C|^2 / h
+tdks_status kb_project(tdks_ctx* c, const ApplyArgs& a);   // Pbar^T in (and kb_alpha without a Lanczos step)
+tdks_status kb_alpha(tdks_ctx* c, const ApplyArgs& a);     // C = s_j Pbar^T in; alpha_j += sum |C|^2 / h
 tdks_status kb_add(tdks_ctx* c, const ApplyArgs& a);       // out += Pbar D C (+ norm partials)
 int kb_norm_blocks(const tdks_ctx* c);                      // partials of the Lanczos correction
 const double* kb_norm_parts(const tdks_ctx* c);             // [n_orb][kb_norm_blocks]
