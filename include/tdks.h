@@ -420,8 +420,8 @@ tdks_status tdks_set_lanczos(tdks_ctx* ctx, int reorth);
  * iteration after the first a conditional node whose condition a one-block kernel sets
  * from the Lanczos state of the previous iteration (some orbital still active; under
  * TDKS_MIXED also the contraction arithmetic), so the host reads that state once per
- * sub-step.  The graph is captured on first use for a given starting vector and
- * settings and kept with the context.  on = 0: the host launches every iteration and
+ * sub-step.  The graph is captured on first use for given settings (it starts from a copy
+ * of the vector in the basis) and kept with the context.  on = 0: the host launches every iteration and
  * reads the state after each.  Both run the same kernels in the same order, so the
  * results are identical. */
 tdks_status tdks_set_device_loop(tdks_ctx* ctx, int on);

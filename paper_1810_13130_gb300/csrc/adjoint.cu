@@ -34,12 +34,11 @@ int grid_for(long long n) {
 }
 
 // out[o] = sum_j coef[o][j] V_j[o], V_0 = base vector, V_j (j >= 1) in the workspace
-__global__ void k_combine_basis(long long n, double2* out, const double2* V0, const double2* Vw,
-                                int64_t wsorb, const double2* coef, int kcap, const int* kk) {
+__global__ void k_combine_basis(long long n, double2* out, const double2* Vw, int64_t wsorb, const double2* coef,
+                                int kcap, const int* kk) {
   const int o = blockIdx.y;
   const int m = kk[o];
   const double2* c = coef + (long long)o * kcap;
-  const double2* v0 = V0 + (long long)o * n;
   const double2* vw = Vw + (long long)o * wsorb;
   double2* dst = out + (long long)o * n;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
@@ -47,7 +46,7 @@ __global__ void k_combine_basis(long long n, double2* out, const double2* V0, co
     double re = 0.0, im = 0.0;
 #pragma unroll 4
     for (int j = 0; j < m; ++j) {
-      const double2 v = (j == 0) ? v0[i] : vw[(long long)(j - 1) * n + i];
+      const double2 v = vw[(long long)j * n + i];
       const double2 cj = c[j];
       re = fma(cj.x, v.x, fma(-cj.y, v.y, re));
       im = fma(cj.x, v.y, fma(cj.y, v.x, im));
@@ -231,11 +230,11 @@ tdks_status frechet(tdks_ctx* c, AdjState* A, const double2* psi, const double2*
     TDKS_CU(c, cudaMemcpyAsync(A->d_coef, cp.data(), cp.size() * sizeof(double2), cudaMemcpyHostToDevice,
                                c->stream));
     k_combine_basis<<<dim3(nb, n_orb), kThreads, 0, c->stream>>>(
-        n, A->phis, psi, c->d_Vw[0], (int64_t)c->Vw_kmax[0] * n, A->d_coef, kcap, A->d_k);
+        n, A->phis, c->d_Vw[0], (int64_t)(c->Vw_kmax[0] + 1) * n, A->d_coef, kcap, A->d_k);
     TDKS_CU(c, cudaMemcpyAsync(A->d_coef + (size_t)n_orb * kcap, cl.data(), cl.size() * sizeof(double2),
                                cudaMemcpyHostToDevice, c->stream));
     k_combine_basis<<<dim3(nb, n_orb), kThreads, 0, c->stream>>>(
-        n, A->mus, lam, c->d_Vw[1], (int64_t)c->Vw_kmax[1] * n, A->d_coef + (size_t)n_orb * kcap, kcap,
+        n, A->mus, c->d_Vw[1], (int64_t)(c->Vw_kmax[1] + 1) * n, A->d_coef + (size_t)n_orb * kcap, kcap,
         A->d_k + n_orb);
     c->n_launch += 2;
     TDKS_TRY(launch_cross(c, A->mus, A->phis, n_orb, sw[i] * tau, g_out));

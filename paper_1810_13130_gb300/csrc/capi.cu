@@ -489,12 +489,7 @@ tdks_status tdks_expm(tdks_ctx* c, const double* in, double* out, int n_orb, dou
   TDKS_TRY(check_orb(c, n_orb));
   if (!(tol > 0) || !std::isfinite(tau)) return tdks_fail(c, TDKS_ERR_ARG, "tol > 0, finite tau");
   if (!valid_prec(prec)) return tdks_fail(c, TDKS_ERR_ARG, "precision");
-  if (in != out)
-    TDKS_CU(c, cudaMemcpyAsync(out, in, (size_t)n_orb * c->n_int * sizeof(double2),
-                               cudaMemcpyDeviceToDevice, c->stream));
-  // the recurrence starts from `out` so that `in` is never written
-  return run_expm(c, (const double2*)out, (double2*)out, n_orb, tau, tol, k_max, prec, k_used,
-                  nullptr, nullptr, nullptr);
+  return run_expm(c, (const double2*)in, (double2*)out, n_orb, tau, tol, k_max, prec, k_used, nullptr, nullptr, nullptr);
 }
 
 tdks_status tdks_kick(tdks_ctx* c, double* psi, int n_orb, double kappa, const double dir[3]) {
@@ -621,8 +616,7 @@ tdks_status magnus_step_impl(tdks_ctx* c, double2* psi, int n_orb, double dt, co
   // predictor: V(t + dt/4) = V_N + 1.25 V_HXC^{n-1} - 0.25 V_HXC^{n-2} - E(t + dt/4).r
   TDKS_TRY(launch_combine(c, c->d_vks, c->d_vnuc, 1.25, c->d_vhxc1, -0.25, c->d_vhxc2, nullptr, Eq));
   if (keep_vpred) TDKS_CU(c, cudaMemcpyAsync(keep_vpred, c->d_vks, fb, cudaMemcpyDeviceToDevice, c->stream));
-  TDKS_CU(c, cudaMemcpyAsync(c->d_psi_half, psi, vb, cudaMemcpyDeviceToDevice, c->stream));
-  TDKS_TRY(run_expm(c, c->d_psi_half, c->d_psi_half, n_orb, 0.5 * dt, tol, k_max, prec, nullptr,
+  TDKS_TRY(run_expm(c, psi, c->d_psi_half, n_orb, 0.5 * dt, tol, k_max, prec, nullptr,
                     &kseen, &app, &nsub));
   if (keep_half) TDKS_CU(c, cudaMemcpyAsync(keep_half, c->d_psi_half, vb, cudaMemcpyDeviceToDevice, c->stream));
   st.k_half_max = kseen;

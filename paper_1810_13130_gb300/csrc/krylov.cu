@@ -97,6 +97,27 @@ __global__ void k_norm_part(const double2* v, int64_t stride, long long n, const
   if (threadIdx.x == 0) part[(long long)o * pstride + blockIdx.x] = s;
 }
 
+// the start of a sub-step: V_0 of every active orbital copied into the basis, with the
+// partials of its norm
+__global__ void k_copy_norm(const double2* v, double2* V0, int64_t wsorb, long long n, const KryOrb* kry,
+                            double* part, int64_t pstride) {
+  __shared__ double red[kThreads / 32];
+  const int o = blockIdx.y;
+  double acc = 0.0;
+  if (kry[o].status == KRY_ACTIVE) {
+    const double2* p = v + (long long)o * n;
+    double2* q = V0 + (long long)o * wsorb;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
+         i += (long long)gridDim.x * blockDim.x) {
+      const double2 a = p[i];
+      q[i] = a;
+      acc = fma(a.x, a.x, fma(a.y, a.y, acc));
+    }
+  }
+  const double s = block_reduce_sum(acc, red);
+  if (threadIdx.x == 0) part[(long long)o * pstride + blockIdx.x] = s;
+}
+
 __global__ void k_kry_start(KryOrb* kry, const double* part, int64_t pstride, int nb) {
   __shared__ double red[kThreads / 32];
   const int o = blockIdx.x;
@@ -419,8 +440,8 @@ __global__ void __launch_bounds__(kExpThreads) k_kry_exp(int j, int kmax, double
 }
 
 // out = ||psi|| sum_j y_j s_j V_j
-__global__ void k_kry_recomb(long long n, double2* out, int64_t so, const double2* V0, int64_t s0,
-                             const double2* Vw, int64_t sw, int kmax, const KryOrb* kry) {
+__global__ void k_kry_recomb(long long n, double2* out, int64_t so, const double2* Vw, int64_t sw,
+                             const KryOrb* kry) {
   __shared__ double cr[TDKS_KMAX], ci[TDKS_KMAX];
   const int o = blockIdx.y;
   const KryOrb& K = kry[o];
@@ -433,7 +454,6 @@ __global__ void k_kry_recomb(long long n, double2* out, int64_t so, const double
     ci[j] = f * K.yim[j];
   }
   __syncthreads();
-  const double2* v0 = V0 + (long long)o * s0;
   const double2* vw = Vw + (long long)o * sw;
   double2* dst = out + (long long)o * so;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
@@ -441,7 +461,7 @@ __global__ void k_kry_recomb(long long n, double2* out, int64_t so, const double
     double re = 0.0, im = 0.0;
 #pragma unroll 4
     for (int j = 0; j < m; ++j) {
-      const double2 v = (j == 0) ? v0[i] : vw[(long long)(j - 1) * n + i];
+      const double2 v = vw[(long long)j * n + i];
       re = fma(cr[j], v.x, fma(-ci[j], v.y, re));
       im = fma(cr[j], v.y, fma(ci[j], v.x, im));
     }
@@ -484,8 +504,8 @@ __device__ __forceinline__ double2 recomb_df_node(const RecombCoef* __restrict__
   return make_double2(f2d_bits(r.hi) + f2d_bits(r.lo), f2d_bits(s.hi) + f2d_bits(s.lo));
 }
 
-__global__ void k_kry_recomb_df(long long n, double2* out, int64_t so, const double2* V0, int64_t s0,
-                                const double2* Vw, int64_t sw, const KryOrb* kry) {
+__global__ void k_kry_recomb_df(long long n, double2* out, int64_t so, const double2* Vw, int64_t sw,
+                                const KryOrb* kry) {
   __shared__ RecombCoef cf[TDKS_KMAX];
   const int o = blockIdx.y;
   const KryOrb& K = kry[o];
@@ -494,12 +514,11 @@ __global__ void k_kry_recomb_df(long long n, double2* out, int64_t so, const dou
   const int m = K.k;
   for (int j = threadIdx.x; j < m; j += blockDim.x) cf[j] = recomb_coef(K.nrm * K.s[j], K.yre[j], K.yim[j]);
   __syncthreads();
-  const double2* v0 = V0 + (long long)o * s0;
   const double2* vw = Vw + (long long)o * sw;
   double2* dst = out + (long long)o * so;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x)
-    dst[i] = recomb_df_node(cf, m, v0, vw, n, i);
+    dst[i] = recomb_df_node(cf, m, vw, vw + n, n, i);
 }
 
 __global__ void k_kry_after(KryOrb* kry, int n_orb) {
@@ -844,7 +863,7 @@ static tdks_status ensure_krylov(tdks_ctx* c, int w, int n_orb, int kmax) {
   if (c->d_Vw[w] && c->Vw_orb[w] >= n_orb && c->Vw_kmax[w] == kmax) return TDKS_OK;
   if (c->d_Vw[w]) cudaFree(c->d_Vw[w]);
   c->d_Vw[w] = nullptr;
-  const size_t bytes = (size_t)n_orb * kmax * c->n_int * sizeof(double2);
+  const size_t bytes = (size_t)n_orb * (kmax + 1) * c->n_int * sizeof(double2);
   if (cudaMalloc(&c->d_Vw[w], bytes) != cudaSuccess) {
     cudaGetLastError();
     return tdks_fail(c, TDKS_ERR_NOMEM, "Krylov basis (" + std::to_string(bytes >> 20) + " MiB)");
@@ -887,8 +906,9 @@ tdks_status run_expm(tdks_ctx* c, const double2* in, double2* out, int n_orb, do
 
 // Lanczos exponential with workspace w (0 for propagation; 1 is a second basis
 // kept alive alongside the first by the adjoint).  The basis V_0 = in (when no
-// sub-step is needed), V_1.. in the workspace, and the per-orbital state stay
-// valid until the next call on the same workspace.
+// sub-step is needed), V_1.. are V_j at j n of each orbital's block of (k_max + 1) n entries
+// in the workspace; they and the per-orbital state stay valid until the next call on the
+// same workspace.
 __global__ void k_kry_ctl(const KryOrb* __restrict__ kry, int n_orb, double theta, int mixed,
                           cudaGraphConditionalHandle h64, cudaGraphConditionalHandle h32,
                           int* __restrict__ n32) {
@@ -933,20 +953,18 @@ __global__ void k_stamp(unsigned long long* t) {
 // fused three-term update (contraction arithmetic pj), the optional CGS2 passes, and the
 // small exponential with the stopping decision.  Timing of the application: stamp
 // (device loop) receives %globaltimer before and after it, ev (host loop) two events.
-static tdks_status iteration_kernels(tdks_ctx* c, KryOrb* kry, const double2* cur, double2* VW,
-                                     int64_t wsorb, long long n, int n_orb, int j, int kmax, int pj,
+static tdks_status iteration_kernels(tdks_ctx* c, KryOrb* kry, double2* VW, int64_t wsorb,
+                                     long long n, int n_orb, int j, int kmax, int pj,
                                      double tol, int nb, int nasm, unsigned long long* stamp,
                                      cudaEvent_t* ev) {
   const int64_t ps = c->part_stride;
   double* apart = c->d_part;
   double* npart = c->d_part + (int64_t)c->n_orb * ps;
-  const double2* Vj = (j == 0) ? cur : VW + (int64_t)(j - 1) * n;
-  const int64_t sj = (j == 0) ? n : wsorb;
-  const double2* Vm = (j == 1) ? cur : (j >= 2 ? VW + (int64_t)(j - 2) * n : nullptr);
-  const int64_t sm = (j == 1) ? n : wsorb;
-  double2* Vn = VW + (int64_t)j * n;
+  const double2* Vj = VW + (int64_t)j * n;
+  const double2* Vm = j > 0 ? Vj - n : nullptr;
+  double2* Vn = VW + (int64_t)(j + 1) * n;
   // Hbar q_j and the three-term update fused: V_{j+1} = Hbar q_j - alpha_j q_j - beta q_{j-1}
-  ApplyArgs a{Vj, sj, Vn, wsorb, n_orb, kry, j, apart, ps, 1, Vm, sm, npart, ps, 0};
+  ApplyArgs a{Vj, wsorb, Vn, wsorb, n_orb, kry, j, apart, ps, 1, Vm, wsorb, npart, ps, 0};
   if (stamp) k_stamp<<<1, 1, 0, c->stream>>>(stamp + 2 * j);
   if (ev) TDKS_CU(c, cudaEventRecord(ev[0], c->stream));
   TDKS_TRY(launch_hbar_apply(c, a, pj));
@@ -955,13 +973,13 @@ static tdks_status iteration_kernels(tdks_ctx* c, KryOrb* kry, const double2* cu
   if (c->lanczos_reorth) {
     TDKS_TRY(ensure_reorth(c));
     for (int pass = 0; pass < 2; ++pass) {
-      k_ro_dot<<<dim3(kRoChunks, j + 1, n_orb), kThreads, 0, c->stream>>>(n, cur, n, VW, wsorb, j, kry,
+      k_ro_dot<<<dim3(kRoChunks, j + 1, n_orb), kThreads, 0, c->stream>>>(n, VW, wsorb, VW + n, wsorb, j, kry,
                                                                           c->d_ro_part);
       k_ro_fin<<<dim3(j + 1, n_orb), 32, 0, c->stream>>>(kry, c->d_ro_part, kRoChunks, c->d_ro_h);
-      k_ro_update<<<dim3(nb, n_orb), kThreads, 0, c->stream>>>(n, cur, n, VW, wsorb, j, kry, c->d_ro_h);
+      k_ro_update<<<dim3(nb, n_orb), kThreads, 0, c->stream>>>(n, VW, wsorb, VW + n, wsorb, j, kry, c->d_ro_h);
     }
     // ||w||^2 after the passes (the assembly's and the nonlocal partials are stale)
-    k_norm_part<<<dim3(nb, n_orb), kThreads, 0, c->stream>>>(VW + (int64_t)j * n, wsorb, n, kry, npart, ps);
+    k_norm_part<<<dim3(nb, n_orb), kThreads, 0, c->stream>>>(Vn, wsorb, n, kry, npart, ps);
     k_kry_exp<<<n_orb, kExpThreads, 0, c->stream>>>(j, kmax, tol, kry, npart, ps, nb, nullptr, 0);
   } else {
     k_kry_exp<<<n_orb, kExpThreads, 0, c->stream>>>(j, kmax, tol, kry, npart, ps, nasm, kb_norm_parts(c),
@@ -980,10 +998,10 @@ static tdks_status iteration_kernels(tdks_ctx* c, KryOrb* kry, const double2* cu
 // iteration whose condition stays 0 is skipped by the graph, so one launch runs the
 // whole loop and the host reads the Lanczos state once per sub-step instead of once per
 // iteration.  Each iteration keeps its own launch parameters (the kernels are those of
-// the host-driven loop), so the results are identical.  Graphs are cached per
-// starting vector and settings.
+// the host-driven loop), so the results are identical.  The starting vector is copied into
+// the basis first, so a graph depends on the workspace and the settings alone and serves
+// every starting vector (capturing and instantiating one takes milliseconds).
 struct KGraph {
-  const double2* cur = nullptr;
   const void* VW = nullptr;
   const void* evec = nullptr;
   const void* kb = nullptr;
@@ -1072,7 +1090,7 @@ static tdks_status add_if_nodes(tdks_ctx* c, cudaStream_t cap, const cudaGraphCo
   return TDKS_OK;
 }
 
-// Capture of iterations 0 .. kmax-1 of a sub-step starting from `cur`.
+// Capture of iterations 0 .. G.len-1 of a sub-step.
 static tdks_status capture_loop(tdks_ctx* c, KGraphCache* K, KGraph& G, KryOrb* kry, double2* VW,
                                 int64_t wsorb, long long n, int nb, int nasm) {
   const int kmax = G.kmax, n_orb = G.n_orb, L = G.len;
@@ -1094,7 +1112,7 @@ static tdks_status capture_loop(tdks_ctx* c, KGraphCache* K, KGraph& G, KryOrb* 
   auto ctl = [&](int jn) {
     k_kry_ctl<<<1, kThreads, 0, c->stream>>>(kry, n_orb, theta, mixed ? 1 : 0, h64[jn], h32[jn], K->d_n32);
   };
-  st = iteration_kernels(c, kry, G.cur, VW, wsorb, n, n_orb, 0, kmax, p64, G.tol, nb, nasm, stamp, nullptr);
+  st = iteration_kernels(c, kry, VW, wsorb, n, n_orb, 0, kmax, p64, G.tol, nb, nasm, stamp, nullptr);
   if (st == TDKS_OK && L > 1) ctl(1);
   for (int j = 1; j < L && st == TDKS_OK; ++j) {
     const int nv = mixed ? 2 : 1;
@@ -1108,7 +1126,7 @@ static tdks_status capture_loop(tdks_ctx* c, KGraphCache* K, KGraph& G, KryOrb* 
         break;
       }
       c->stream = K->body;
-      st = iteration_kernels(c, kry, G.cur, VW, wsorb, n, n_orb, j, kmax, v == 1 ? TDKS_FP32 : p64, G.tol,
+      st = iteration_kernels(c, kry, VW, wsorb, n, n_orb, j, kmax, v == 1 ? TDKS_FP32 : p64, G.tol,
                              nb, nasm, stamp, nullptr);
       if (st == TDKS_OK && j + 1 < L) ctl(j + 1);
       cudaGraph_t outb = nullptr;
@@ -1128,11 +1146,11 @@ static tdks_status capture_loop(tdks_ctx* c, KGraphCache* K, KGraph& G, KryOrb* 
   return TDKS_OK;
 }
 
-static tdks_status get_loop_graph(tdks_ctx* c, KGraphCache* K, const double2* cur, KryOrb* kry, double2* VW,
+static tdks_status get_loop_graph(tdks_ctx* c, KGraphCache* K, KryOrb* kry, double2* VW,
                                   int64_t wsorb, long long n, int n_orb, int kmax, int len, int prec,
                                   double tol, int nb, int nasm, KGraph** out) {
   for (auto& G : K->graphs) {
-    if (G.cur == cur && G.VW == VW && G.evec == c->d_evec && G.kb == c->kb && G.n_orb == n_orb &&
+    if (G.VW == VW && G.evec == c->d_evec && G.kb == c->kb && G.n_orb == n_orb &&
         G.kmax == kmax && G.len == len && G.prec == prec && G.reorth == c->lanczos_reorth && G.opc == c->opc_force &&
         G.timing == (c->timing ? 1 : 0) && G.tol == tol && G.relax == c->mixed_relax &&
         G.f32_stages == c->f32_stages) {
@@ -1144,7 +1162,6 @@ static tdks_status get_loop_graph(tdks_ctx* c, KGraphCache* K, const double2* cu
   TDKS_TRY(ensure_evec(c, n_orb));     // the capture must not reallocate the element results
   K->graphs.emplace_back();
   KGraph& G = K->graphs.back();
-  G.cur = cur;
   G.VW = VW;
   G.evec = c->d_evec;
   G.kb = c->kb;
@@ -1185,7 +1202,7 @@ tdks_status run_expm_ws(tdks_ctx* c, int w, const double2* in, double2* out, int
   double* npart = c->d_part + (int64_t)c->n_orb * ps;
   const int nb = grid_for(n);
   const int nasm = assemble_blocks(c, n_orb);   // partials of ||w||^2 per orbital
-  const int64_t wsorb = (int64_t)kmax * n;   // stride between orbitals in the workspace
+  const int64_t wsorb = (int64_t)(kmax + 1) * n;   // V_0 .. V_kmax of one orbital
   std::vector<KrySummary> h(n_orb);
   // the device-driven loop, unless disabled or the stream is being captured by the caller
   bool device_loop = c->device_loop != 0;
@@ -1208,7 +1225,7 @@ tdks_status run_expm_ws(tdks_ctx* c, int w, const double2* in, double2* out, int
   int n_active = n_orb;
   const double2* cur = in;
   for (int sub = 0; sub <= TDKS_MAX_SUBSTEPS; ++sub) {
-    k_norm_part<<<dim3(nb, n_orb), kThreads, 0, c->stream>>>(cur, n, n, kry, npart, ps);
+    k_copy_norm<<<dim3(nb, n_orb), kThreads, 0, c->stream>>>(cur, VW, wsorb, n, kry, npart, ps);
     k_kry_start<<<n_orb, kThreads, 0, c->stream>>>(kry, npart, ps, nb);
     c->n_launch += 2;
     TDKS_CU(c, cudaGetLastError());
@@ -1216,7 +1233,7 @@ tdks_status run_expm_ws(tdks_ctx* c, int w, const double2* in, double2* out, int
     KGraph* G = nullptr;
     const int len = device_loop ? (K->len_hint < kmax ? K->len_hint : kmax) : 0;
     if (device_loop) {
-      if (get_loop_graph(c, K, cur, kry, VW, wsorb, n, n_orb, kmax, len, prec, tol, nb, nasm, &G) != TDKS_OK) {
+      if (get_loop_graph(c, K, kry, VW, wsorb, n, n_orb, kmax, len, prec, tol, nb, nasm, &G) != TDKS_OK) {
         // capture is not available here: the host-driven loop from now on
         cudaGetLastError();
         K->broken = true;
@@ -1273,7 +1290,7 @@ tdks_status run_expm_ws(tdks_ctx* c, int w, const double2* in, double2* out, int
           if (emax <= c->mixed_relax * tol) pj = TDKS_FP32;
         }
         if (pj == TDKS_FP32 && prec == TDKS_MIXED) c->n_apply_fp32 += 1;
-        TDKS_TRY(iteration_kernels(c, kry, cur, VW, wsorb, n, n_orb, j, kmax, pj, tol, nb, nasm, nullptr,
+        TDKS_TRY(iteration_kernels(c, kry, VW, wsorb, n, n_orb, j, kmax, pj, tol, nb, nasm, nullptr,
                                    c->timing ? c->ev : nullptr));
         c->n_apply_units += (int64_t)n_active * c->n_elem;
         c->n_launch += c->lanczos_reorth ? 8 : 1;
@@ -1289,10 +1306,9 @@ tdks_status run_expm_ws(tdks_ctx* c, int w, const double2* in, double2* out, int
       }
     }
     if (prec == TDKS_DF64 || prec == TDKS_MIXED)
-      k_kry_recomb_df<<<dim3(nb, n_orb), kThreads, 0, c->stream>>>(n, out, n, cur, n, VW, wsorb, kry);
+      k_kry_recomb_df<<<dim3(nb, n_orb), kThreads, 0, c->stream>>>(n, out, n, VW, wsorb, kry);
     else
-      k_kry_recomb<<<dim3(nb, n_orb), kThreads, 0, c->stream>>>(n, out, n, cur, n, VW, wsorb,
-                                                               kmax, kry);
+      k_kry_recomb<<<dim3(nb, n_orb), kThreads, 0, c->stream>>>(n, out, n, VW, wsorb, kry);
     k_kry_after<<<(n_orb + 63) / 64, 64, 0, c->stream>>>(kry, n_orb);
     c->n_launch += 2;
     TDKS_CU(c, cudaGetLastError());

@@ -124,7 +124,7 @@ struct tdks_ctx {
   double* d_fdmL[3] = {nullptr, nullptr, nullptr};    // per-axis eigenvalues
   double *d_z = nullptr, *d_t1 = nullptr, *d_t2 = nullptr, *d_invdiag = nullptr;
   // Krylov
-  double2* d_Vw[2] = {nullptr, nullptr};      // Krylov bases [n_orb][kmax][n_int]
+  double2* d_Vw[2] = {nullptr, nullptr};      // Krylov bases [n_orb][kmax + 1][n_int]
   int Vw_orb[2] = {0, 0}, Vw_kmax[2] = {0, 0};
   KryOrb* d_kryw[2] = {nullptr, nullptr};     // per-orbital Lanczos state of each basis
   double2* d_psi_half = nullptr;
