@@ -96,7 +96,8 @@ struct AdjState {
           *mus = nullptr;
   double *gh1 = nullptr, *gh2 = nullptr, *gh1n = nullptr, *grho = nullptr, *gvmid = nullptr,
          *gvpred = nullptr, *ny = nullptr, *nz = nullptr;
-  double2* d_coef = nullptr;
+  double2* d_coef = nullptr;    // Frechet coefficients of coef_nodes quadrature nodes
+  int coef_nodes = 0;
   int* d_k = nullptr;
   bool ready = false;
 };
@@ -131,13 +132,63 @@ struct TriEig {
   std::vector<double> ev, lam;
 };
 
+// Implicit symmetric QR steps with the Wilkinson shift (Golub & Van Loan, Matrix
+// Computations, Sec. 8.3.3): a bulge chased down each unreduced block, O(m^2) rotations of
+// the vectors' columns in all; the cyclic Jacobi iteration (O(m^3) a sweep, 0.3 ms at m = 20,
+// two per Frechet term) is left for a block that does not converge.
+bool tri_qr(int m, std::vector<double>& d, std::vector<double>& e, std::vector<double>& Z) {
+  const double eps = 2.2e-16;
+  int hi = m - 1, steps = 0;
+  while (hi > 0) {
+    for (int k = 0; k < hi; ++k)
+      if (std::fabs(e[k]) <= eps * (std::fabs(d[k]) + std::fabs(d[k + 1]))) e[k] = 0.0;
+    if (e[hi - 1] == 0.0) {
+      --hi;
+      steps = 0;
+      continue;
+    }
+    if (++steps > 60) return false;
+    int lo = hi - 1;
+    while (lo > 0 && e[lo - 1] != 0.0) --lo;
+    const double dl = 0.5 * (d[hi - 1] - d[hi]);
+    const double mu = d[hi] - e[hi - 1] * e[hi - 1] / (dl + std::copysign(std::hypot(dl, e[hi - 1]), dl));
+    double x = d[lo] - mu, z = e[lo];
+    for (int k = lo; k < hi; ++k) {
+      const double r = std::hypot(x, z);
+      const double cs = r > 0.0 ? x / r : 1.0, sn = r > 0.0 ? z / r : 0.0;
+      if (k > lo) e[k - 1] = r;
+      const double a = d[k], b = e[k], g = d[k + 1];
+      d[k] = cs * cs * a + 2.0 * cs * sn * b + sn * sn * g;
+      d[k + 1] = sn * sn * a - 2.0 * cs * sn * b + cs * cs * g;
+      e[k] = cs * sn * (g - a) + (cs * cs - sn * sn) * b;
+      if (k + 1 < hi) {
+        x = e[k];
+        z = sn * e[k + 1];
+        e[k + 1] *= cs;
+      }
+      for (int i = 0; i < m; ++i) {
+        double* row = &Z[(size_t)i * m + k];
+        const double t = row[0];
+        row[0] = cs * t + sn * row[1];
+        row[1] = cs * row[1] - sn * t;
+      }
+    }
+  }
+  return true;
+}
+
 void tri_eig(const double* alpha, const double* beta, int m, TriEig& E) {
+  E.m = m;
+  E.lam.assign(alpha, alpha + m);
+  std::vector<double> off(beta, beta + (m > 1 ? m - 1 : 0));
+  E.ev.assign((size_t)m * m, 0.0);
+  for (int i = 0; i < m; ++i) E.ev[(size_t)i * m + i] = 1.0;
+  if (tri_qr(m, E.lam, off, E.ev)) return;
   std::vector<double> C((size_t)m * m, 0.0);
   for (int i = 0; i < m; ++i) {
     C[(size_t)i * m + i] = alpha[i];
     if (i + 1 < m) C[(size_t)i * m + i + 1] = C[(size_t)(i + 1) * m + i] = beta[i];
   }
-  E.m = m;
   tdks_sym_eigen(C, m, E.ev, E.lam);
 }
 
@@ -197,8 +248,17 @@ tdks_status frechet(tdks_ctx* c, AdjState* A, const double2* psi, const double2*
     sx[i] = 0.5 * (x + 1.0);
     sw[i] = 1.0 / ((1.0 - x * x) * dp * dp);      // (2 / ((1-x^2) P'^2)) / 2
   }
+  // coefficients of every node first, in one copy: [node][psi | lambda][orbital][k]
   const int kcap = TDKS_KMAX;
-  std::vector<double2> cp((size_t)n_orb * kcap), cl((size_t)n_orb * kcap);
+  const size_t node = 2 * (size_t)n_orb * kcap;
+  if (A->coef_nodes < n_s) {
+    cudaFree(A->d_coef);
+    A->d_coef = nullptr;
+    A->coef_nodes = 0;
+    TDKS_TRY(amalloc(c, &A->d_coef, node * n_s));
+    A->coef_nodes = n_s;
+  }
+  std::vector<double2> cf(node * n_s);
   std::vector<int> kk(2 * n_orb);
   for (int o = 0; o < n_orb; ++o) {
     kk[o] = kp[o].k;
@@ -206,41 +266,33 @@ tdks_status frechet(tdks_ctx* c, AdjState* A, const double2* psi, const double2*
   }
   TDKS_CU(c, cudaMemcpyAsync(A->d_k, kk.data(), 2 * n_orb * sizeof(int), cudaMemcpyHostToDevice, c->stream));
   const int nb = grid_for(n);
-  std::vector<TriEig> ep(n_orb), el(n_orb);
-  for (int o = 0; o < n_orb; ++o) {
-    tri_eig(kp[o].alpha, kp[o].beta, kp[o].k, ep[o]);
-    tri_eig(kl[o].alpha, kl[o].beta, kl[o].k, el[o]);
-  }
   std::vector<std::complex<double>> y;
-  for (int i = 0; i < n_s; ++i) {
-    for (int o = 0; o < n_orb; ++o) {
-      const KryOrb& P = kp[o];
-      tri_exp(ep[o], tau * sx[i], y);
-      for (int j = 0; j < P.k; ++j) {
-        const std::complex<double> v = P.nrm * P.s[j] * y[j];
-        cp[(size_t)o * kcap + j] = make_double2(v.real(), v.imag());
-      }
-      const KryOrb& L = kl[o];
-      tri_exp(el[o], -tau * (1.0 - sx[i]), y);
-      for (int j = 0; j < L.k; ++j) {
-        const std::complex<double> v = L.nrm * L.s[j] * y[j];
-        cl[(size_t)o * kcap + j] = make_double2(v.real(), v.imag());
+  for (int o = 0; o < n_orb; ++o)
+    for (int h = 0; h < 2; ++h) {
+      const KryOrb& P = h == 0 ? kp[o] : kl[o];
+      TriEig e;
+      tri_eig(P.alpha, P.beta, P.k, e);
+      for (int i = 0; i < n_s; ++i) {
+        tri_exp(e, h == 0 ? tau * sx[i] : -tau * (1.0 - sx[i]), y);
+        double2* dst = &cf[node * i + ((size_t)h * n_orb + o) * kcap];
+        for (int j = 0; j < P.k; ++j) {
+          const std::complex<double> v = P.nrm * P.s[j] * y[j];
+          dst[j] = make_double2(v.real(), v.imag());
+        }
       }
     }
-    TDKS_CU(c, cudaMemcpyAsync(A->d_coef, cp.data(), cp.size() * sizeof(double2), cudaMemcpyHostToDevice,
-                               c->stream));
-    k_combine_basis<<<dim3(nb, n_orb), kThreads, 0, c->stream>>>(
-        n, A->phis, c->d_Vw[0], (int64_t)(c->Vw_kmax[0] + 1) * n, A->d_coef, kcap, A->d_k);
-    TDKS_CU(c, cudaMemcpyAsync(A->d_coef + (size_t)n_orb * kcap, cl.data(), cl.size() * sizeof(double2),
-                               cudaMemcpyHostToDevice, c->stream));
-    k_combine_basis<<<dim3(nb, n_orb), kThreads, 0, c->stream>>>(
-        n, A->mus, c->d_Vw[1], (int64_t)(c->Vw_kmax[1] + 1) * n, A->d_coef + (size_t)n_orb * kcap, kcap,
-        A->d_k + n_orb);
+  TDKS_CU(c, cudaMemcpyAsync(A->d_coef, cf.data(), cf.size() * sizeof(double2), cudaMemcpyHostToDevice, c->stream));
+  for (int i = 0; i < n_s; ++i) {
+    const double2* ci = A->d_coef + node * i;
+    k_combine_basis<<<dim3(nb, n_orb), kThreads, 0, c->stream>>>(n, A->phis, c->d_Vw[0],
+                                                                 (int64_t)(c->Vw_kmax[0] + 1) * n, ci, kcap, A->d_k);
+    k_combine_basis<<<dim3(nb, n_orb), kThreads, 0, c->stream>>>(n, A->mus, c->d_Vw[1],
+                                                                 (int64_t)(c->Vw_kmax[1] + 1) * n,
+                                                                 ci + (size_t)n_orb * kcap, kcap, A->d_k + n_orb);
     c->n_launch += 2;
     TDKS_TRY(launch_cross(c, A->mus, A->phis, n_orb, sw[i] * tau, g_out));
-    // the host coefficient arrays are reused: wait for the copies of this node
-    TDKS_CU(c, cudaStreamSynchronize(c->stream));
   }
+  TDKS_CU(c, cudaStreamSynchronize(c->stream));   // the host coefficients were copied from pageable memory
   return TDKS_OK;
 }
 
@@ -348,7 +400,6 @@ tdks_status tdks_objective_backward(tdks_ctx* c, int n_s, double* dJdE_host) {
     for (auto f : fs) TDKS_TRY(amalloc(c, f, nf));
     TDKS_TRY(amalloc(c, &A->ny, nn));
     TDKS_TRY(amalloc(c, &A->nz, nn));
-    TDKS_TRY(amalloc(c, &A->d_coef, 2 * (size_t)n_orb * TDKS_KMAX));
     TDKS_TRY(amalloc(c, &A->d_k, 2 * (size_t)n_orb));
   }
   TDKS_CU(c, cudaMemsetAsync(A->lam, 0, nv * sizeof(double2), c->stream));
