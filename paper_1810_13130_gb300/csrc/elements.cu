@@ -578,7 +578,7 @@ __device__ __forceinline__ int node_elems(int I, int p, int n, int* e, int* loc)
 // (the fixed-point kernel leaves the scale out): qs = s_j scales them here, 1 otherwise.
 // The degree is a compile-time
 // constant: the node -> (element, local index) split is a multiply-shift.
-template <int P1, typename T>
+template <int P1, typename T, bool kMany>
 __device__ __forceinline__ double assemble_rows(const Geom& g, const Cx<T>* __restrict__ evo,
                                                 const double2* qj, const double2* qm,
                                                 double2* out, double qs, double ca, double cb, int lanczos,
@@ -594,97 +594,110 @@ __device__ __forceinline__ double assemble_rows(const Geom& g, const Cx<T>* __re
   const int tI = nix >= nt ? (int)threadIdx.x : (int)threadIdx.x % nix;
   const int tstep = nix >= nt ? nt : nix;
   double acc = 0.0;
-  if (tr >= rpb) return acc;
   const long long xstride = P3;                             // next element along x
-  for (int r = r0 + tr * rstride; r < rows; r += rpb * rstride) {
-    const int J = r % g.niy + 1, K = r / g.niy + 1;
-    int ey[2], by[2], ez[2], bz[2];
-    const int ny = node_elems(J, p, g.ny, ey, by);
-    const int nz = node_elems(K, p, g.nz, ez, bz);
-    // element rows (y, z) holding this node row, in the order z then y
-    long long base[4] = {0, 0, 0, 0};
-    const int nb = ny * nz;
-#pragma unroll
-    for (int kz = 0; kz < 2; ++kz)
-#pragma unroll
-      for (int ky = 0; ky < 2; ++ky)
-        if (kz < nz && ky < ny)
-          base[kz * ny + ky] = (long long)g.nx * (ey[ky] + (long long)g.ny * ez[kz]) * P3 + bz[kz] * P2 + by[ky] * P1;
-    const double syz = g.s[1][J] * g.s[2][K] * qs;
-    const float syzf = g.sf[1][J] * g.sf[2][K];
-    const long long rowbase = (long long)g.nix * (r);
-    for (int I = tI + 1; I <= g.nix; I += tstep) {
-      // x: one element inside, two on a shared face (left element first)
-      const int eh = I / p, l = I - eh * p;
-      long long xo[2] = {0, 0};
-      int nxc;
-      if (l != 0) {
-        xo[0] = eh * xstride + l;
-        nxc = 1;
-      } else {
-        nxc = 0;
-        if (eh - 1 >= 0) xo[nxc++] = (eh - 1) * xstride + p;
-        if (eh < g.nx) xo[nxc++] = eh * xstride;
+  // FP64 operations are what this costs (79 % of the FP64 pipe before, 12 operations a node
+  // and more for half-empty warps), so the first contribution is taken as it is instead of
+  // added to zero and, with many rows per block (kMany), the row scales are formed once per
+  // row, not per node (FP64 Lanczos step of 16 orbitals on 16^3 elements, p = 6: 491 -> 397 us;
+  // a block with a few rows only is bound by latency, and the barriers cost more than they save).
+  constexpr int kRows = 128;
+  __shared__ double srow[kMany ? kRows : 1];
+  for (int k0 = 0; r0 + k0 * rstride < rows; k0 += kRows) {
+    if (kMany && !kF32) {
+      __syncthreads();
+      for (int k = threadIdx.x; k < kRows && r0 + (k0 + k) * rstride < rows; k += nt) {
+        const int r = r0 + (k0 + k) * rstride;
+        srow[k] = g.s[1][r % g.niy + 1] * g.s[2][r / g.niy + 1] * qs;
       }
-      double re = 0.0, im = 0.0;
-      float fre = 0.f, fim = 0.f;
-      Df dre{0.f, 0.f}, dim{0.f, 0.f};
-      // exactly nb * nxc additions in the fixed order (z, y, then x); the offsets are
-      // picked by selects so that base[] and xo[] stay in registers (an unrolled loop
-      // with predicates would turn into 16 unconditional FP64 additions per node)
-      const int ncon = nb * nxc;
-      for (int tcon = 0; tcon < ncon; ++tcon) {
-          const int k = nxc == 2 ? (tcon >> 1) : tcon;
-          const long long bk = k == 0 ? base[0] : (k == 1 ? base[1] : (k == 2 ? base[2] : base[3]));
+      __syncthreads();
+    }
+    for (int k = tr; tr < rpb && k < kRows; k += rpb) {
+      const int r = r0 + (k0 + k) * rstride;
+      if (r >= rows) break;
+      const int J = r % g.niy + 1, K = r / g.niy + 1;
+      int ey[2], by[2], ez[2], bz[2];
+      const int ny = node_elems(J, p, g.ny, ey, by);
+      const int nz = node_elems(K, p, g.nz, ez, bz);
+      // element rows (y, z) holding this node row, in the order z then y
+      long long base[4] = {0, 0, 0, 0};
+      const int nb = ny * nz;
+#pragma unroll
+      for (int kz = 0; kz < 2; ++kz)
+#pragma unroll
+        for (int ky = 0; ky < 2; ++ky)
+          if (kz < nz && ky < ny)
+            base[kz * ny + ky] = (long long)g.nx * (ey[ky] + (long long)g.ny * ez[kz]) * P3 + bz[kz] * P2 + by[ky] * P1;
+      const double syz = kF32 ? 0.0 : (kMany ? srow[kMany ? k : 0] : g.s[1][J] * g.s[2][K] * qs);
+      const float syzf = g.sf[1][J] * g.sf[2][K];
+      const long long rowbase = (long long)g.nix * (r);
+      for (int I = tI + 1; I <= g.nix; I += tstep) {
+        // x: one element inside, two on a shared face (left element first)
+        const int eh = I / p, l = I - eh * p;
+        long long xo[2] = {0, 0};
+        int nxc;
+        if (l != 0) {
+          xo[0] = eh * xstride + l;
+          nxc = 1;
+        } else {
+          nxc = 0;
+          if (eh - 1 >= 0) xo[nxc++] = (eh - 1) * xstride + p;
+          if (eh < g.nx) xo[nxc++] = eh * xstride;
+        }
+        // exactly nb * nxc contributions in the fixed order (z, y, then x); the offsets are
+        // picked by selects so that base[] and xo[] stay in registers (an unrolled loop
+        // with predicates would turn into 16 unconditional FP64 additions per node)
+        const int ncon = nb * nxc;
+        Cx<T> sum = evo[base[0] + xo[0]];
+        for (int tcon = 1; tcon < ncon; ++tcon) {
+          const int kc = nxc == 2 ? (tcon >> 1) : tcon;
+          const long long bk = kc == 0 ? base[0] : (kc == 1 ? base[1] : (kc == 2 ? base[2] : base[3]));
           const long long xk = (nxc == 2 && (tcon & 1)) ? xo[1] : xo[0];
           const Cx<T> c = evo[bk + xk];
-          if constexpr (kF32) {
-            fre += c.re;
-            fim += c.im;
-          } else if constexpr (kDF) {
-            dre = df_add(dre, c.re);
-            dim = df_add(dim, c.im);
+          if constexpr (kDF) {
+            sum.re = df_add(sum.re, c.re);
+            sum.im = df_add(sum.im, c.im);
           } else {
-            re += c.re;
-            im += c.im;
+            sum.re += c.re;
+            sum.im += c.im;
           }
         }
-      if constexpr (kDF) {
-        re = f2d_bits(dre.hi) + f2d_bits(dre.lo);
-        im = f2d_bits(dim.hi) + f2d_bits(dim.lo);
-      }
-      const long long idx = rowbase + (I - 1);
-      double2 w;
-      if constexpr (kF32) {   // sum, scale and convert without the FP64 pipe
-        const float f = g.sf[0][I] * syzf;
-        w = make_double2(f2d_bits(f * fre), f2d_bits(f * fim));
-      } else {
-        const double f = g.s[0][I] * syz;
-        w = make_double2(f * re, f * im);
-      }
-      if (lanczos) {
-        const double2 x = qj[idx];
-        w.x = fma(-ca, x.x, w.x);
-        w.y = fma(-ca, x.y, w.y);
-        if (qm) {
-          const double2 y = qm[idx];
-          w.x = fma(-cb, y.x, w.x);
-          w.y = fma(-cb, y.y, w.y);
+        const long long idx = rowbase + (I - 1);
+        double2 w;
+        if constexpr (kF32) {   // sum, scale and convert without the FP64 pipe
+          const float f = g.sf[0][I] * syzf;
+          w = make_double2(f2d_bits(f * sum.re), f2d_bits(f * sum.im));
+        } else if constexpr (kDF) {
+          const double f = g.s[0][I] * syz;
+          w = make_double2(f * (f2d_bits(sum.re.hi) + f2d_bits(sum.re.lo)),
+                           f * (f2d_bits(sum.im.hi) + f2d_bits(sum.im.lo)));
+        } else {
+          const double f = g.s[0][I] * syz;
+          w = make_double2(f * sum.re, f * sum.im);
         }
-        acc = fma(w.x, w.x, fma(w.y, w.y, acc));
+        if (lanczos) {
+          const double2 x = qj[idx];
+          w.x = fma(-ca, x.x, w.x);
+          w.y = fma(-ca, x.y, w.y);
+          if (qm) {
+            const double2 y = qm[idx];
+            w.x = fma(-cb, y.x, w.x);
+            w.y = fma(-cb, y.y, w.y);
+          }
+          acc = fma(w.x, w.x, fma(w.y, w.y, acc));
+        }
+        if (accumulate) {
+          const double2 o2 = out[idx];
+          w.x += o2.x;
+          w.y += o2.y;
+        }
+        out[idx] = w;
       }
-      if (accumulate) {
-        const double2 o2 = out[idx];
-        w.x += o2.x;
-        w.y += o2.y;
-      }
-      out[idx] = w;
     }
   }
   return acc;
 }
 
-template <int P1, typename T>
+template <int P1, typename T, bool kMany>
 __global__ void __launch_bounds__(128) k_assemble(Geom g, const Cx<T>* __restrict__ ev, ApplyArgs a) {
   __shared__ double red[4];
   const int o = blockIdx.y;
@@ -703,7 +716,7 @@ __global__ void __launch_bounds__(128) k_assemble(Geom g, const Cx<T>* __restric
   const double2* qj = a.in_base + (long long)o * a.in_stride;
   const double2* qm = a.vm_base ? a.vm_base + (long long)o * a.vm_stride : nullptr;
   double2* out = a.out_base + (long long)o * a.out_stride;
-  const double acc = assemble_rows<P1, T>(g, evo, qj, qm, out, qs, ca, cb, a.lanczos, a.accumulate,
+  const double acc = assemble_rows<P1, T, kMany>(g, evo, qj, qm, out, qs, ca, cb, a.lanczos, a.accumulate,
                                           blockIdx.x, gridDim.x);
   if (a.npart) {
     const double s = block_sum(acc, red);
@@ -942,7 +955,7 @@ __global__ void __launch_bounds__(128) k_bassemble(const BSys* __restrict__ sys,
   const Cx<T>* evo = static_cast<const Cx<T>*>(S.ev) +
                      (long long)w.o * S.n_elem * (P1 * P1 * P1) * batch_omul<T>();
   const double qs = std::is_same<T, double>::value ? K.s[j] : 1.0;
-  const double acc = assemble_rows<P1, T>(S.g, evo, qj, qm, out, qs, ca, cb, 1, 0, w.rblk, S.n_rblk);
+  const double acc = assemble_rows<P1, T, true>(S.g, evo, qj, qm, out, qs, ca, cb, 1, 0, w.rblk, S.n_rblk);
   const double sum = block_sum(acc, red);
   if (threadIdx.x == 0) S.npart[(long long)w.o * S.n_rblk + w.rblk] = sum;
 }
@@ -1494,6 +1507,14 @@ int elem_blocks_t(const tdks_ctx* c) {
   return (int)((c->n_elem + Cfg<P1>::E - 1) / Cfg<P1>::E);
 }
 
+template <int P1, typename T>
+void assemble_t(tdks_ctx* c, const Geom& g, const Cx<T>* ev, const ApplyArgs& a) {
+  const int rows = c->Ni[1] * c->Ni[2], gx = assemble_blocks(c, a.n_orb);
+  const int rpb = c->Ni[0] >= 128 ? 1 : 128 / c->Ni[0];      // rows in flight per block
+  if (rows > 4 * gx * rpb) k_assemble<P1, T, true><<<dim3(gx, a.n_orb), 128, 0, c->stream>>>(g, ev, a);
+  else k_assemble<P1, T, false><<<dim3(gx, a.n_orb), 128, 0, c->stream>>>(g, ev, a);
+}
+
 template <int P1, typename T, bool kBF = false>
 tdks_status hbar_t(tdks_ctx* c, const ApplyArgs& a) {
   constexpr int P2 = Cfg<P1>::P2, P3 = Cfg<P1>::P3, E = Cfg<P1>::E;
@@ -1562,8 +1583,7 @@ tdks_status hbar_t(tdks_ctx* c, const ApplyArgs& a) {
     k_alpha<<<a.n_orb, 256, 0, c->stream>>>(a.kry, a.part, a.part_stride, bpe, a.kj);
     if (c->kb) TDKS_TRY(kb_alpha(c, a));
   }
-  const int gx = assemble_blocks(c, a.n_orb);
-  k_assemble<P1, T><<<dim3(gx, a.n_orb), 128, 0, c->stream>>>(g, ev, a);
+  assemble_t<P1, T>(c, g, ev, a);
   if (c->kb) TDKS_TRY(kb_add(c, a));
   c->n_launch += (a.lanczos && a.kry && a.part) ? 3 : 2;
   c->n_apply_launch += 1;
@@ -1700,7 +1720,7 @@ tdks_status dens_adj_t(tdks_ctx* c, const double2* psi, int n_orb, const double*
       g, c->d_tab, psi, c->n_int, n_orb, c->d_occ, grho, ev);
   ApplyArgs a{psi, c->n_int, lam, c->n_int, n_orb, nullptr, 0, nullptr, 0, 0, nullptr, 0, nullptr, 0,
               accumulate};
-  k_assemble<P1, double><<<dim3(assemble_blocks(c, n_orb), n_orb), 128, 0, c->stream>>>(g, ev, a);
+  assemble_t<P1, double>(c, g, ev, a);
   c->n_launch += 2;
   TDKS_CU(c, cudaGetLastError());
   return TDKS_OK;
@@ -1941,7 +1961,7 @@ static tdks_status hbar_gll_t(tdks_ctx* c, const double2* psi, const double* vn,
   k_hbar_gll<P1><<<dim3(bpe, (n_orb + opc - 1) / opc), dim3(P2, E), smem, c->stream>>>(g, c->d_tab, psi, c->n_int,
                                                                                    n_orb, opc, ev);
   ApplyArgs a{psi, c->n_int, out, c->n_int, n_orb, nullptr, 0, nullptr, 0, 0, nullptr, 0, nullptr, 0, 0};
-  k_assemble<P1, double><<<dim3(assemble_blocks(c, n_orb), n_orb), 128, 0, c->stream>>>(g, ev, a);
+  assemble_t<P1, double>(c, g, ev, a);
   k_diag_add<<<608, 256, 0, c->stream>>>(c->n_int, n_orb, vn, psi, out);
   c->n_launch += 3;
   TDKS_CU(c, cudaGetLastError());
