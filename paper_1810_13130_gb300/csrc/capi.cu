@@ -360,6 +360,8 @@ tdks_status tdks_create(const tdks_mesh_desc* m, const tdks_system_desc* s, void
     c->fx.c = c->fx_c.data();
     c->fx.dK = c->d_fxK;
     c->fx.kinf = t.kw_inf;
+    c->fx_w = t.omega;
+    c->fx.w = c->fx_w.data();
   }
   if ((st = upload(c, &c->d_occ, c->occ)) != TDKS_OK) return fail(st);
   if ((st = upload(c, &c->d_R, c->R)) != TDKS_OK) return fail(st);

@@ -1227,63 +1227,6 @@ __global__ void __launch_bounds__(256) k_interp(Geom g, const double* __restrict
   }
 }
 
-// ---------------------------------------------------------------------------
-// Density rho(x_q) = sum_a occ_a |(B^(x)3 M^-1/2 psibar_a)(x_q)|^2   (Eq. 2)
-// ---------------------------------------------------------------------------
-template <int P1>
-__global__ void __launch_bounds__(256) k_density(Geom g, const double* __restrict__ tab,
-                                                 const double2* __restrict__ psi, int64_t stride,
-                                                 int n_orb, const double* __restrict__ occ,
-                                                 double* __restrict__ rho) {
-  constexpr int P2 = Cfg<P1>::P2, P3 = Cfg<P1>::P3;
-  constexpr int CS = 2 * (P1 / 2) * (P1 / 2) + 2 * (P1 / 2) + 1;
-  typedef Cx<double> V;
-  extern __shared__ __align__(16) unsigned char smem[];
-  double* sB = reinterpret_cast<double*>(smem);
-  const size_t off = (CS * sizeof(double) + 15) & ~size_t(15);
-  V* S1 = reinterpret_cast<V*>(smem + off) + (size_t)threadIdx.y * 2 * P3;
-  V* S2 = S1 + P3;
-  const int tid = threadIdx.x + blockDim.x * threadIdx.y;
-  const int nthr = blockDim.x * blockDim.y;
-  for (int i = tid; i < CS; i += nthr) sB[i] = tab[tab_off_csB(P1) + i];
-  const int u = threadIdx.x % P1, v = threadIdx.x / P1;
-  int ex = 0, ey = 0, ez = 0;
-  const bool valid = plain_elem(g, (long long)blockIdx.x * blockDim.y + threadIdx.y, ex, ey, ez);
-  __syncthreads();
-  const int I = ex * g.p + u, Jn = ey * g.p + v;
-  const bool inIJ = valid && I >= 1 && I <= g.nix && Jn >= 1 && Jn <= g.niy;
-  const double sxy = inIJ ? g.s[0][I] * g.s[1][Jn] : 0.0;
-  const long long base = inIJ ? (long long)(I - 1) + (long long)g.nix * (Jn - 1) : 0;
-  const long long plane = (long long)g.nix * g.niy;
-  double acc[P1];
-#pragma unroll
-  for (int q = 0; q < P1; ++q) acc[q] = 0.0;
-  for (int o = 0; o < n_orb; ++o) {
-    const double2* in = psi + (long long)o * stride;
-    V col[P1], uq[P1];
-#pragma unroll
-    for (int c = 0; c < P1; ++c) {
-      const int K = ez * g.p + c;
-      vzero(col[c]);
-      if (inIJ && K >= 1 && K <= g.niz) {
-        const double f = sxy * g.s[2][K];
-        const double2 w2 = in[base + plane * (K - 1)];
-        col[c].re = w2.x * f;
-        col[c].im = w2.y * f;
-      }
-    }
-    forward_lines<P1, V, double>(col, uq, S1, S2, sB, u, v);
-    const double f = occ[o];
-#pragma unroll
-    for (int q = 0; q < P1; ++q) acc[q] += f * (uq[q].re * uq[q].re + uq[q].im * uq[q].im);
-    __syncthreads();
-  }
-  if (valid) {
-    const long long e = ex + (long long)g.nx * (ey + (long long)g.ny * ez);
-    store_line(acc, rho + e * P3 + v * P2 + u * P1, 1);
-  }
-}
-
 // Density in the double-float runs: the interpolation to the Gauss points is a
 // cell-level contraction and runs in double-float (real, then imaginary part, as
 // in the split element kernel); |psi_q|^2 is formed in double-float, rounded once
@@ -1671,10 +1614,7 @@ tdks_status density_t(tdks_ctx* c, const double2* psi, int n_orb, double* rho, i
     k_density_df<P1><<<grid, block, smem, c->stream>>>(tdks_geom(c), (const Df*)c->d_tabdf, psi, c->n_int,
                                                       n_orb, c->d_occ, rho);
   } else {
-    const size_t smem = ((CS * sizeof(double) + 15) & ~size_t(15)) + (size_t)E * 2 * P3 * sizeof(Cx<double>);
-    TDKS_CU(c, set_smem(k_density<P1>, smem));
-    k_density<P1><<<grid, block, smem, c->stream>>>(tdks_geom(c), c->d_tab, psi, c->n_int, n_orb,
-                                                   c->d_occ, rho);
+    TDKS_CU(c, launch_density_fx(P1, tdks_geom(c), c->fx, psi, c->n_int, n_orb, c->d_occ, rho, c->stream));
   }
   c->n_launch += 1;
   TDKS_CU(c, cudaGetLastError());

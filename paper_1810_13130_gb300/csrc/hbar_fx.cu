@@ -41,6 +41,7 @@ struct FxTab {
   float k[2 * KS];      // their tail constants
   const double* dK;     // folded K' (device)
   double kinf;          // largest row sum of |K'|
+  double iw[P1];        // 1 / Gauss weight
 };
 
 // B' and B'^T in shared memory from p = 6 on (with constant-bank operands the compiler
@@ -81,6 +82,23 @@ __device__ __forceinline__ double fx_to_double(long long v, int eb) {
   const double dl = __hiloint2double(0x43300000 + eb, (int)(unsigned)v);   // 2^e (2^52 + vl)
   const double cc = __hiloint2double(0x45300000 + eb, (int)0x80100000u);   // 2^e (2^84 + 2^63 + 2^52)
   return (dh - cc) + dl;
+}
+
+// Integer and tail of a line as 62-bit integers: shifted left by the line's free bits (at
+// most 19; |f| < 8; returned), the tail rounded to the new unit by adding 1.5 2^(23 - s)
+template <int P1>
+__device__ __forceinline__ int fx_join(long long (&t)[P1], const float (&tf)[P1]) {
+  unsigned big = 0;
+#pragma unroll
+  for (int q = 0; q < P1; ++q) {
+    const int hw = (int)(t[q] >> 32);
+    big |= (unsigned)(hw ^ (hw >> 31));
+  }
+  const int s = min(__clz((int)big + 2) - 2, 19);
+  const int mg = 0x4b400000 - (s << 23);
+#pragma unroll
+  for (int q = 0; q < P1; ++q) t[q] = (t[q] << s) + (__float_as_int(tf[q] + __int_as_float(mg)) - mg);
+  return s;
 }
 
 // Elements [eidx] of the calling rows for the orbitals o_begin <= o < o_end that orb(o, in, sc)
@@ -326,19 +344,7 @@ __device__ __forceinline__ void hbar_elem_fx(const Geom& g, const FxTab<P1>& tab
         t[q] = x;
         tf[q] = xf;
       });
-      // integer and tail as one 62-bit integer: shifted left by the line's free bits (at most
-      // 19; |f| < 8), the tail rounded to the new unit by adding 1.5 2^(23 - s)
-      unsigned big = 0;
-#pragma unroll
-      for (int q = 0; q < P1; ++q) {
-        const int hw = (int)(t[q] >> 32);
-        big |= (unsigned)(hw ^ (hw >> 31));
-      }
-      const int s = min(__clz((int)big + 2) - 2, 19);
-      const int mg = 0x4b400000 - (s << 23);
-#pragma unroll
-      for (int q = 0; q < P1; ++q) t[q] = (t[q] << s) + (__float_as_int(tf[q] + __int_as_float(mg)) - mg);
-      const int es = (ec - s) << 20;
+      const int es = (ec - fx_join<P1>(t, tf)) << 20;
       if (valid) {
         double* dst = reinterpret_cast<double*>(evo) + comp;
         if (poison || eo != ec) {   // rare: non-finite, or results near the ends of the FP64 range
@@ -483,6 +489,118 @@ __global__ void __launch_bounds__(256, 2) k_hbar_batch_fx(const BSys* __restrict
   }
 }
 
+// Density rho(x_q) = sum_a occ_a |(B^(x)3 M^-1/2 psibar_a)(x_q)|^2 (Eq. 2): the three forward
+// contractions of the element kernel with B', one exponent per element and orbital; the
+// squares are formed and summed over the orbitals in FP64 and divided by the weights that B'
+// carries.  FP64 contractions were bound by the FP64 pipe (10 orbitals, 14^3 elements, p = 6:
+// 731 us, 394 us here; 16 orbitals, 16^3: 1.75 ms, 0.90 ms).
+template <int P1>
+__global__ void __launch_bounds__(256, 2) k_density_fx(Geom g, const __grid_constant__ FxTab<P1> tab,
+                                                       const double2* __restrict__ psi, int64_t stride, int n_orb,
+                                                       const double* __restrict__ occ, double* __restrict__ rho) {
+  constexpr int P2 = P1 * P1, P3 = P2 * P1, CS = FxTab<P1>::CS;
+  constexpr int LS = SplitLayout<P1, double>::LS, PS = SplitLayout<P1, double>::PS;
+  constexpr int LF = SplitLayout<P1, float>::LS, PF = SplitLayout<P1, float>::PS;
+  constexpr bool kBs = kFxBs<P1>;
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ FxC sB[kBs ? CS : 1];
+  __shared__ unsigned sM[2 * Cfg<P1>::E];
+  const int tid = threadIdx.x + blockDim.x * threadIdx.y, el = threadIdx.y;
+  if (kBs)
+    for (int i = tid; i < CS; i += blockDim.x * blockDim.y) sB[i] = tab.c[i];
+  if (tid < 2 * Cfg<P1>::E) sM[tid] = 0;
+  long long* const S1 = reinterpret_cast<long long*>(smem) + (size_t)el * SplitLayout<P1, double>::ES;
+  float* const F1 = reinterpret_cast<float*>(smem + (size_t)blockDim.y * SplitLayout<P1, double>::ES * sizeof(long long)) +
+                    (size_t)el * SplitLayout<P1, float>::ES;
+  long long* const S2 = S1 + P1 * PS;
+  float* const F2 = F1 + P1 * PF;
+  const int u = threadIdx.x % P1, v = threadIdx.x / P1;
+  const unsigned grp = __match_any_sync(__activemask(), el);
+  const bool lead = (tid & 31) == __ffs(grp) - 1;
+  int ex = 0, ey = 0, ez = 0;
+  const long long eidx = (long long)blockIdx.x * blockDim.y + el;
+  const bool valid = plain_elem(g, eidx, ex, ey, ez);
+  const int I = ex * g.p + u, Jn = ey * g.p + v;
+  const bool inIJ = valid && I >= 1 && I <= g.nix && Jn >= 1 && Jn <= g.niy;
+  const double sxy = inIJ ? g.s[0][I] * g.s[1][Jn] : 0.0;
+  const long long base = inIJ ? (long long)(I - 1) + (long long)g.nix * (Jn - 1) : 0;
+  const long long plane = (long long)g.nix * g.niy;
+  const double* const sz = g.s[2] + ez * g.p;
+  const auto cB = [&](int i) { return kBs ? sB[i] : tab.c[i]; };
+  const auto kB = [&](int i) { return tab.k[i]; };
+  double acc[P1];
+#pragma unroll
+  for (int q = 0; q < P1; ++q) acc[q] = 0.0;
+  __syncthreads();
+  for (int o = 0; o < n_orb; ++o) {
+    const double2* in = psi + (long long)o * stride;
+    double2 w[P1];
+    unsigned mx = 0;
+#pragma unroll
+    for (int c = 0; c < P1; ++c) {
+      const int K = ez * g.p + c;
+      w[c] = make_double2(0.0, 0.0);
+      if (inIJ && K >= 1 && K <= g.niz) {
+        w[c] = in[base + plane * (K - 1)];
+        const double f = sxy * __ldg(sz + c);
+        w[c].x *= f;
+        w[c].y *= f;
+      }
+      mx = max(mx, max((unsigned)__double2hiint(w[c].x) & 0x7fffffffu, (unsigned)__double2hiint(w[c].y) & 0x7fffffffu));
+    }
+    mx = __reduce_max_sync(grp, mx);
+    unsigned* const sm = sM + (o & 1) * Cfg<P1>::E;
+    if (lead) atomicMax(&sm[el], mx);
+    __syncthreads();
+    int eb = (int)(sm[el] >> 20);
+    if (threadIdx.x == 0) sM[((o & 1) ^ 1) * Cfg<P1>::E + el] = 0;   // last read before the previous orbital's stages
+    const bool poison = eb == 2047;
+    eb = eb < 64 ? 64 : (eb > 2046 ? 2046 : eb);
+    const int ec = min(3 - kFxBits + eb - 1022, 900);   // (the squares overflow well below the limit)
+    const double f = poison ? __hiloint2double(0x7ff80000, 0) : occ[o];
+#pragma unroll 1
+    for (int comp = 0; comp < 2; ++comp) {
+      long long col[P1], t[P1];
+      float cf[P1], tf[P1];
+#pragma unroll
+      for (int c = 0; c < P1; ++c) {
+        const double x = comp ? w[c].y : w[c].x;
+        col[c] = fx_from_bits((unsigned)__double2hiint(x), (unsigned)__double2loint(x), eb);
+        cf[c] = 0.0f;
+      }
+      fx_apply<P1>(cB, kB, col, cf, [&](int q, long long x, float xf) {
+        S1[q * PS + v * LS + u] = x;
+        F1[q * PF + v * LF + u] = xf;
+      });
+      __syncthreads();
+      load_line(col, S1 + v * PS + u, LS);
+      load_line(cf, F1 + v * PF + u, LF);
+      fx_apply<P1>(cB, kB, col, cf, [&](int q, long long x, float xf) {
+        S2[v * PS + q * LS + u] = x;
+        F2[v * PF + q * LF + u] = xf;
+      });
+      __syncthreads();
+      load_line(col, S2 + v * PS + u * LS, 1);
+      load_line(cf, F2 + v * PF + u * LF, 1);
+      fx_apply<P1>(cB, kB, col, cf, [&](int q, long long x, float xf) {
+        t[q] = x;
+        tf[q] = xf;
+      });
+      const int es = (ec - fx_join<P1>(t, tf)) << 20;
+#pragma unroll
+      for (int q = 0; q < P1; ++q) {
+        const double x = fx_to_double(t[q], es);
+        acc[q] = fma(f * x, x, acc[q]);
+      }
+    }
+  }
+  if (valid) {
+    const double wuv = tab.iw[u] * tab.iw[v];
+#pragma unroll
+    for (int q = 0; q < P1; ++q) rho[eidx * P3 + v * P2 + u * P1 + q] = acc[q] * (wuv * tab.iw[q]);
+  }
+}
+
 template <int P1>
 FxTab<P1> make_tab(const FxHost& h) {
   FxTab<P1> t;
@@ -492,6 +610,7 @@ FxTab<P1> make_tab(const FxHost& h) {
     for (int i = 0; i < KS; ++i) t.k[m * KS + i] = fx_tail_const<P1>([&](int j) { return t.c[m * CS + j]; }, i);
   t.dK = h.dK;
   t.kinf = h.kinf;
+  for (int q = 0; q < P1; ++q) t.iw[q] = 1.0 / h.w[q];
   return t;
 }
 
@@ -503,6 +622,20 @@ cudaError_t elem_t(const Geom& g, const FxHost& h, const double* vks, const Appl
   if (e != cudaSuccess) return e;
   k_hbar_fx<P1><<<dim3(bpe, (a.n_orb + opc - 1) / opc), dim3(P1 * P1, E), smem, st>>>(g, make_tab<P1>(h), vks, a, opc,
                                                                                      ev);
+  return cudaGetLastError();
+}
+
+template <int P1>
+cudaError_t density_t(const Geom& g, const FxHost& h, const double2* psi, int64_t stride, int n_orb, const double* occ,
+                      double* rho, cudaStream_t st) {
+  const long long ne = (long long)g.nx * g.ny * g.nz;
+  int E = Cfg<P1>::E;
+  while (E > 1 && (ne + E - 1) / E < 2 * 152) E = (E + 1) / 2;   // small meshes: spread over the SMs
+  const size_t smem = (size_t)E * (SplitLayout<P1, double>::ES * sizeof(long long) + SplitLayout<P1, float>::ES * sizeof(float));
+  cudaError_t e = cudaFuncSetAttribute(k_density_fx<P1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  k_density_fx<P1><<<(unsigned)((ne + E - 1) / E), dim3(P1 * P1, E), smem, st>>>(g, make_tab<P1>(h), psi, stride, n_orb,
+                                                                                occ, rho);
   return cudaGetLastError();
 }
 
@@ -547,6 +680,21 @@ cudaError_t launch_hbar_batch_fx(int P1, const FxHost* h, const BSys* sys, const
     case 7: return batch_t<7>(h, sys, items, n_items, E, grid, qctr, st, occ);
     case 8: return batch_t<8>(h, sys, items, n_items, E, grid, qctr, st, occ);
     case 9: return batch_t<9>(h, sys, items, n_items, E, grid, qctr, st, occ);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+cudaError_t launch_density_fx(int P1, const Geom& g, const FxHost& h, const double2* psi, int64_t stride, int n_orb,
+                              const double* occ, double* rho, cudaStream_t st) {
+  switch (P1) {
+    case 2: return density_t<2>(g, h, psi, stride, n_orb, occ, rho, st);
+    case 3: return density_t<3>(g, h, psi, stride, n_orb, occ, rho, st);
+    case 4: return density_t<4>(g, h, psi, stride, n_orb, occ, rho, st);
+    case 5: return density_t<5>(g, h, psi, stride, n_orb, occ, rho, st);
+    case 6: return density_t<6>(g, h, psi, stride, n_orb, occ, rho, st);
+    case 7: return density_t<7>(g, h, psi, stride, n_orb, occ, rho, st);
+    case 8: return density_t<8>(g, h, psi, stride, n_orb, occ, rho, st);
+    case 9: return density_t<9>(g, h, psi, stride, n_orb, occ, rho, st);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -76,6 +76,7 @@ struct FxHost {
   const long long* c = nullptr; // folded B' = W^1/2 B, then B'^T (2 * cs_size entries)
   const double* dK = nullptr;   // device: folded K' = W^-1/2 Kq W^-1/2 (cs_size doubles)
   double kinf = 0.0;            // largest row sum of |K'|
+  const double* w = nullptr;    // Gauss weights
 };
 }  // namespace tdks
 
@@ -104,6 +105,7 @@ struct tdks_ctx {
   float* d_tabf = nullptr;     // float copy
   float* d_tabdf = nullptr;    // double-float copy (hi, lo pairs)
   float* d_tabbf = nullptr;    // float copy rounded to bfloat16 (BF16-operand mode)
+  std::vector<double> fx_w;
   std::vector<long long> fx_c; // fixed-point tables (FxHost::c)
   double* d_fxK = nullptr;     // and the folded K'
   double* d_occ = nullptr;
@@ -243,6 +245,8 @@ tdks_status launch_hbar_apply(tdks_ctx* c, const ApplyArgs& a, int prec);
 // CTA (bpe CTAs) and opc orbitals per CTA; results and alpha as described there
 cudaError_t launch_hbar_fx(int P1, const Geom& g, const tdks::FxHost& h, const double* vks, const ApplyArgs& a,
                            int E, int bpe, int opc, double2* ev, cudaStream_t st);
+cudaError_t launch_density_fx(int P1, const Geom& g, const tdks::FxHost& h, const double2* psi, int64_t stride,
+                              int n_orb, const double* occ, double* rho, cudaStream_t st);
 // element results of K in (c->d_sev), per-CTA partials of in . K in (stiff_blocks of them)
 tdks_status launch_stiffness(tdks_ctx* c, const double* in, double* part, const CgState* cg);
 // gather of the element results in c->d_sev with fused CG vector work (modes in elements.cu)

@@ -93,3 +93,25 @@ def test_non_finite_values_stay_in_their_elements(p, bad):
     hit[:, p - 1:, p - 1:, 3 * p - 1:] = True
     assert np.isnan(out[hit]).all() and np.array_equal(out[~hit], clean[~hit])
     ctx.close()
+
+
+@pytest.mark.parametrize("p,n", SHAPES)
+def test_density(p, n):
+    """The FP64 density (Eq. 2): three contractions, squares summed over the orbitals."""
+    ctx, m, v, psi = _setup(p, n, 3)
+    ref = ham.density(m, psi, [2.0] * 3).ravel()
+    rho = ctx.density(torch.from_numpy(psi).cuda()).cpu().numpy().ravel()
+    # the oracle rounds three FP64 contractions of p + 1 terms: within 1e-13 of the largest value
+    assert np.abs(rho - ref).max() <= 1e-13 * ref.max()
+    for k in (-400, 300):
+        out = ctx.density(torch.from_numpy(psi * 2.0 ** k).cuda()).cpu().numpy().ravel()
+        assert np.array_equal(out, rho * 4.0 ** k), k
+    # a non-finite entry loses its element's density and no other
+    x = psi.copy()
+    x[1, 0] = np.nan
+    out = ctx.density(torch.from_numpy(x).cuda()).cpu().numpy().ravel()
+    nq = m.nq ** 3
+    own = 1 if p > 1 else 8     # (p = 1: the first interior node belongs to eight elements)
+    assert np.isnan(out[:nq]).all() and np.isnan(out).sum() == own * nq
+    assert np.array_equal(out[8 * nq:], rho[8 * nq:]) if p == 1 else np.array_equal(out[nq:], rho[nq:])
+    ctx.close()
