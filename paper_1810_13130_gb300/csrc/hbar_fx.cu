@@ -104,7 +104,9 @@ __device__ __forceinline__ int fx_join(long long (&t)[P1], const float (&tf)[P1]
 // Elements [eidx] of the calling rows for the orbitals o_begin <= o < o_end that orb(o, in, sc)
 // accepts; element results (of V_j, not q_j) to ev, orbital stride ev_ostride entries,
 // alpha partials (times sc^2) to part.  sV, sM[2]: zero and synchronized on entry.
-template <int P1, class OrbFn>
+// kPair: rows 2 e and 2 e + 1 of the block share element e, one takes the real parts, the
+// other the imaginary parts (each with its own lines and tables); the results are the same.
+template <int P1, bool kPair, class OrbFn>
 __device__ __forceinline__ void hbar_elem_fx(const Geom& g, const FxTab<P1>& tab, FxC* sK, float* sKk, long long* S1,
                                              float* F1,
                                              int* sA, int* sE, unsigned* sV, unsigned* sM, int sM_stride,
@@ -234,7 +236,7 @@ __device__ __forceinline__ void hbar_elem_fx(const Geom& g, const FxTab<P1>& tab
     const int ec = eo < -980 ? -980 : (eo > 900 ? 900 : eo);
     double2* evo = ev + (long long)o * ev_ostride + eidx * P3 + v * P2 + u * P1;
 #pragma unroll 1
-    for (int comp = 0; comp < 2; ++comp) {   // real part, then imaginary part
+    for (int comp = kPair ? el & 1 : 0; comp < 2; comp += kPair ? 2 : 1) {   // real part, then imaginary part
       long long col[P1], t[P1];
       float cf[P1], tf[P1];
 #pragma unroll
@@ -243,7 +245,7 @@ __device__ __forceinline__ void hbar_elem_fx(const Geom& g, const FxTab<P1>& tab
         col[c] = fx_from_bits(w.y, w.x, eb);
         cf[c] = 0.0f;
       }
-      if (comp == 1) {   // the thread's slots are free: the next active orbital's column
+      if (kPair || comp == 1) {   // the thread's slots are free: the next active orbital's column
         const double2* in_n = nullptr;
         on = o + 1;
         while (on < o_end && !orb(on, in_n, sc_n)) ++on;
@@ -362,14 +364,23 @@ __device__ __forceinline__ void hbar_elem_fx(const Geom& g, const FxTab<P1>& tab
     // written, and at least three before the next orbital adds to them
     if (part && tid < 32) {
       double s = 0.0;
-      for (int e = tid; e < (int)blockDim.y; e += 32) {
-        int* A = sA + kAcc * e;
+      const int ne = (int)blockDim.y >> (kPair ? 1 : 0);
+      for (int e = tid; e < ne; e += 32) {
+        constexpr int rows = kPair ? 2 : 1;
+        int A[kAcc];
+#pragma unroll
+        for (int i = 0; i < kAcc; ++i) {
+          A[i] = sA[kAcc * rows * e + i];
+          sA[kAcc * rows * e + i] = 0;
+          if (kPair) {
+            A[i] += sA[kAcc * (rows * e + 1) + i];
+            sA[kAcc * (rows * e + 1) + i] = 0;
+          }
+        }
         const long long l = (unsigned)A[0] + ((long long)(unsigned)A[1] << 24) + ((long long)A[2] << 48);
         const long long m = (unsigned)A[3] + ((long long)(unsigned)A[4] << 24) + ((long long)A[5] << 48);
         const long long h = (unsigned)A[6] + ((long long)A[7] << 24);
-#pragma unroll
-        for (int i = 0; i < kAcc; ++i) A[i] = 0;
-        const int x = sE[e];
+        const int x = sE[rows * e];
         const double d = fma((double)h, 0x1p64, fma((double)m, 0x1p32, (double)l * 0x1p10));
         s += x == 1 << 30 ? __hiloint2double(0x7ff80000, 0) : d * pow2(x / 2) * pow2(x - x / 2);
       }
@@ -386,7 +397,7 @@ __device__ __forceinline__ void hbar_elem_fx(const Geom& g, const FxTab<P1>& tab
   }
 }
 
-template <int P1>
+template <int P1, bool kPair>
 __global__ void __launch_bounds__(256, 2) k_hbar_fx(Geom g, const __grid_constant__ FxTab<P1> tab,
                                                     const double* __restrict__ vks, ApplyArgs a, int orb_per_cta,
                                                     double2* __restrict__ ev) {
@@ -417,12 +428,15 @@ __global__ void __launch_bounds__(256, 2) k_hbar_fx(Geom g, const __grid_constan
     in = a.in_base + (long long)o * a.in_stride;
     return true;
   };
-  hbar_elem_fx<P1>(g, tab, reinterpret_cast<FxC*>(smem) + threadIdx.y * 3 * CS,
-                   reinterpret_cast<float*>(smem + FxSmem<P1>::kc(blockDim.y)) + threadIdx.y * 3 * FxTab<P1>::KS,
-                   reinterpret_cast<long long*>(smem + FxSmem<P1>::lines(blockDim.y)) + (size_t)threadIdx.y * ES,
-                   reinterpret_cast<float*>(smem + FxSmem<P1>::tails(blockDim.y)) + (size_t)threadIdx.y * SplitLayout<P1, float>::ES, sA, sE, sV, sM, Cfg<P1>::E, vks, (long long)blockIdx.x * blockDim.y + threadIdx.y, o0, o1, orb, ev,
-                   (long long)g.nx * g.ny * g.nz * P3, a.part, a.part_stride, blockIdx.x,
-                   reinterpret_cast<double2*>(smem + FxSmem<P1>::pf(blockDim.y)));
+  hbar_elem_fx<P1, kPair>(g, tab, reinterpret_cast<FxC*>(smem) + threadIdx.y * 3 * CS,
+                          reinterpret_cast<float*>(smem + FxSmem<P1>::kc(blockDim.y)) + threadIdx.y * 3 * FxTab<P1>::KS,
+                          reinterpret_cast<long long*>(smem + FxSmem<P1>::lines(blockDim.y)) + (size_t)threadIdx.y * ES,
+                          reinterpret_cast<float*>(smem + FxSmem<P1>::tails(blockDim.y)) +
+                              (size_t)threadIdx.y * SplitLayout<P1, float>::ES,
+                          sA, sE, sV, sM, Cfg<P1>::E, vks,
+                          ((long long)blockIdx.x * blockDim.y + threadIdx.y) >> (kPair ? 1 : 0), o0, o1, orb, ev,
+                          (long long)g.nx * g.ny * g.nz * P3, a.part, a.part_stride, blockIdx.x,
+                          reinterpret_cast<double2*>(smem + FxSmem<P1>::pf(blockDim.y)));
 }
 
 // Batched form: a persistent grid draws the work items of one degree class from a ticket
@@ -480,12 +494,14 @@ __global__ void __launch_bounds__(256, 2) k_hbar_batch_fx(const BSys* __restrict
       }
       if (!any) continue;
     }
-    hbar_elem_fx<P1>(g, tab, reinterpret_cast<FxC*>(smem) + threadIdx.y * 3 * CS,
-                   reinterpret_cast<float*>(smem + FxSmem<P1>::kc(blockDim.y)) + threadIdx.y * 3 * FxTab<P1>::KS,
-                     reinterpret_cast<long long*>(smem + FxSmem<P1>::lines(blockDim.y)) + (size_t)threadIdx.y * ES,
-                     reinterpret_cast<float*>(smem + FxSmem<P1>::tails(blockDim.y)) + (size_t)threadIdx.y * SplitLayout<P1, float>::ES, sA, sE, sV, sM, Cfg<P1>::E, S.vks, (long long)w.eblk * blockDim.y + threadIdx.y, w.o0, w.o1, orb,
-                     static_cast<double2*>(S.ev), S.n_elem * P3, S.apart, S.n_eblk, w.eblk,
-                     reinterpret_cast<double2*>(smem + FxSmem<P1>::pf(blockDim.y)));
+    hbar_elem_fx<P1, false>(
+        g, tab, reinterpret_cast<FxC*>(smem) + threadIdx.y * 3 * CS,
+        reinterpret_cast<float*>(smem + FxSmem<P1>::kc(blockDim.y)) + threadIdx.y * 3 * FxTab<P1>::KS,
+        reinterpret_cast<long long*>(smem + FxSmem<P1>::lines(blockDim.y)) + (size_t)threadIdx.y * ES,
+        reinterpret_cast<float*>(smem + FxSmem<P1>::tails(blockDim.y)) + (size_t)threadIdx.y * SplitLayout<P1, float>::ES,
+        sA, sE, sV, sM, Cfg<P1>::E, S.vks, (long long)w.eblk * blockDim.y + threadIdx.y, w.o0, w.o1, orb,
+        static_cast<double2*>(S.ev), S.n_elem * P3, S.apart, S.n_eblk, w.eblk,
+        reinterpret_cast<double2*>(smem + FxSmem<P1>::pf(blockDim.y)));
   }
 }
 
@@ -617,12 +633,20 @@ FxTab<P1> make_tab(const FxHost& h) {
 template <int P1>
 cudaError_t elem_t(const Geom& g, const FxHost& h, const double* vks, const ApplyArgs& a, int E, int bpe, int opc,
                    double2* ev, cudaStream_t st) {
-  const size_t smem = FxSmem<P1>::bytes(E);
-  cudaError_t e = cudaFuncSetAttribute(k_hbar_fx<P1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  k_hbar_fx<P1><<<dim3(bpe, (a.n_orb + opc - 1) / opc), dim3(P1 * P1, E), smem, st>>>(g, make_tab<P1>(h), vks, a, opc,
-                                                                                     ev);
-  return cudaGetLastError();
+  const dim3 grid(bpe, (a.n_orb + opc - 1) / opc);
+  const long long warps = (long long)bpe * grid.y * ((P1 * P1 * E + 31) / 32);
+  // With less than four warps per SM one CTA's chain of stages is the launch's time: the real
+  // and the imaginary parts side by side (p = 4, 6^3 elements, one orbital: 15.3 -> 11.7 us).
+  // With more, both parts in turn share the set-up and the gather.
+  const bool pair = 2 * E <= Cfg<P1>::E && warps < 4 * 152;
+  const auto launch = [&](auto kern, int rows) {
+    const size_t smem = FxSmem<P1>::bytes(rows);
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    kern<<<grid, dim3(P1 * P1, rows), smem, st>>>(g, make_tab<P1>(h), vks, a, opc, ev);
+    return cudaGetLastError();
+  };
+  return pair ? launch(k_hbar_fx<P1, true>, 2 * E) : launch(k_hbar_fx<P1, false>, E);
 }
 
 template <int P1>
