@@ -69,20 +69,6 @@ struct FxSmem {
 constexpr int kAcc = 8;   // integer accumulators of an element's u . r (24-bit limbs)
 
 __device__ __forceinline__ int exp_field(double x) { return (int)(((unsigned)__double2hiint(x) >> 20) & 0x7ffu); }
-__device__ __forceinline__ double pow2(int e) {   // 2^e, e clamped to the normal range
-  e = e < -1022 ? -1022 : (e > 1023 ? 1023 : e);
-  return __hiloint2double((e + 1023) << 20, 0);
-}
-
-// V 2^e -> double, correctly rounded, |V| < 2^62, e in [-1074, 939], eb = e << 20 (two
-// additions, the first exact)
-__device__ __forceinline__ double fx_to_double(long long v, int eb) {
-  const unsigned hi = (unsigned)((unsigned long long)v >> 32) ^ 0x80000000u;
-  const double dh = __hiloint2double(0x45300000 + eb, (int)hi);            // 2^e (2^84 + (vh + 2^31) 2^32)
-  const double dl = __hiloint2double(0x43300000 + eb, (int)(unsigned)v);   // 2^e (2^52 + vl)
-  const double cc = __hiloint2double(0x45300000 + eb, (int)0x80100000u);   // 2^e (2^84 + 2^63 + 2^52)
-  return (dh - cc) + dl;
-}
 
 // Integer and tail of a line as 62-bit integers: shifted left by the line's free bits (at
 // most 19; |f| < 8; returned), the tail rounded to the new unit by adding 1.5 2^(23 - s)

@@ -8,8 +8,8 @@
 //     mesh is separable (see fdm.cpp), so K^-1 = S D^-1 S^T with S = Sx (x) Sy (x) Sz,
 //     applied as six strided matrix products along the three axes and a diagonal
 //     scaling; for these meshes it is the exact inverse up to rounding and CG stops
-//     after one or two iterations.  The products are FP64, or double-float for the
-//     double-float runs (a preconditioner exact to ~1e-14; the CG stays FP64);
+//     after one or two iterations.  The products are fixed point (FP64 on axes of more
+//     than 255 nodes), or double-float for the double-float runs (a preconditioner exact to ~1e-14; the CG stays FP64);
 //   * Jacobi (diagonal of K from 1-D sums).
 // Convergence is decided on the device: once converged every later kernel of the
 // iteration returns at once, and the host polls the flag after iterations
@@ -18,9 +18,10 @@
 #include <vector>
 
 #include "df64.cuh"
+#include "fixed.cuh"
 #include "tdks_internal.h"
 
-using tdks::Df;
+using namespace tdks;
 
 namespace {
 
@@ -234,6 +235,121 @@ __global__ void __launch_bounds__(256) k_gemm(Gemm g, const CgState* cg) {
   }
 }
 
+// The same product in fixed point (fixed.cuh): every row of A and every column of B has the
+// exponent of its largest entry (one pass over the panels first; the second read is a cache
+// hit), entries are 55-bit integers, a dot product of up to kFxK terms keeps h h' and
+// h l' + l h' exactly in 64 bits and l l' in FP32, and each output is rounded once.  Three
+// wide integer multiply-adds and one FP32 one per term instead of an FP64 multiply-add, which
+// takes five times as long on the FP64 pipe.  (Double-float products take the same time.)
+constexpr int kFxK = 255;   // 2 K 2^54 < 2^63
+template <int GT>
+__global__ void __launch_bounds__(256) k_gemm_fx(Gemm g, const CgState* cg) {
+  if (cg && cg->done) return;
+  constexpr int R = GT / 16, KS = 256 / GT;
+  __shared__ int2 As[GK][GT + 1], Bs[GK][GT + 1];
+  __shared__ float Af[GK][GT + 1], Bf[GK][GT + 1];
+  __shared__ unsigned eA[GT], eB[GT];
+  const int tid = threadIdx.x;
+  const int tx = tid % 16, ty = tid / 16;
+  const long long b = blockIdx.z;
+  const int m0 = blockIdx.y * GT, n0 = blockIdx.x * GT;
+  const double* A = g.A + b * g.sAb;
+  const double* B = g.B + b * g.sBb;
+  if (tid < GT) eA[tid] = eB[tid] = 0;
+  __syncthreads();
+  {
+    const int l = tid % GT;
+    const bool inA = m0 + l < g.M, inB = n0 + l < g.N;
+    const double* pa = A + (inA ? (long long)(m0 + l) * g.sAm : 0);
+    const double* pb = B + (inB ? (long long)(n0 + l) * g.sBn : 0);
+    unsigned ma = 0, mb = 0;
+#pragma unroll 4
+    for (int k = tid / GT; k < g.K; k += KS) {
+      if (inA) ma = max(ma, (unsigned)__double2hiint(pa[k * g.sAk]) & 0x7fffffffu);
+      if (inB) mb = max(mb, (unsigned)__double2hiint(pb[k * g.sBk]) & 0x7fffffffu);
+    }
+    atomicMax(&eA[l], ma);
+    atomicMax(&eB[l], mb);
+  }
+  __syncthreads();
+  if (tid < GT) {   // exponent fields, those of zero and tiny rows raised as fx_from_bits wants them
+    eA[tid] = max(eA[tid] >> 20, 64u);
+    eB[tid] = max(eB[tid] >> 20, 64u);
+  }
+  __syncthreads();
+  long long mid[R][R], hi[R][R];
+  float f[R][R];
+#pragma unroll
+  for (int i = 0; i < R; ++i)
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+      mid[i][j] = hi[i][j] = 0;
+      f[i][j] = 0.0f;
+    }
+  const bool a_k_fast = (g.sAk == 1);
+  const bool b_n_fast = (g.sBn == 1);
+  const auto put = [](double x, int eb, int2* s, float* sf) {   // limbs, and l 2^-32
+    const FxV v = fx_operand(fx_from_bits((unsigned)__double2hiint(x), (unsigned)__double2loint(x), min(eb, 2046)) + kFxHalf, 0.0f);
+    *s = make_int2(v.h, v.l);
+    *sf = v.g - 1.5f;
+  };
+  for (int k0 = 0; k0 < g.K; k0 += GK) {
+#pragma unroll
+    for (int r = 0; r < (GT * GK) / 256; ++r) {
+      const int e = tid + 256 * r;
+      const int kk = a_k_fast ? e % GK : e / GT, mm = a_k_fast ? e / GK : e % GT;
+      const long long gm = m0 + mm, gk = k0 + kk;
+      put((gm < g.M && gk < g.K) ? A[gm * g.sAm + gk * g.sAk] : 0.0, eA[mm], &As[kk][mm], &Af[kk][mm]);
+      const int kb = b_n_fast ? e / GT : e % GK, nn = b_n_fast ? e % GT : e / GK;
+      const long long gn = n0 + nn, gk2 = k0 + kb;
+      put((gn < g.N && gk2 < g.K) ? B[gk2 * g.sBk + gn * g.sBn] : 0.0, eB[nn], &Bs[kb][nn], &Bf[kb][nn]);
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (int kk = 0; kk < GK; ++kk) {
+      int2 a[R], w[R];
+      float af[R], wf[R];
+#pragma unroll
+      for (int i = 0; i < R; ++i) {
+        a[i] = As[kk][ty * R + i];
+        af[i] = Af[kk][ty * R + i];
+        w[i] = Bs[kk][tx * R + i];
+        wf[i] = Bf[kk][tx * R + i];
+      }
+#pragma unroll
+      for (int i = 0; i < R; ++i)
+#pragma unroll
+        for (int j = 0; j < R; ++j) {
+          mid[i][j] = fx_mad(a[i].x, w[j].y, fx_mad(a[i].y, w[j].x, mid[i][j]));
+          hi[i][j] = fx_mad(a[i].x, w[j].x, hi[i][j]);
+          f[i][j] = fmaf(af[i], wf[j], f[i][j]);
+        }
+    }
+    __syncthreads();
+  }
+  double* C = g.C + b * g.sCb;
+#pragma unroll
+  for (int i = 0; i < R; ++i) {
+    const long long gm = m0 + ty * R + i;
+    if (gm >= g.M) continue;
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+      const long long gn = n0 + tx * R + j;
+      if (gn >= g.N) continue;
+      // t + (low word of mid) 2^-32 + f in units of 2^64, shifted left by the free bits
+      const long long t = hi[i][j] + (mid[i][j] >> 32);
+      const int s = min(__clzll(t ^ (t >> 63)) - 2, 20);
+      const float fr = ldexpf(f[i][j], s);
+      const long long v = (t << s) + (long long)((unsigned)mid[i][j] >> (32 - s)) + __float2int_rn(fr);
+      const int ea = eA[ty * R + i], eb = eB[tx * R + j];
+      const int e = 64 - s + (ea - 1022 - kFxBits) + (eb - 1022 - kFxBits);
+      double x = e > -1000 && e < 900 ? fx_to_double(v, e << 20) : fx_to_double(v, 0) * pow2(e / 2) * pow2(e - e / 2);
+      if (ea == 2047 || eb == 2047) x = __hiloint2double(0x7ff80000, 0);   // a non-finite row or column
+      C[gm * g.sCm + gn * g.sCn] = x;
+    }
+  }
+}
+
 // The same product in double-float arithmetic on the FP32 pipe (FP64 in and out):
 // operands split into float pairs on the integer pipe, every output an accumulator
 // (hi, err) -- hi grows by exact two-sums, the product tails and rounding errors of
@@ -349,8 +465,7 @@ int grid_for(long long n) {
 
 // Output tile of an M x N product (batch b): the least work of the busiest SM, counted in
 // outputs of whole tiles (152 SMs); the larger tile on a tie (fewer shared-memory loads).
-// 95 x 9025 (p = 6, 16^3 elements): 64 pads 95 to 128, 32 to 96: 134 -> 104 us a product;
-// 23 x 529 (p = 4, 6^3): 9 CTAs of 64 against 68 of 16: 18.5 -> 4 us.
+// 23 x 529 (p = 4, 6^3 elements) in FP64: 9 CTAs of 64 against 68 of 16: 18.5 -> 4 us.
 int gemm_tile(long long M, long long N, long long b) {
   int best = 64;
   long long cost = -1;
@@ -427,10 +542,16 @@ void axis_gemm(tdks_ctx* c, int axis, bool forward, const double* in, double* ou
     g.N = (int)(nx * ny);
     g.K = (int)nz;
   }
-  const int t = gemm_tile(g.M, g.N, batch);
+  // Fixed point wherever its accumulators allow it.  Tiles of 32 while they give every SM a
+  // CTA, then 16 (83 x 6889, p = 6, 14^3 elements: 16: 59, 32: 48, 64: 98 us, FP64 112 us;
+  // 95 x 9025: 73, 57, 100 us, FP64 141 us); longer axes keep the FP64 product.
+  const bool fx = !df && g.K <= kFxK;
+  const auto ctas = [&](int s) { return (long long)((g.M + s - 1) / s) * ((g.N + s - 1) / s) * batch; };
+  const int t = !fx ? gemm_tile(g.M, g.N, batch) : ctas(32) >= 152 ? 32 : 16;
   const dim3 grid((g.N + t - 1) / t, (g.M + t - 1) / t, (unsigned)batch);
   const auto go = [&](auto* kernel) { kernel<<<grid, 256, 0, c->stream>>>(g, cg); };
   if (df) go(t == 64 ? k_gemm_df<64> : t == 32 ? k_gemm_df<32> : k_gemm_df<16>);
+  else if (fx) go(t == 32 ? k_gemm_fx<32> : k_gemm_fx<16>);
   else go(t == 64 ? k_gemm<64> : t == 32 ? k_gemm<32> : k_gemm<16>);
 }
 
