@@ -377,7 +377,6 @@ tdks_status tdks_create(const tdks_mesh_desc* m, const tdks_system_desc* s, void
     if ((st = dalloc(c, f, (size_t)c->n_int)) != TDKS_OK) return fail(st);
     if (cudaMemset(*f, 0, c->n_int * sizeof(double)) != cudaSuccess) return fail(TDKS_ERR_CUDA);
   }
-  if ((st = dalloc(c, &c->d_sev, nf)) != TDKS_OK) return fail(st);
   if ((st = dalloc(c, &c->d_cg, 1)) != TDKS_OK) return fail(st);
   const int bpc = hbar_blocks(c);
   c->part_stride = std::max<int64_t>(2048, 8 * (int64_t)bpc);

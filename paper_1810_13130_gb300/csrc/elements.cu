@@ -1744,7 +1744,20 @@ tdks_status launch_hbar_apply(tdks_ctx* c, const ApplyArgs& a, int prec) {
   return tdks_fail(c, TDKS_ERR_ARG, "unsupported degree");
 }
 
+// The Poisson operator's element results, allocated when first needed: a context that only
+// applies Hbar does without them.
+static tdks_status ensure_sev(tdks_ctx* c) {
+  if (c->d_sev) return TDKS_OK;
+  if (cudaMalloc(&c->d_sev, (size_t)c->n_elem * c->P1 * c->P1 * c->P1 * sizeof(double)) != cudaSuccess) {
+    cudaGetLastError();
+    c->d_sev = nullptr;
+    return tdks_fail(c, TDKS_ERR_NOMEM, "Poisson element-result buffer");
+  }
+  return TDKS_OK;
+}
+
 tdks_status launch_stiffness(tdks_ctx* c, const double* in, double* part, const CgState* cg) {
+  TDKS_TRY(ensure_sev(c));
   TDKS_DISPATCH(c->P1, (stiff_t<P1>(c, in, part, cg)));
   return tdks_fail(c, TDKS_ERR_ARG, "unsupported degree");
 }
@@ -1756,6 +1769,7 @@ tdks_status launch_gather(tdks_ctx* c, const GatherArgs& a, int mode) {
 
 tdks_status launch_load_vector(tdks_ctx* c, const double* f_q, double* out, double scale,
                                int weighted) {
+  TDKS_TRY(ensure_sev(c));
   TDKS_DISPATCH(c->P1, (load_t<P1>(c, f_q, out, scale, weighted)));
   return tdks_fail(c, TDKS_ERR_ARG, "unsupported degree");
 }

@@ -116,7 +116,7 @@ struct tdks_ctx {
   double *d_vtmp = nullptr, *d_rho = nullptr, *d_vh = nullptr;
   // Poisson
   double *d_phi = nullptr, *d_b = nullptr, *d_r = nullptr, *d_pv = nullptr;
-  double* d_sev = nullptr;     // element results of the stiffness and load kernels [n_elem][P1^3]
+  double* d_sev = nullptr;     // element results of the stiffness and load kernels [n_elem][P1^3] (first use)
   CgState* d_cg = nullptr;
   double cg_tol = 1e-12;
   int cg_maxit = 5000;
