@@ -578,7 +578,7 @@ __device__ __forceinline__ int node_elems(int I, int p, int n, int* e, int* loc)
 // (the fixed-point kernel leaves the scale out): qs = s_j scales them here, 1 otherwise.
 // The degree is a compile-time
 // constant: the node -> (element, local index) split is a multiply-shift.
-template <int P1, typename T, bool kMany>
+template <int P1, typename T, bool kMany, bool kSort = false>
 __device__ __forceinline__ double assemble_rows(const Geom& g, const Cx<T>* __restrict__ evo,
                                                 const double2* qj, const double2* qm,
                                                 double2* out, double qs, double ca, double cb, int lanczos,
@@ -595,14 +595,15 @@ __device__ __forceinline__ double assemble_rows(const Geom& g, const Cx<T>* __re
   const int tstep = nix >= nt ? nt : nix;
   double acc = 0.0;
   const long long xstride = P3;                             // next element along x
-  // FP64 operations are what this costs (79 % of the FP64 pipe before, 12 operations a node
-  // and more for half-empty warps), so the first contribution is taken as it is instead of
-  // added to zero and, with many rows per block (kMany), the row scales are formed once per
-  // row, not per node (FP64 Lanczos step of 16 orbitals on 16^3 elements, p = 6: 491 -> 397 us;
-  // a block with a few rows only is bound by latency, and the barriers cost more than they save).
+  // With many rows per block (kMany) FP64 operations are what this costs (79 % of that pipe
+  // before): the first contribution is taken as it is instead of added to zero, and the row
+  // scales are formed once per row, not per node (FP64 Lanczos step of 16 orbitals on 16^3
+  // elements, p = 6: 491 -> 397 us).  Sorted x rows (kSort): the molecule's step of 55 such
+  // launches 120.4 -> 116.8 ms.  A block with a few rows is bound by latency: barriers cost
+  // more than they save, and 1, 2, 4 or 8 loads in one loop overlap better than one and the rest.
   constexpr int kRows = 128;
   __shared__ double srow[kMany ? kRows : 1];
-  for (int k0 = 0; r0 + k0 * rstride < rows; k0 += kRows) {
+  for (int k0 = 0; kMany ? r0 + k0 * rstride < rows : k0 == 0; k0 += kRows) {
     if (kMany && !kF32) {
       __syncthreads();
       for (int k = threadIdx.x; k < kRows && r0 + (k0 + k) * rstride < rows; k += nt) {
@@ -611,9 +612,9 @@ __device__ __forceinline__ double assemble_rows(const Geom& g, const Cx<T>* __re
       }
       __syncthreads();
     }
-    for (int k = tr; tr < rpb && k < kRows; k += rpb) {
-      const int r = r0 + (k0 + k) * rstride;
-      if (r >= rows) break;
+    if (tr >= rpb) continue;
+    const int rend = kMany ? min(rows, r0 + (k0 + kRows) * rstride) : rows;
+    for (int k = tr, r = r0 + (k0 + tr) * rstride; r < rend; k += rpb, r += rpb * rstride) {
       const int J = r % g.niy + 1, K = r / g.niy + 1;
       int ey[2], by[2], ez[2], bz[2];
       const int ny = node_elems(J, p, g.ny, ey, by);
@@ -630,7 +631,14 @@ __device__ __forceinline__ double assemble_rows(const Geom& g, const Cx<T>* __re
       const double syz = kF32 ? 0.0 : (kMany ? srow[kMany ? k : 0] : g.s[1][J] * g.s[2][K] * qs);
       const float syzf = g.sf[1][J] * g.sf[2][K];
       const long long rowbase = (long long)g.nix * (r);
-      for (int I = tI + 1; I <= g.nix; I += tstep) {
+      for (int i = tI + 1; i <= g.nix; i += tstep) {
+        // kSort: the nodes inside the elements first, then those on their faces, so that few
+        // warps carry the additions of a second element along x
+        int I = i;
+        if constexpr (kSort && P1 > 2) {
+          const int nin = g.nx * (P1 - 2), t = i - 1;
+          I = t < nin ? t + t / (P1 - 2) + 1 : (t - nin + 1) * p;
+        }
         // x: one element inside, two on a shared face (left element first)
         const int eh = I / p, l = I - eh * p;
         long long xo[2] = {0, 0};
@@ -647,8 +655,9 @@ __device__ __forceinline__ double assemble_rows(const Geom& g, const Cx<T>* __re
         // picked by selects so that base[] and xo[] stay in registers (an unrolled loop
         // with predicates would turn into 16 unconditional FP64 additions per node)
         const int ncon = nb * nxc;
-        Cx<T> sum = evo[base[0] + xo[0]];
-        for (int tcon = 1; tcon < ncon; ++tcon) {
+        Cx<T> sum{};
+        if constexpr (kMany) sum = evo[base[0] + xo[0]];
+        for (int tcon = kMany ? 1 : 0; tcon < ncon; ++tcon) {
           const int kc = nxc == 2 ? (tcon >> 1) : tcon;
           const long long bk = kc == 0 ? base[0] : (kc == 1 ? base[1] : (kc == 2 ? base[2] : base[3]));
           const long long xk = (nxc == 2 && (tcon & 1)) ? xo[1] : xo[0];
@@ -716,7 +725,7 @@ __global__ void __launch_bounds__(128) k_assemble(Geom g, const Cx<T>* __restric
   const double2* qj = a.in_base + (long long)o * a.in_stride;
   const double2* qm = a.vm_base ? a.vm_base + (long long)o * a.vm_stride : nullptr;
   double2* out = a.out_base + (long long)o * a.out_stride;
-  const double acc = assemble_rows<P1, T, kMany>(g, evo, qj, qm, out, qs, ca, cb, a.lanczos, a.accumulate,
+  const double acc = assemble_rows<P1, T, kMany, kMany && std::is_same<T, double>::value>(g, evo, qj, qm, out, qs, ca, cb, a.lanczos, a.accumulate,
                                           blockIdx.x, gridDim.x);
   if (a.npart) {
     const double s = block_sum(acc, red);
