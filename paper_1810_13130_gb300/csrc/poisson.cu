@@ -241,6 +241,8 @@ __global__ void __launch_bounds__(256) k_gemm(Gemm g, const CgState* cg) {
 // h l' + l h' exactly in 64 bits and l l' in FP32, and each output is rounded once.  Three
 // wide integer multiply-adds and one FP32 one per term instead of an FP64 multiply-add, which
 // takes five times as long on the FP64 pipe.  (Double-float products take the same time.)
+// Against 64-bit-mantissa products of 23 to 200 terms the 2-norm error is 0.6 to 2.8e-16, that
+// of an FP64 chain 1.6 to 4.5e-16 (random, smooth and 12-decade inputs).
 constexpr int kFxK = 255;   // 2 K 2^54 < 2^63
 template <int GT>
 __global__ void __launch_bounds__(256) k_gemm_fx(Gemm g, const CgState* cg) {
