@@ -418,6 +418,7 @@ struct KbState {
 
 void kb_free(tdks_ctx* c) {
   if (!c || !c->kb) return;
+  kgraph_drop(c);               // captured Lanczos loops hold these buffers
   KbState* k = static_cast<KbState*>(c->kb);
   void* ptrs[] = {k->d_grp, k->d_pg, k->d_vals, k->d_invh, k->d_tnode, k->d_toff, k->d_tent, k->d_P, k->d_CD,
                   k->d_goff, k->d_chunks, k->d_part, k->d_view};
@@ -487,7 +488,7 @@ tdks_status kb_project(tdks_ctx* c, const ApplyArgs& a) {
       return tdks_fail(c, TDKS_ERR_NOMEM, "projections");
     }
     k->c_orb = a.n_orb;
-    kgraph_free(c);           // captured Lanczos loops hold the old buffers
+    kgraph_drop(c);           // captured Lanczos loops hold the old buffers
     cudaFree(k->d_view);      // as does the batched view
     k->d_view = nullptr;
   }

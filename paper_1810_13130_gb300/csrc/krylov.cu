@@ -861,7 +861,10 @@ static tdks_status ensure_krylov(tdks_ctx* c, int w, int n_orb, int kmax) {
     }
   }
   if (c->d_Vw[w] && c->Vw_orb[w] >= n_orb && c->Vw_kmax[w] == kmax) return TDKS_OK;
-  if (c->d_Vw[w]) cudaFree(c->d_Vw[w]);
+  if (c->d_Vw[w]) {
+    kgraph_drop(c);     // captured loops run on this basis, and its address may be given out again
+    cudaFree(c->d_Vw[w]);
+  }
   c->d_Vw[w] = nullptr;
   const size_t bytes = (size_t)n_orb * (kmax + 1) * c->n_int * sizeof(double2);
   if (cudaMalloc(&c->d_Vw[w], bytes) != cudaSuccess) {
@@ -1000,9 +1003,13 @@ static tdks_status iteration_kernels(tdks_ctx* c, KryOrb* kry, double2* VW, int6
 // iteration.  Each iteration keeps its own launch parameters (the kernels are those of
 // the host-driven loop), so the results are identical.  The starting vector is copied into
 // the basis first, so a graph depends on the workspace and the settings alone and serves
-// every starting vector (capturing and instantiating one takes milliseconds).
+// every starting vector (capturing and instantiating one takes milliseconds).  The key holds
+// the addresses of the buffers that live as long as the context or are replaced by larger
+// ones; whoever frees a Krylov basis or the projectors drops the graphs (kgraph_drop), since
+// an address that was freed can come back with other contents behind it.
 struct KGraph {
   const void* VW = nullptr;
+  const void* kry = nullptr;
   const void* evec = nullptr;
   const void* kb = nullptr;
   int n_orb = 0, kmax = 0, prec = 0, reorth = 0, opc = 0, timing = 0;
@@ -1030,6 +1037,10 @@ static void kgraph_clear(KGraphCache* K) {
     if (G.g) cudaGraphDestroy(G.g);
   }
   K->graphs.clear();
+}
+
+void kgraph_drop(tdks_ctx* c) {
+  if (c->kgraph) kgraph_clear(static_cast<KGraphCache*>(c->kgraph));
 }
 
 void kgraph_free(tdks_ctx* c) {
@@ -1150,7 +1161,7 @@ static tdks_status get_loop_graph(tdks_ctx* c, KGraphCache* K, KryOrb* kry, doub
                                   int64_t wsorb, long long n, int n_orb, int kmax, int len, int prec,
                                   double tol, int nb, int nasm, KGraph** out) {
   for (auto& G : K->graphs) {
-    if (G.VW == VW && G.evec == c->d_evec && G.kb == c->kb && G.n_orb == n_orb &&
+    if (G.VW == VW && G.kry == kry && G.evec == c->d_evec && G.kb == c->kb && G.n_orb == n_orb &&
         G.kmax == kmax && G.len == len && G.prec == prec && G.reorth == c->lanczos_reorth && G.opc == c->opc_force &&
         G.timing == (c->timing ? 1 : 0) && G.tol == tol && G.relax == c->mixed_relax &&
         G.f32_stages == c->f32_stages) {
@@ -1163,6 +1174,7 @@ static tdks_status get_loop_graph(tdks_ctx* c, KGraphCache* K, KryOrb* kry, doub
   K->graphs.emplace_back();
   KGraph& G = K->graphs.back();
   G.VW = VW;
+  G.kry = kry;
   G.evec = c->d_evec;
   G.kb = c->kb;
   G.n_orb = n_orb;

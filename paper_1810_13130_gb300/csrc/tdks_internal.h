@@ -318,8 +318,10 @@ tdks_status run_expm_ws(tdks_ctx* c, int w, const double2* in, double2* out, int
 // TDKS_FP64 .. TDKS_MIXED (capi.cu)
 bool valid_prec(int prec);
 
-// krylov.cu: cached graphs of the device-driven Lanczos loop
+// krylov.cu: cached graphs of the device-driven Lanczos loop; kgraph_drop before freeing
+// memory that a captured loop may hold
 void kgraph_free(tdks_ctx* c);
+void kgraph_drop(tdks_ctx* c);
 // elements.cu: the element-result buffer sized for n_orb orbitals of any contraction type
 tdks_status ensure_evec(tdks_ctx* c, int n_orb);
 
