@@ -465,23 +465,6 @@ int grid_for(long long n) {
   return (int)(b < kBlocks ? (b < 1 ? 1 : b) : kBlocks);
 }
 
-// Output tile of an M x N product (batch b): the least work of the busiest SM, counted in
-// outputs of whole tiles (152 SMs); the larger tile on a tie (fewer shared-memory loads).
-// 23 x 529 (p = 4, 6^3 elements) in FP64: 9 CTAs of 64 against 68 of 16: 18.5 -> 4 us.
-int gemm_tile(long long M, long long N, long long b) {
-  int best = 64;
-  long long cost = -1;
-  for (int t : {64, 32, 16}) {
-    const long long ctas = ((M + t - 1) / t) * ((N + t - 1) / t) * b;
-    const long long c = ((ctas + 151) / 152) * t * t;
-    if (cost < 0 || c < cost) {
-      cost = c;
-      best = t;
-    }
-  }
-  return best;
-}
-
 // out = transform of `in` along `axis` with S (n_a x n_a, row-major [i][mode]):
 // forward out[.., mode, ..] = sum_i S[i][mode] in[.., i, ..]; backward uses S^T.
 void axis_gemm(tdks_ctx* c, int axis, bool forward, const double* in, double* out,

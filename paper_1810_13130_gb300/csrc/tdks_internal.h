@@ -249,6 +249,25 @@ cudaError_t launch_density_fx(int P1, const Geom& g, const tdks::FxHost& h, cons
                               int n_orb, const double* occ, double* rho, cudaStream_t st);
 // element results of K in (c->d_sev), per-CTA partials of in . K in (stiff_blocks of them)
 tdks_status launch_stiffness(tdks_ctx* c, const double* in, double* part, const CgState* cg);
+// Output tile of the Poisson preconditioner's M x N product (batch b; poisson.cu): the least
+// work of the busiest SM, counted in outputs of whole tiles (152 SMs); the larger tile on a
+// tie (fewer shared-memory loads), and only tiles whose rows fit the grid's y extent (65535;
+// two axes of 1024 nodes make 1024^2 rows).  23 x 529 (p = 4, 6^3 elements) in FP64: 9 CTAs
+// of 64 against 68 of 16: 18.5 -> 4 us.
+inline int gemm_tile(long long M, long long N, long long b) {
+  int best = 64;
+  long long cost = -1;
+  for (int t : {64, 32, 16}) {
+    if ((M + t - 1) / t > 65535) continue;
+    const long long ctas = ((M + t - 1) / t) * ((N + t - 1) / t) * b;
+    const long long c = ((ctas + 151) / 152) * t * t;
+    if (cost < 0 || c < cost) {
+      cost = c;
+      best = t;
+    }
+  }
+  return best;
+}
 // gather of the element results in c->d_sev with fused CG vector work (modes in elements.cu)
 struct GatherArgs {
   double* out;                 // mode 0: assembled vector
