@@ -61,7 +61,8 @@ typedef enum {
  * double-float as well. */
 typedef enum {
   TDKS_FP64 = 0,   /* FP64-accurate contractions (55-bit fixed point with a
-                      float tail per element: below the FP64 rounding)     */
+                      float tail per element and part: no further from the
+                      exact result than FP64 contractions)                 */
   TDKS_FP32 = 1,   /* float contractions with float accumulation, FP64 I/O  */
   TDKS_DF64 = 2,   /* double-float (compensated float-pair) contractions:
                       ~48-bit accurate products and sums on the FP32 pipe   */

@@ -354,8 +354,10 @@ tdks_status tdks_create(const tdks_mesh_desc* m, const tdks_system_desc* s, void
       fold_centrosymmetric(m->data(), P1, f.data());
       for (long double x : f) c->fx_c.push_back(llrintl(ldexpl(x, 63)));
     }
-    std::vector<double> fk(cs_size(P1));
-    fold_centrosymmetric(t.Kw.data(), P1, fk.data());
+    fold_centrosymmetric(t.Kw.data(), P1, f.data());
+    std::vector<double> fk;
+    for (long double x : f) fk.push_back((double)x);
+    for (long double x : f) fk.push_back((double)(x - (double)x));
     if ((st = upload(c, &c->d_fxK, fk)) != TDKS_OK) return fail(st);
     c->fx.c = c->fx_c.data();
     c->fx.dK = c->d_fxK;

@@ -3,7 +3,8 @@
 // GB300 runs 2 FP64 operations per clock and SM; its integer pipe multiplies 32 x 32 bits
 // into 64 sixteen times as fast, its FP32 pipe is 64 times as fast.  So a contraction is
 // carried out in 55-bit integers with an FP32 tail below them: faster than the FP64 pipe
-// and more accurate.  All values of one element and orbital share a power of two:
+// and at least as accurate.  All values of an element's part (real or imaginary) of one
+// orbital share a power of two:
 //   value x = (V + f) 2^E,    V a 64-bit integer, |V| < 2^55, f a float of a few units;
 //   coefficient c = C 2^-63,  C = h 2^32 + l, |c| < 1, l signed.
 // With V = vh 2^32 + vl (vl signed; taken from V + 2^31, whose high word is vh)
@@ -12,11 +13,15 @@
 // 1), which keeps h in 32 bits.  A dot product sums h vh and mid = sum (h vl + l vh)
 // exactly in 64 bits (three wide multiply-adds per term); the integer part is
 // sum h vh + (mid >> 32), rounded to nearest.  What is left goes to the tail in FP32: the
-// fraction of mid 2^-32, sum (c / 2) f and the low products, each to about 2^-21 of a
-// unit, so a result is good to some 2^-75 of the element's largest value.  Measured on the
-// CPU against 80-bit arithmetic the whole element operator is off by 4.7e-17 .. 9.7e-17
-// relative in the 2-norm (p = 2..8, smooth and random vectors: little more than the
-// rounding of the result), the FP64 contractions by 2.4e-16 .. 1.2e-15.
+// fraction of mid 2^-32, sum (c / 2) f and the low products, each to about 2^-23 of a unit.
+// What a stage loses is fixed in units, so the values have to fill their 55 bits: a vector
+// with one large entry loses three bits per contraction (the element operator was off by up
+// to 4e-15 at p = 8), and is raised once on the way (fx_raise).  Relative error of the whole
+// element operator in the 2-norm, p = 1..8, against extended precision, over dense vectors,
+// ones that fall off by up to 69 e-folds along the element and ones with a single large
+// entry, with mild and with steep potentials: 2.3e-17 .. 1.6e-16 (little more than the rounding
+// of the result), FP64 contractions 6.8e-17 .. 7.7e-15, and for every vector at most 0.75
+// times theirs.
 //
 // Range: with row sums sum |c| = R, |sum h vl| <= R 2^62 and |sum l vh| <= 5 2^31 2^(56 - 32)
 // R^2, so |mid| < 2^63 for R <= 1.54, the largest row sum (the transposed interpolation of
@@ -24,6 +29,8 @@
 #pragma once
 
 #include <cuda_runtime.h>
+
+#include <cmath>
 
 namespace tdks {
 
@@ -51,6 +58,15 @@ __host__ __device__ __forceinline__ float fx_bits_float(unsigned b) {
   float f;
   __builtin_memcpy(&f, &b, 4);
   return f;
+#endif
+}
+__host__ __device__ __forceinline__ unsigned fx_float_bits(float f) {
+#ifdef __CUDA_ARCH__
+  return __float_as_uint(f);
+#else
+  unsigned b;
+  __builtin_memcpy(&b, &f, 4);
+  return b;
 #endif
 }
 // 1 + w 2^-32, cut to 23 bits
@@ -167,16 +183,54 @@ __host__ __device__ __forceinline__ float fx_tail_const(CF c, int i) {
   return -1.5f - 1.5f * s;
 }
 
-// y -> V at the block exponent eb (biased exponent of the block's largest |y|, in
-// [64, 2046]): |V| < 2^kFxBits.  Bits below one unit are cut off (sign-magnitude); subnormal
-// y give 0.
-__host__ __device__ __forceinline__ long long fx_from_bits(unsigned hw, unsigned lw, int eb) {
+// y -> V and its tail at the block exponent eb (biased exponent of the block's largest |y|,
+// in [64, 2046]): |V| < 2^kFxBits, cut towards zero; the bits below one unit, to 2^-32 of it,
+// go to the tail.  An entry 2^-k of the largest has only 55 - k bits in V: without the tail
+// the element operator was off by up to 1e-13 on vectors that fall off steeply inside an
+// element, by 2e-16 .. 7e-15 with FP64 contractions.  Subnormal y give 0.
+__host__ __device__ __forceinline__ long long fx_from_bits(unsigned hw, unsigned lw, int eb, float& f) {
   const int e = (int)((hw >> 20) & 0x7ffu);
-  unsigned long long m = ((unsigned long long)((hw & 0xfffffu) | 0x100000u) << 32) | lw;
+  const unsigned long long m = (((unsigned long long)((hw & 0xfffffu) | 0x100000u) << 32) | lw) << (kFxBits - 53);
   int d = eb - e;
-  d = (e == 0 || d > 63) ? 63 : d;
-  m = (m << (kFxBits - 53)) >> d;
-  return (hw & 0x80000000u) ? -(long long)m : (long long)m;
+  d = (e == 0 || d > 95) ? 95 : d;
+  const unsigned long long v = d < 64 ? m >> d : 0;
+  const unsigned w = d == 0 ? 0u : d < 64 ? (unsigned)((m << (64 - d)) >> 32) : (unsigned)(m >> 32) >> (d - 64);
+  const float t = (float)w * 0x1p-32f;
+  const bool neg = (hw & 0x80000000u) != 0;
+  f = neg ? -t : t;
+  return neg ? -(long long)v : (long long)v;
+}
+
+// The values of a block raised to use the bits that the contractions so far have left free:
+// the shift for big, the OR of fx_magnitude of all of them (at most 18, 0 for a block of
+// zeros; raised values stay below 2^54 + 2^23), and the raise of one value, |f| < 8.
+__host__ __device__ __forceinline__ unsigned fx_magnitude(long long v) {
+  const int h = (int)(v >> 32);
+  return (unsigned)(h ^ (h >> 31)) | (unsigned)((unsigned)v != 0u);
+}
+__host__ __device__ __forceinline__ int fx_free_bits(unsigned big) {
+#ifdef __CUDA_ARCH__
+  const int z = __clz((int)big);
+#else
+  const int z = big ? __builtin_clz(big) : 32;
+#endif
+  return z == 32 ? 0 : (z - 10 < 18 ? z - 10 : 18);
+}
+__host__ __device__ __forceinline__ void fx_raise(long long& v, float& f, int s) {
+  const float g = f * fx_bits_float((unsigned)(127 + s) << 23);
+  const float m = g + 12582912.0f;                   // 1.5 2^23 + nearest integer, |g| < 2^21
+  v = (long long)((unsigned long long)v << s) + ((int)fx_float_bits(m) - 0x4b400000);
+  f = g - (m - 12582912.0f);
+}
+
+// c (hi + lo) scale to the nearest integer, scale a power of two
+__host__ __device__ __forceinline__ long long fx_scaled(double c, double hi, double lo, double scale) {
+  const double q = c * hi, r = fma(c, hi, -q) + c * lo;
+#ifdef __CUDA_ARCH__
+  return __double2ll_rn(q * scale) + __double2ll_rn(r * scale);
+#else
+  return llrint(q * scale) + llrint(r * scale);
+#endif
 }
 
 #ifdef __CUDACC__

@@ -17,8 +17,9 @@
 //
 // Layout: one P1 x P1 thread plane per element, real lines, the real and the imaginary
 // part one after the other, the next orbital's columns copied to shared memory meanwhile.
-// The largest value of an element and orbital (both parts) sets its exponent: one integer
-// maximum over the element's threads.  Measured per application of 16 orbitals on 16^3
+// The largest value of an element's part (real or imaginary) sets its exponent: one integer
+// maximum over the element's threads.  (With one exponent for both, the imaginary part of an
+// orbital after a weak kick kept only the bits that the real part left.)  Measured per application of 16 orbitals on 16^3
 // elements, p = 6: 4.62 ms with FP64 contractions (95 % of the FP64 pipe), 1.36 ms here
 // (7800 instructions per warp and orbital at 50 % issue activity, wide multiply-adds 44 % of
 // their pipe, two CTAs of 128 registers per SM); 5 orbitals on 20^3, p = 8: 7.1 -> 2.0 ms.
@@ -39,7 +40,7 @@ struct FxTab {
   static constexpr int CS = FxOp<P1>::CS, KS = FxOp<P1>::KS;
   FxC c[2 * CS];        // folded B', then B'^T
   float k[2 * KS];      // their tail constants
-  const double* dK;     // folded K' (device)
+  const double* dK;     // folded K' (device): leading parts, then the rest
   double kinf;          // largest row sum of |K'|
   double iw[P1];        // 1 / Gauss weight
 };
@@ -66,7 +67,7 @@ struct FxSmem {
   static size_t bytes(int E) { return vx(E) + (kFxVs<P1> ? (size_t)E * P2 * P1 * sizeof(FxL) : 0); }
 };
 
-constexpr int kAcc = 8;   // integer accumulators of an element's u . r (24-bit limbs)
+constexpr int kAcc = 8;   // integer accumulators of u . r of an element's part (24-bit limbs)
 
 __device__ __forceinline__ int exp_field(double x) { return (int)(((unsigned)__double2hiint(x) >> 20) & 0x7ffu); }
 
@@ -89,13 +90,14 @@ __device__ __forceinline__ int fx_join(long long (&t)[P1], const float (&tf)[P1]
 
 // Elements [eidx] of the calling rows for the orbitals o_begin <= o < o_end that orb(o, in, sc)
 // accepts; element results (of V_j, not q_j) to ev, orbital stride ev_ostride entries,
-// alpha partials (times sc^2) to part.  sV, sM[2]: zero and synchronized on entry.
+// alpha partials (times sc^2) to part.  sV, sM[4], sR[2] and sA (a set per element and
+// part) are zero and synchronized on entry.
 // kPair: rows 2 e and 2 e + 1 of the block share element e, one takes the real parts, the
 // other the imaginary parts (each with its own lines and tables); the results are the same.
 template <int P1, bool kPair, class OrbFn>
 __device__ __forceinline__ void hbar_elem_fx(const Geom& g, const FxTab<P1>& tab, FxC* sK, float* sKk, long long* S1,
                                              float* F1,
-                                             int* sA, int* sE, unsigned* sV, unsigned* sM, int sM_stride,
+                                             int* sA, int* sE, unsigned* sV, unsigned* sM, unsigned* sR, int sm_stride,
                                              const double* __restrict__ vks, long long eidx, int o_begin, int o_end,
                                              OrbFn orb, double2* __restrict__ ev, long long ev_ostride, double* part,
                                              int64_t part_stride, long long pslot, double2* __restrict__ pfbuf) {
@@ -146,7 +148,7 @@ __device__ __forceinline__ void hbar_elem_fx(const Geom& g, const FxTab<P1>& tab
       er = max(exp_field(bound) - 1022, -900);
       scale = pow2(63 - er);
       for (int i = threadIdx.x; i < 3 * CS; i += P2)
-        sK[i] = fx_coef(__double2ll_rn((i < CS ? cd[0] : (i < 2 * CS ? cd[1] : cd[2])) * tab.dK[i % CS] * scale));
+        sK[i] = fx_coef(fx_scaled(i < CS ? cd[0] : (i < 2 * CS ? cd[1] : cd[2]), tab.dK[i % CS], tab.dK[CS + i % CS], scale));
     }
     __syncthreads();
     for (int i = threadIdx.x; i < 3 * KS; i += P2)
@@ -183,7 +185,7 @@ __device__ __forceinline__ void hbar_elem_fx(const Geom& g, const FxTab<P1>& tab
     for (int i = tid; i < 2 * CS; i += nthr) sB[i] = tab.c[i];
     __syncthreads();
   }
-  int o = o_begin, it = 0;
+  int o = o_begin, it = 0, rb = 0;
   double sc = 1.0;
   {
     const double2* in0 = nullptr;
@@ -198,38 +200,49 @@ __device__ __forceinline__ void hbar_elem_fx(const Geom& g, const FxTab<P1>& tab
     int on = o_end;
     double sc_n = 1.0;
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-    // scaled column, back into the thread's own buffer slots; block maximum
-    unsigned mx = 0;
+    // scaled column, back into the thread's own buffer slots; maxima of the parts
+    unsigned mx[2] = {0, 0};
 #pragma unroll
     for (int c = 0; c < P1; ++c) {
       double2 w = pfbuf[c * nthr + tid];
       const double f = sxy * __ldg(sz + c);   // (the buffer holds 0 outside the interior)
       w.x *= f;
       w.y *= f;
-      mx = max(mx, max((unsigned)__double2hiint(w.x) & 0x7fffffffu, (unsigned)__double2hiint(w.y) & 0x7fffffffu));
+      mx[0] = max(mx[0], (unsigned)__double2hiint(w.x) & 0x7fffffffu);
+      mx[1] = max(mx[1], (unsigned)__double2hiint(w.y) & 0x7fffffffu);
       pfbuf[c * nthr + tid] = w;
     }
-    mx = __reduce_max_sync(grp, mx);
-    if (lead) atomicMax(&sM[(it & 1) * sM_stride + el], mx);
+    // sM[2 (orbital parity) + part]: zeroed one orbital ahead, after the barrier that follows
+    // the last read
+    unsigned* const sm = sM + 2 * (it & 1) * sm_stride + el;
+    unsigned* const sm_next = sM + 2 * ((it & 1) ^ 1) * sm_stride + el;
+    if (kPair) {
+      const unsigned r = __reduce_max_sync(grp, el & 1 ? mx[1] : mx[0]);
+      if (lead) atomicMax(sm, r);
+    } else {
+      const unsigned r0 = __reduce_max_sync(grp, mx[0]), r1 = __reduce_max_sync(grp, mx[1]);
+      if (lead) {
+        atomicMax(sm, r0);
+        atomicMax(sm + sm_stride, r1);
+      }
+    }
     __syncthreads();
-    int eb = (int)(sM[(it & 1) * sM_stride + el] >> 20);
-    if (threadIdx.x == 0) sM[((it & 1) ^ 1) * sM_stride + el] = 0;   // last read before the previous orbital's stages
+    if (threadIdx.x == 0) sm_next[0] = sm_next[sm_stride] = 0;
     ++it;
-    const bool poison = bad || eb == 2047;
-    eb = eb < 64 ? 64 : (eb > 2046 ? 2046 : eb);
-    // V = y 2^sh, sh = kFxBits - (eb - 1022); element results = V 2^(er - sh)
-    const int eo = er + 7 - kFxBits + eb - 1022;
-    const int ec = eo < -980 ? -980 : (eo > 900 ? 900 : eo);
     double2* evo = ev + (long long)o * ev_ostride + eidx * P3 + v * P2 + u * P1;
 #pragma unroll 1
     for (int comp = kPair ? el & 1 : 0; comp < 2; comp += kPair ? 2 : 1) {   // real part, then imaginary part
+      int eb = (int)(sm[kPair ? 0 : comp * sm_stride] >> 20);
+      const bool poison = bad || eb == 2047;
+      eb = eb < 64 ? 64 : (eb > 2046 ? 2046 : eb);
+      // V = y 2^sh, sh = kFxBits - (eb - 1022); element results = V 2^(er - sh), less the raise
+      const int e0 = er + 7 - kFxBits + eb - 1022;
       long long col[P1], t[P1];
       float cf[P1], tf[P1];
 #pragma unroll
       for (int c = 0; c < P1; ++c) {
         const uint2 w = reinterpret_cast<const uint2*>(pfbuf + c * nthr + tid)[comp];
-        col[c] = fx_from_bits(w.y, w.x, eb);
-        cf[c] = 0.0f;
+        col[c] = fx_from_bits(w.y, w.x, eb, cf[c]);
       }
       if (kPair || comp == 1) {   // the thread's slots are free: the next active orbital's column
         const double2* in_n = nullptr;
@@ -254,10 +267,27 @@ __device__ __forceinline__ void hbar_elem_fx(const Geom& g, const FxTab<P1>& tab
       __syncthreads();
       load_line(col, Sy, LS);
       load_line(cf, Fy, LF);
-      fx_apply<P1>(cB, kB, col, cf, to(Ry, LS, Gy, LF));
+      unsigned big = 0;
+      fx_apply<P1>(cB, kB, col, cf, [&](int q, long long x, float xf) {
+        Ry[q * LS] = x;
+        Gy[q * LF] = xf;
+        big |= fx_magnitude(x);
+      });
+      // the part raised by its free bits: a vector with one large entry loses three bits per
+      // contraction, and the middle operator's bound takes up to ten more
+      big = __reduce_or_sync(grp, big);
+      if (lead) atomicOr(&sR[rb * sm_stride + el], big);
       __syncthreads();
+      const int up = fx_free_bits(sR[rb * sm_stride + el]);
+      rb ^= 1;
+      if (threadIdx.x == 0) sR[rb * sm_stride + el] = 0;   // last read a part ago, several barriers back
+      const int eo = e0 - up;
+      const int ec = eo < -980 ? -980 : (eo > 900 ? 900 : eo);
+      const int slot = kPair ? el : 2 * el + comp;         // of the alpha sums
       load_line(col, Rx, 1);
       load_line(cf, Gx, 1);
+#pragma unroll
+      for (int q = 0; q < P1; ++q) fx_raise(col[q], cf[q], up);
       fx_apply<P1>(cB, kB, col, cf, [&](int q, long long x, float xf) {   // U (Gauss-point values)
         t[q] = x;
         tf[q] = xf;
@@ -314,9 +344,9 @@ __device__ __forceinline__ void hbar_elem_fx(const Geom& g, const FxTab<P1>& tab
 #pragma unroll
           for (int i = 0; i < kAcc; ++i) {
             const int w = __reduce_add_sync(grp, lim[i]);
-            if (lead) atomicAdd(&sA[kAcc * el + i], w);
+            if (lead) atomicAdd(&sA[kAcc * slot + i], w);
           }
-          if (threadIdx.x == 0) sE[el] = poison ? 1 << 30 : er + 2 * (7 - (kFxBits - eb + 1022)) - 7;
+          if (threadIdx.x == 0) sE[slot] = poison ? 1 << 30 : er + 2 * (7 - (kFxBits - eb + 1022)) - 7 - 2 * up;
         }
       }
       // backward z (on the thread's own z-line), y, x
@@ -351,25 +381,21 @@ __device__ __forceinline__ void hbar_elem_fx(const Geom& g, const FxTab<P1>& tab
     if (part && tid < 32) {
       double s = 0.0;
       const int ne = (int)blockDim.y >> (kPair ? 1 : 0);
-      for (int e = tid; e < ne; e += 32) {
-        constexpr int rows = kPair ? 2 : 1;
-        int A[kAcc];
+      for (int e = tid; e < ne; e += 32)
+        for (int c = 2 * e; c < 2 * e + 2; ++c) {   // real part, imaginary part
+          int A[kAcc];
 #pragma unroll
-        for (int i = 0; i < kAcc; ++i) {
-          A[i] = sA[kAcc * rows * e + i];
-          sA[kAcc * rows * e + i] = 0;
-          if (kPair) {
-            A[i] += sA[kAcc * (rows * e + 1) + i];
-            sA[kAcc * (rows * e + 1) + i] = 0;
+          for (int i = 0; i < kAcc; ++i) {
+            A[i] = sA[kAcc * c + i];
+            sA[kAcc * c + i] = 0;
           }
+          const long long l = (unsigned)A[0] + ((long long)(unsigned)A[1] << 24) + ((long long)A[2] << 48);
+          const long long m = (unsigned)A[3] + ((long long)(unsigned)A[4] << 24) + ((long long)A[5] << 48);
+          const long long h = (unsigned)A[6] + ((long long)A[7] << 24);
+          const int x = sE[c];
+          const double d = fma((double)h, 0x1p64, fma((double)m, 0x1p32, (double)l * 0x1p10));
+          s += x == 1 << 30 ? __hiloint2double(0x7ff80000, 0) : d * pow2(x / 2) * pow2(x - x / 2);
         }
-        const long long l = (unsigned)A[0] + ((long long)(unsigned)A[1] << 24) + ((long long)A[2] << 48);
-        const long long m = (unsigned)A[3] + ((long long)(unsigned)A[4] << 24) + ((long long)A[5] << 48);
-        const long long h = (unsigned)A[6] + ((long long)A[7] << 24);
-        const int x = sE[rows * e];
-        const double d = fma((double)h, 0x1p64, fma((double)m, 0x1p32, (double)l * 0x1p10));
-        s += x == 1 << 30 ? __hiloint2double(0x7ff80000, 0) : d * pow2(x / 2) * pow2(x - x / 2);
-      }
       const int nl = nthr < 32 ? nthr : 32;
       const unsigned mask = nl == 32 ? 0xffffffffu : (1u << nl) - 1u;
       for (int off = 16; off > 0; off >>= 1) {
@@ -389,8 +415,8 @@ __global__ void __launch_bounds__(256, 2) k_hbar_fx(Geom g, const __grid_constan
                                                     double2* __restrict__ ev) {
   constexpr int P3 = P1 * P1 * P1, ES = SplitLayout<P1, double>::ES, CS = FxTab<P1>::CS;
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ int sA[kAcc * Cfg<P1>::E], sE[Cfg<P1>::E];
-  __shared__ unsigned sV[Cfg<P1>::E], sM[2 * Cfg<P1>::E];
+  __shared__ int sA[2 * kAcc * Cfg<P1>::E], sE[2 * Cfg<P1>::E];
+  __shared__ unsigned sV[Cfg<P1>::E], sM[4 * Cfg<P1>::E], sR[2 * Cfg<P1>::E];
   const int o0 = blockIdx.y * orb_per_cta;
   const int o1 = min(o0 + orb_per_cta, a.n_orb);
   if (a.kry) {   // a CTA whose orbitals have all left the recurrence skips the element set-up
@@ -399,11 +425,11 @@ __global__ void __launch_bounds__(256, 2) k_hbar_fx(Geom g, const __grid_constan
     if (!any) return;
   }
   const int tid = threadIdx.x + blockDim.x * threadIdx.y;
-  if (tid < Cfg<P1>::E) {
-    sV[tid] = 0;
-    sM[tid] = 0;
-    sM[Cfg<P1>::E + tid] = 0;
-    for (int i = 0; i < kAcc; ++i) sA[kAcc * tid + i] = 0;
+  const int nthr = blockDim.x * blockDim.y;
+  for (int i = tid; i < 2 * kAcc * Cfg<P1>::E; i += nthr) sA[i] = 0;
+  for (int i = tid; i < 2 * Cfg<P1>::E; i += nthr) {
+    sV[i % Cfg<P1>::E] = 0;
+    sM[i] = sM[2 * Cfg<P1>::E + i] = sR[i] = 0;
   }
   __syncthreads();
   auto orb = [&](int o, const double2*& in, double& sc) -> bool {
@@ -419,7 +445,7 @@ __global__ void __launch_bounds__(256, 2) k_hbar_fx(Geom g, const __grid_constan
                           reinterpret_cast<long long*>(smem + FxSmem<P1>::lines(blockDim.y)) + (size_t)threadIdx.y * ES,
                           reinterpret_cast<float*>(smem + FxSmem<P1>::tails(blockDim.y)) +
                               (size_t)threadIdx.y * SplitLayout<P1, float>::ES,
-                          sA, sE, sV, sM, Cfg<P1>::E, vks,
+                          sA, sE, sV, sM, sR, Cfg<P1>::E, vks,
                           ((long long)blockIdx.x * blockDim.y + threadIdx.y) >> (kPair ? 1 : 0), o0, o1, orb, ev,
                           (long long)g.nx * g.ny * g.nz * P3, a.part, a.part_stride, blockIdx.x,
                           reinterpret_cast<double2*>(smem + FxSmem<P1>::pf(blockDim.y)));
@@ -434,8 +460,8 @@ __global__ void __launch_bounds__(256, 2) k_hbar_batch_fx(const BSys* __restrict
                                                           int* __restrict__ qctr) {
   constexpr int P3 = P1 * P1 * P1, ES = SplitLayout<P1, double>::ES, CS = FxTab<P1>::CS;
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ int sA[kAcc * Cfg<P1>::E], sE[Cfg<P1>::E];
-  __shared__ unsigned sV[Cfg<P1>::E], sM[2 * Cfg<P1>::E];
+  __shared__ int sA[2 * kAcc * Cfg<P1>::E], sE[2 * Cfg<P1>::E];
+  __shared__ unsigned sV[Cfg<P1>::E], sM[4 * Cfg<P1>::E], sR[2 * Cfg<P1>::E];
   __shared__ BSys sS;
   __shared__ BItem sW;
   __shared__ int sIt;
@@ -448,11 +474,10 @@ __global__ void __launch_bounds__(256, 2) k_hbar_batch_fx(const BSys* __restrict
       sIt = it;
       if (it < n_items) sW = items[it];
     }
-    if (tid < Cfg<P1>::E) {
-      sV[tid] = 0;
-      sM[tid] = 0;
-      sM[Cfg<P1>::E + tid] = 0;
-      for (int i = 0; i < kAcc; ++i) sA[kAcc * tid + i] = 0;
+    for (int i = tid; i < 2 * kAcc * Cfg<P1>::E; i += nthr) sA[i] = 0;
+    for (int i = tid; i < 2 * Cfg<P1>::E; i += nthr) {
+      sV[i % Cfg<P1>::E] = 0;
+      sM[i] = sM[2 * Cfg<P1>::E + i] = sR[i] = 0;
     }
     __syncthreads();
     if (sIt >= n_items) break;
@@ -485,7 +510,7 @@ __global__ void __launch_bounds__(256, 2) k_hbar_batch_fx(const BSys* __restrict
         reinterpret_cast<float*>(smem + FxSmem<P1>::kc(blockDim.y)) + threadIdx.y * 3 * FxTab<P1>::KS,
         reinterpret_cast<long long*>(smem + FxSmem<P1>::lines(blockDim.y)) + (size_t)threadIdx.y * ES,
         reinterpret_cast<float*>(smem + FxSmem<P1>::tails(blockDim.y)) + (size_t)threadIdx.y * SplitLayout<P1, float>::ES,
-        sA, sE, sV, sM, Cfg<P1>::E, S.vks, (long long)w.eblk * blockDim.y + threadIdx.y, w.o0, w.o1, orb,
+        sA, sE, sV, sM, sR, Cfg<P1>::E, S.vks, (long long)w.eblk * blockDim.y + threadIdx.y, w.o0, w.o1, orb,
         static_cast<double2*>(S.ev), S.n_elem * P3, S.apart, S.n_eblk, w.eblk,
         reinterpret_cast<double2*>(smem + FxSmem<P1>::pf(blockDim.y)));
   }
@@ -567,8 +592,7 @@ __global__ void __launch_bounds__(256, 2) k_density_fx(Geom g, const __grid_cons
 #pragma unroll
       for (int c = 0; c < P1; ++c) {
         const double x = comp ? w[c].y : w[c].x;
-        col[c] = fx_from_bits((unsigned)__double2hiint(x), (unsigned)__double2loint(x), eb);
-        cf[c] = 0.0f;
+        col[c] = fx_from_bits((unsigned)__double2hiint(x), (unsigned)__double2loint(x), eb, cf[c]);
       }
       fx_apply<P1>(cB, kB, col, cf, [&](int q, long long x, float xf) {
         S1[q * PS + v * LS + u] = x;

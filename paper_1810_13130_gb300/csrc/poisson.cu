@@ -291,7 +291,8 @@ __global__ void __launch_bounds__(256) k_gemm_fx(Gemm g, const CgState* cg) {
   const bool a_k_fast = (g.sAk == 1);
   const bool b_n_fast = (g.sBn == 1);
   const auto put = [](double x, int eb, int2* s, float* sf) {   // limbs, and l 2^-32
-    const FxV v = fx_operand(fx_from_bits((unsigned)__double2hiint(x), (unsigned)__double2loint(x), min(eb, 2046)) + kFxHalf, 0.0f);
+    float cut;
+    const FxV v = fx_operand(fx_from_bits((unsigned)__double2hiint(x), (unsigned)__double2loint(x), min(eb, 2046), cut) + kFxHalf, 0.0f);
     *s = make_int2(v.h, v.l);
     *sf = v.g - 1.5f;
   };

@@ -166,7 +166,7 @@ Tables1D tdks_build_tables(int p, int nq) {
       ld s = 0.0L;
       for (int m = 0; m < nq; ++m) s += Dg[m * nq + a] * om[m] * Dg[m * nq + b];
       s /= sqrtl(om[a] * om[b]);
-      t.Kw[a * nq + b] = (double)s;
+      t.Kw[a * nq + b] = s;
       row += fabsl(s);
     }
     kinf = row > kinf ? row : kinf;

@@ -74,7 +74,7 @@ namespace tdks {
 // Fixed-point tables of a degree (fixed.cuh), units of 2^-63.
 struct FxHost {
   const long long* c = nullptr; // folded B' = W^1/2 B, then B'^T (2 * cs_size entries)
-  const double* dK = nullptr;   // device: folded K' = W^-1/2 Kq W^-1/2 (cs_size doubles)
+  const double* dK = nullptr;   // device: folded K' = W^-1/2 Kq W^-1/2, as cs_size doubles and the rest of each
   double kinf = 0.0;            // largest row sum of |K'|
   const double* w = nullptr;    // Gauss weights
 };
@@ -183,7 +183,7 @@ struct Tables1D {
   std::vector<double> Kq;          // [nq][nq] Dg^T diag(omega) Dg on Gauss-point Lagrange basis
   std::vector<double> K1, Mg;      // [P1][P1] D^T W D and B^T W B
   std::vector<long double> Bw;     // [nq][P1] W^1/2 B
-  std::vector<double> Kw;          // [nq][nq] W^-1/2 Kq W^-1/2
+  std::vector<long double> Kw;     // [nq][nq] W^-1/2 Kq W^-1/2
   double kw_inf = 0.0;             // largest row sum of |Kw|
 };
 Tables1D tdks_build_tables(int p, int nq);
