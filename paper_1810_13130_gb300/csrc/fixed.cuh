@@ -112,6 +112,21 @@ struct FxDot {
   __host__ __device__ __forceinline__ void top(FxC c, const FxV& x) { hi = fx_mad(c.h, x.h, hi); }
 };
 
+// sum u r of two sets of values: dh 2^64 + (dm + da) 2^32 + dl 2^10, exact but for the
+// rounding of da (the tails' products with the other value's high word; the rest of them is
+// below 2^-54 of u r) and the cut of dl.
+struct FxInner {
+  long long dh = 0, dm = 0, dl = 0;
+  float da = 0.0f;
+  __host__ __device__ __forceinline__ void add(long long u, float uf, long long r, float rf) {
+    const FxV a = fx_operand(u + kFxHalf, 0.0f), b = fx_operand(r + kFxHalf, 0.0f);
+    da = fmaf((float)a.h, rf, fmaf((float)b.h, uf, da));
+    dm = fx_mad(a.h, b.l, fx_mad(a.l, b.h, dm));
+    dh = fx_mad(a.h, b.h, dh);
+    dl += fx_mad(a.l, b.l, 0) >> 10;
+  }
+};
+
 // Folded operator: coefficients in the layout of tdks_internal.h (CS of them), tail
 // constants of the even, odd and middle rows (KS).
 template <int N>

@@ -322,22 +322,16 @@ __device__ __forceinline__ void hbar_elem_fx(const Geom& g, const FxTab<P1>& tab
       {
         const long long* const Rz = S2 + v * LS + u;
         const float* const Gz = F2 + v * LF + u;
-        // sum_q u_q r_q: dh 2^64 + (dm + da) 2^32 + dl 2^10, exact but for the rounding of da and dl
-        long long dh = 0, dm = 0, dl = 0;
-        float da = 0.0f;
+        FxInner ur;
         fx_apply<P1>([&](int i) { return sK[2 * CS + i]; }, [&](int i) { return sKk[2 * KS + i]; }, col, cf,
                      [&](int q, long long x, float xf) {                  // r = R + cz K'_z U, and u r
                        x += Rz[q * PS];
                        t[q] = x;
                        tf[q] = xf + Gz[q * PF];
-                       const FxV a = fx_operand(col[q] + kFxHalf, 0.0f), b = fx_operand(x + kFxHalf, 0.0f);
-                       da = fmaf((float)a.h, tf[q], da);
-                       dm = fx_mad(a.h, b.l, fx_mad(a.l, b.h, dm));
-                       dh = fx_mad(a.h, b.h, dh);
-                       dl += fx_mad(a.l, b.l, 0) >> 10;
+                       ur.add(col[q], Fz[q * PF], x, tf[q]);
                      });
         if (part) {   // the element's sum: 24-bit limbs, added over its lanes and warps
-          dm += __float2ll_rn(da);
+          const long long dh = ur.dh, dm = ur.dm + __float2ll_rn(ur.da), dl = ur.dl;
           const int lim[kAcc] = {(int)(dl & 0xffffff), (int)((dl >> 24) & 0xffffff), (int)(dl >> 48),
                                  (int)(dm & 0xffffff), (int)((dm >> 24) & 0xffffff), (int)(dm >> 48),
                                  (int)(dh & 0xffffff), (int)(dh >> 24)};

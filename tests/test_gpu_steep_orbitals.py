@@ -185,3 +185,28 @@ def test_parts_are_independent(p, n, n_orb):
         out = ctx.apply_H(torch.complex(a * 2.0 ** -k, b).contiguous())
         assert torch.equal(out.real, Ha.real * 2.0 ** -k) and torch.equal(out.imag, Hb.real), k
     ctx.close()
+
+
+@pytest.mark.parametrize("decay", [0.0, 8.0, 20.0])
+@pytest.mark.parametrize("p,n", [(3, (2, 2, 1)), (4, (2, 1, 2)), (6, (1, 1, 2)), (7, (2, 1, 1)), (8, (2, 1, 1))])
+def test_first_lanczos_coefficient(p, n, decay):
+    """alpha_0 = <psi|Hbar|psi> / <psi|psi> is the phase per time of a one-dimensional Krylov exponential."""
+    ctx, ref, m = _setup(p, n, 2)
+    rng = np.random.default_rng(92)
+    v = -20.0 * np.exp(3 * rng.uniform(-1, 1, (m.n_elem, (p + 1) ** 3)))
+    psi = _steep(ref, p, decay, 2, 91)
+    ctx.set_potential(torch.from_numpy(v).cuda())
+    vq = _grid(v, n, p + 1)
+    # the roundings of an entry of Hbar psi (test_apply) and 2 of the sums, for the larger part;
+    # the angle of a component comes back within 4 roundings of 1
+    bound = (18 + 3 + 7 + 2 * (p + 1) + 11 + 2) * U
+    for o in range(2):
+        x = [psi[o].real.astype(LD), psi[o].imag.astype(LD)]
+        nrm = sum((t * t).sum() for t in x)
+        alpha = sum((t * ref.apply(vq, t)).sum() for t in x) / nrm
+        mag = sum((abs(t) * ref.apply(vq, abs(t), mag=True)).sum() for t in x) / nrm
+        tau = float(1 / mag)
+        out, _ = ctx.expm(torch.from_numpy(psi[o:o + 1].reshape(1, -1).copy()).cuda(), tau, tol=1e30, k_max=1)
+        got = -np.angle(np.vdot(psi[o].ravel(), out.cpu().numpy().ravel())) / tau
+        assert abs(got - alpha) <= bound * mag + 4 * U / tau
+    ctx.close()
