@@ -478,17 +478,17 @@ tdks_status kb_project(tdks_ctx* c, const ApplyArgs& a) {
   KbState* k = static_cast<KbState*>(c->kb);
   if (!k) return TDKS_OK;
   if (a.n_orb > k->c_orb) {   // a plain application of more vectors than the system's orbitals
-    cudaFree(k->d_P);
-    cudaFree(k->d_CD);
-    k->d_P = k->d_CD = nullptr;
-    k->c_orb = 0;
-    if (cudaMalloc(&k->d_P, ((size_t)a.n_orb * k->n_chunks * k->npg + 1) * sizeof(double2)) != cudaSuccess ||
-        cudaMalloc(&k->d_CD, (size_t)a.n_orb * k->n_proj * sizeof(double2)) != cudaSuccess) {
+    const auto alloc = [](size_t n) {
+      double2* p = nullptr;
+      if (cudaMalloc(&p, n * sizeof(double2)) == cudaSuccess) return p;
       cudaGetLastError();
+      return (double2*)nullptr;
+    };
+    // (captured Lanczos loops hold the old buffers: dropped before these are freed)
+    if (!replace_pair(k->d_P, (size_t)a.n_orb * k->n_chunks * k->npg + 1, k->d_CD, (size_t)a.n_orb * k->n_proj, alloc,
+                      [](double2* p) { cudaFree(p); }, [&] { kgraph_drop(c); }))
       return tdks_fail(c, TDKS_ERR_NOMEM, "projections");
-    }
     k->c_orb = a.n_orb;
-    kgraph_drop(c);           // captured Lanczos loops hold the old buffers
     cudaFree(k->d_view);      // as does the batched view
     k->d_view = nullptr;
   }

@@ -175,6 +175,25 @@ tdks_status tdks_cuda_check(tdks_ctx* c, cudaError_t e, const char* what);
 
 Geom tdks_geom(const tdks_ctx* c);
 
+// Two buffers replaced by others of na and nb entries, both allocated before the old ones go:
+// a failed allocation leaves those in place, for whoever holds their addresses.  before():
+// called once the new ones are there, while the old ones still are.
+template <class T, class Alloc, class Free, class Before>
+bool replace_pair(T*& a, size_t na, T*& b, size_t nb, Alloc alloc, Free release, Before before) {
+  T* const x = alloc(na);
+  T* const y = x ? alloc(nb) : nullptr;
+  if (!y) {
+    if (x) release(x);
+    return false;
+  }
+  before();
+  release(a);
+  release(b);
+  a = x;
+  b = y;
+  return true;
+}
+
 // tables.cpp: host construction of the 1-D tables (long double)
 struct Tables1D {
   std::vector<double> xi, w;       // GLL nodes and weights (P1)

@@ -26,6 +26,29 @@ int main() {
 }
 """
 
+PAIR = r"""
+#include <cstdio>
+#include <set>
+#include "tdks_internal.h"
+// projections replaced by larger ones: the allocation that fails (0: none), what is left after it
+int main() {
+  for (int fail = 0; fail < 3; ++fail) {
+    static int heap[8];
+    std::set<int*> live{heap, heap + 1};
+    int *a = heap, *b = heap + 1, calls = 0, dropped = 0;
+    const auto alloc = [&](size_t) -> int* {
+      if (++calls == fail) return nullptr;
+      live.insert(heap + 1 + calls);
+      return heap + 1 + calls;
+    };
+    const bool ok = replace_pair(a, 5, b, 6, alloc, [&](int* p) { live.erase(p); },
+                                 [&] { dropped += live.count(heap) && live.count(heap + 1); });
+    const bool kept = a == heap && b == heap + 1, fresh = a == heap + 2 && b == heap + 3;
+    printf("%d %d %d %d\n", (int)ok, fail ? kept : fresh, (int)(live == std::set<int*>{a, b}), dropped);
+  }
+}
+"""
+
 
 def _run(tmp_path, src):
     cxx = shutil.which("g++")
@@ -42,3 +65,10 @@ def _run(tmp_path, src):
 def test_product_tiles_fit_the_grid(tmp_path):
     n, bad = map(int, _run(tmp_path, GEMM).split())
     assert n > 10000 and bad == 0
+
+
+def test_a_failed_allocation_leaves_the_projections(tmp_path):
+    """Captured Lanczos loops hold the addresses of the projections: they may go only once their successors are
+    there, and the loops with them."""
+    rows = _run(tmp_path, PAIR).split("\n")
+    assert rows[:3] == ["1 1 1 1", "0 1 1 0", "0 1 1 0"]
