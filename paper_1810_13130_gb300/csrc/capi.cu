@@ -131,23 +131,6 @@ float round_bf16(float x) {
   return r;
 }
 
-// Folded storage of a centrosymmetric n x n matrix (layout in tdks_internal.h).
-template <typename T>
-void fold_centrosymmetric(const T* M, int n, T* out) {
-  const int h = n / 2;
-  const T half = (T)0.5;
-  for (int q = 0; q < h; ++q)
-    for (int i = 0; i < h; ++i) {
-      out[q * h + i] = half * (M[q * n + i] + M[q * n + (n - 1 - i)]);
-      out[h * h + q * h + i] = half * (M[q * n + i] - M[q * n + (n - 1 - i)]);
-    }
-  T* mc = out + 2 * h * h;
-  T* mr = mc + h;
-  for (int q = 0; q < h; ++q) mc[q] = (n & 1) ? M[q * n + h] : (T)0;
-  for (int i = 0; i < h; ++i) mr[i] = (n & 1) ? M[h * n + i] : (T)0;
-  mr[h] = (n & 1) ? M[h * n + h] : (T)0;
-}
-
 tdks_status check_orb(tdks_ctx* c, int n_orb) {
   if (n_orb < 1 || n_orb > c->n_orb)
     return tdks_fail(c, TDKS_ERR_ARG, "n_orb must be in [1, system n_orb]");
@@ -328,8 +311,8 @@ tdks_status tdks_create(const tdks_mesh_desc* m, const tdks_system_desc* s, void
     fold_centrosymmetric(t.Kq.data(), P1, &tab[tab_off_csK(P1)]);
     // GLL-collocation variant: GLL weights and the folded 1-D stiffness K1 = D^T W D
     std::memcpy(&tab[tab_off_wl(P1)], t.w.data(), P1 * sizeof(double));
-    fold_centrosymmetric(t.K1.data(), P1, &tab[tab_off_csK1(P1)]);
-    fold_centrosymmetric(t.Mg.data(), P1, &tab[tab_off_csMg(P1)]);
+    std::copy(t.csK1.begin(), t.csK1.end(), &tab[tab_off_csK1(P1)]);
+    std::copy(t.csMg.begin(), t.csMg.end(), &tab[tab_off_csMg(P1)]);
   }
   std::vector<float> tabf(tab.begin(), tab.end());
   std::vector<float> tabdf(2 * tab.size());

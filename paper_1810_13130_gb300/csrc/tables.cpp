@@ -172,17 +172,23 @@ Tables1D tdks_build_tables(int p, int nq) {
     kinf = row > kinf ? row : kinf;
   }
   t.kw_inf = (double)kinf;
-  t.K1.resize(P1 * P1);
-  t.Mg.resize(P1 * P1);
+  // The 1-D stiffness and mass, folded before they are rounded.  A constant has no stiffness:
+  // what the rounded rows leave of it comes back in the potential, larger by h^2 over the lowest
+  // eigenvalue.  Folding rounded entries rounds them again: Hartree potentials of solves far
+  // inside their tolerance were off by 5.8e-14 (18 x 17 x 9 elements, p = 3) and 8.0e-14
+  // (16 x 5 x 5, p = 7), 2.0e-14 and 4.5e-14 with the full rounded matrices; now 2.5e-16, 1.6e-14.
+  std::vector<ld> K1(P1 * P1), Mg(P1 * P1), cs(cs_size(P1));
   for (int i = 0; i < P1; ++i)
-    for (int j = 0; j < P1; ++j) {
-      ld sk = 0.0L, sm = 0.0L;
+    for (int j = 0; j < P1; ++j)
       for (int q = 0; q < nq; ++q) {
-        sk += D[q * P1 + i] * om[q] * D[q * P1 + j];
-        sm += B[q * P1 + i] * om[q] * B[q * P1 + j];
+        K1[i * P1 + j] += D[q * P1 + i] * om[q] * D[q * P1 + j];
+        Mg[i * P1 + j] += B[q * P1 + i] * om[q] * B[q * P1 + j];
       }
-      t.K1[i * P1 + j] = (double)sk;
-      t.Mg[i * P1 + j] = (double)sm;
-    }
+  t.K1.assign(K1.begin(), K1.end());
+  t.Mg.assign(Mg.begin(), Mg.end());
+  fold_centrosymmetric(K1.data(), P1, cs.data());
+  t.csK1.assign(cs.begin(), cs.end());
+  fold_centrosymmetric(Mg.data(), P1, cs.data());
+  t.csMg.assign(cs.begin(), cs.end());
   return t;
 }

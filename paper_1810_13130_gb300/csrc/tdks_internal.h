@@ -201,6 +201,7 @@ struct Tables1D {
   std::vector<double> B, D;        // [nq][P1] Lagrange values / derivatives at Gauss points
   std::vector<double> Kq;          // [nq][nq] Dg^T diag(omega) Dg on Gauss-point Lagrange basis
   std::vector<double> K1, Mg;      // [P1][P1] D^T W D and B^T W B
+  std::vector<double> csK1, csMg;  // the same, folded (fold_centrosymmetric)
   std::vector<long double> Bw;     // [nq][P1] W^1/2 B
   std::vector<long double> Kw;     // [nq][nq] W^-1/2 Kq W^-1/2
   double kw_inf = 0.0;             // largest row sum of |Kw|
@@ -225,6 +226,21 @@ void tdks_fdm_axis(const Tables1D& t, int p, const double* br, int n_el, std::ve
 // and M[h][h].  B, B^T and Kq are centrosymmetric because the GLL nodes and the
 // Gauss points are symmetric about 0.
 TDKS_HD inline int cs_size(int P1) { return 2 * (P1 / 2) * (P1 / 2) + 2 * (P1 / 2) + 1; }
+template <typename T>
+void fold_centrosymmetric(const T* M, int n, T* out) {
+  const int h = n / 2;
+  const T half = (T)0.5;
+  for (int q = 0; q < h; ++q)
+    for (int i = 0; i < h; ++i) {
+      out[q * h + i] = half * (M[q * n + i] + M[q * n + (n - 1 - i)]);
+      out[h * h + q * h + i] = half * (M[q * n + i] - M[q * n + (n - 1 - i)]);
+    }
+  T* mc = out + 2 * h * h;
+  T* mr = mc + h;
+  for (int q = 0; q < h; ++q) mc[q] = (n & 1) ? M[q * n + h] : (T)0;
+  for (int i = 0; i < h; ++i) mr[i] = (n & 1) ? M[h * n + i] : (T)0;
+  mr[h] = (n & 1) ? M[h * n + h] : (T)0;
+}
 TDKS_HD inline int tab_off_B(int) { return 0; }
 TDKS_HD inline int tab_off_Kq(int P1) { return P1 * P1; }
 TDKS_HD inline int tab_off_w(int P1) { return 2 * P1 * P1; }
