@@ -1330,9 +1330,16 @@ tdks_status run_expm_ws(tdks_ctx* c, int w, const double2* in, double2* out, int
       any |= (h[o].status == KRY_ACTIVE);
       failed |= (h[o].status == KRY_FAILED);
     }
-    if (failed)
+    if (failed) {
+      // an orbital that fails before its first sub-step ends is handed back as it came, as with in == out
+      for (int o = 0; o < n_orb; ++o)
+        if (in != out && h[o].status != KRY_DONE && h[o].nsub == 0)
+          TDKS_CU(c, cudaMemcpyAsync(out + (int64_t)o * n, in + (int64_t)o * n, (size_t)n * sizeof(double2),
+                                     cudaMemcpyDeviceToDevice, c->stream));
+      TDKS_CU(c, cudaStreamSynchronize(c->stream));
       return tdks_fail(c, TDKS_ERR_NOT_CONVERGED,
                        "Lanczos: no admissible sub-step, sub-step cap or non-finite norm");
+    }
     if (!any) break;
     n_active = 0;
     for (int o = 0; o < n_orb; ++o) n_active += (h[o].status == KRY_ACTIVE);
