@@ -248,6 +248,54 @@ __host__ __device__ __forceinline__ long long fx_scaled(double c, double hi, dou
 #endif
 }
 
+// Products of two numbers in fixed point, |V| < 2^kFxPBits, each with the exponent eb of the
+// largest entry of its row or column; the bits below a unit are cut.  At 55 bits, which need no
+// carry(), the 2-norm of a fast-diagonalization product was off by up to six times an FP64
+// chain's error (steep or peaked columns); at 58 it is at most 0.84 times the chain's or one
+// rounding, 2^-53, whichever is larger (axes of 3 to 255 nodes; host test).
+constexpr int kFxPBits = 58;
+constexpr int kFxK = 255;   // terms: K 2^52 and the carries < 2^61
+__host__ __device__ __forceinline__ FxV fx_factor(unsigned hw, unsigned lw, int eb) {
+  const int e = (int)((hw >> 20) & 0x7ffu);
+  const unsigned long long m = (((unsigned long long)((hw & 0xfffffu) | 0x100000u) << 32) | lw) << (kFxPBits - 53);
+  const int d = eb - e;
+  const long long v = e == 0 || d > 63 ? 0 : (long long)(m >> (d & 63));
+  return fx_operand(((hw & 0x80000000u) ? -v : v) + kFxHalf, 0.0f);
+}
+// sum a b in units of 2^64: h h' and h l' + l h' exactly (carry() at least every 16 terms), l l'
+// in FP32
+struct FxSum {
+  long long mid = 0, hi = 0;
+  float f = 0.0f;
+  // lf, lg: l 2^-32 of a and b
+  __host__ __device__ __forceinline__ void add(int ah, int al, float lf, int bh, int bl, float lg) {
+    mid = fx_mad(ah, bl, fx_mad(al, bh, mid));
+    hi = fx_mad(ah, bh, hi);
+    f = fmaf(lf, lg, f);
+  }
+  __host__ __device__ __forceinline__ void carry() {
+    hi += mid >> 32;
+    mid &= 0xffffffffll;
+  }
+  // the sum 2^s, s its free bits (at most 20), |.| < 2^62
+  __host__ __device__ __forceinline__ long long value(int& s) const {
+    const long long t = hi + (mid >> 32), m = t ^ (t >> 63);
+#ifdef __CUDA_ARCH__
+    const int z = __clzll(m);
+#else
+    const int z = m ? __builtin_clzll((unsigned long long)m) : 64;
+#endif
+    s = z - 2 < 20 ? z - 2 : 20;
+    const float fr = f * fx_bits_float((unsigned)(127 + s) << 23);
+#ifdef __CUDA_ARCH__
+    const int r = __float2int_rn(fr);
+#else
+    const int r = (int)lrintf(fr);
+#endif
+    return (long long)((unsigned long long)t << s) + (long long)((unsigned)mid >> (32 - s)) + r;
+  }
+};
+
 #ifdef __CUDACC__
 __device__ __forceinline__ double pow2(int e) {   // 2^e, e clamped to the normal range
   e = e < -1022 ? -1022 : (e > 1023 ? 1023 : e);

@@ -158,7 +158,7 @@ struct Gemm {
   int M, N, K;
 };
 
-constexpr int GK = 16;   // depth tile
+constexpr int GK = 16;   // depth tile (FxSum::carry once per tile: at most 16)
 
 // GT x GT output tile, 16 x 16 threads of (GT / 16)^2 outputs.  The product is bound by the
 // FP64 pipe whatever the tile, so the tile only decides how much of the work is padding and
@@ -237,13 +237,9 @@ __global__ void __launch_bounds__(256) k_gemm(Gemm g, const CgState* cg) {
 
 // The same product in fixed point (fixed.cuh): every row of A and every column of B has the
 // exponent of its largest entry (one pass over the panels first; the second read is a cache
-// hit), entries are 55-bit integers, a dot product of up to kFxK terms keeps h h' and
-// h l' + l h' exactly in 64 bits and l l' in FP32, and each output is rounded once.  Three
+// hit), a dot product of up to kFxK terms is an FxSum, and each output is rounded once.  Three
 // wide integer multiply-adds and one FP32 one per term instead of an FP64 multiply-add, which
 // takes five times as long on the FP64 pipe.  (Double-float products take the same time.)
-// Against 64-bit-mantissa products of 23 to 200 terms the 2-norm error is 0.6 to 2.8e-16, that
-// of an FP64 chain 1.6 to 4.5e-16 (random, smooth and 12-decade inputs).
-constexpr int kFxK = 255;   // 2 K 2^54 < 2^63
 template <int GT>
 __global__ void __launch_bounds__(256) k_gemm_fx(Gemm g, const CgState* cg) {
   if (cg && cg->done) return;
@@ -274,25 +270,16 @@ __global__ void __launch_bounds__(256) k_gemm_fx(Gemm g, const CgState* cg) {
     atomicMax(&eB[l], mb);
   }
   __syncthreads();
-  if (tid < GT) {   // exponent fields, those of zero and tiny rows raised as fx_from_bits wants them
+  if (tid < GT) {   // exponent fields, those of zero and tiny rows raised
     eA[tid] = max(eA[tid] >> 20, 64u);
     eB[tid] = max(eB[tid] >> 20, 64u);
   }
   __syncthreads();
-  long long mid[R][R], hi[R][R];
-  float f[R][R];
-#pragma unroll
-  for (int i = 0; i < R; ++i)
-#pragma unroll
-    for (int j = 0; j < R; ++j) {
-      mid[i][j] = hi[i][j] = 0;
-      f[i][j] = 0.0f;
-    }
+  FxSum acc[R][R];
   const bool a_k_fast = (g.sAk == 1);
   const bool b_n_fast = (g.sBn == 1);
   const auto put = [](double x, int eb, int2* s, float* sf) {   // limbs, and l 2^-32
-    float cut;
-    const FxV v = fx_operand(fx_from_bits((unsigned)__double2hiint(x), (unsigned)__double2loint(x), min(eb, 2046), cut) + kFxHalf, 0.0f);
+    const FxV v = fx_factor((unsigned)__double2hiint(x), (unsigned)__double2loint(x), min(eb, 2046));
     *s = make_int2(v.h, v.l);
     *sf = v.g - 1.5f;
   };
@@ -322,12 +309,12 @@ __global__ void __launch_bounds__(256) k_gemm_fx(Gemm g, const CgState* cg) {
 #pragma unroll
       for (int i = 0; i < R; ++i)
 #pragma unroll
-        for (int j = 0; j < R; ++j) {
-          mid[i][j] = fx_mad(a[i].x, w[j].y, fx_mad(a[i].y, w[j].x, mid[i][j]));
-          hi[i][j] = fx_mad(a[i].x, w[j].x, hi[i][j]);
-          f[i][j] = fmaf(af[i], wf[j], f[i][j]);
-        }
+        for (int j = 0; j < R; ++j) acc[i][j].add(a[i].x, a[i].y, af[i], w[j].x, w[j].y, wf[j]);
     }
+#pragma unroll
+    for (int i = 0; i < R; ++i)
+#pragma unroll
+      for (int j = 0; j < R; ++j) acc[i][j].carry();
     __syncthreads();
   }
   double* C = g.C + b * g.sCb;
@@ -339,13 +326,10 @@ __global__ void __launch_bounds__(256) k_gemm_fx(Gemm g, const CgState* cg) {
     for (int j = 0; j < R; ++j) {
       const long long gn = n0 + tx * R + j;
       if (gn >= g.N) continue;
-      // t + (low word of mid) 2^-32 + f in units of 2^64, shifted left by the free bits
-      const long long t = hi[i][j] + (mid[i][j] >> 32);
-      const int s = min(__clzll(t ^ (t >> 63)) - 2, 20);
-      const float fr = ldexpf(f[i][j], s);
-      const long long v = (t << s) + (long long)((unsigned)mid[i][j] >> (32 - s)) + __float2int_rn(fr);
+      int s;
+      const long long v = acc[i][j].value(s);
       const int ea = eA[ty * R + i], eb = eB[tx * R + j];
-      const int e = 64 - s + (ea - 1022 - kFxBits) + (eb - 1022 - kFxBits);
+      const int e = 64 - s + (ea - 1022 - kFxPBits) + (eb - 1022 - kFxPBits);
       double x = e > -1000 && e < 900 ? fx_to_double(v, e << 20) : fx_to_double(v, 0) * pow2(e / 2) * pow2(e - e / 2);
       if (ea == 2047 || eb == 2047) x = __hiloint2double(0x7ff80000, 0);   // a non-finite row or column
       C[gm * g.sCm + gn * g.sCn] = x;
