@@ -784,11 +784,14 @@ tdks_status tdks_batch_set_kb(tdks_batch* b, int sys, int n_atoms, const double*
   if (!b || sys < 0 || sys >= b->n_sys) return TDKS_ERR_ARG;
   tdks_ctx* cx = b->ctx[sys];
   B_CU(b, cudaStreamSynchronize(b->st));
-  B_TRY(b, ctx_try(b, cx, tdks_set_kb(cx, n_atoms, R, a, bb, c, lmax)), "tdks_set_kb");
+  // the old projectors are gone whatever comes of this: the step graph and the descriptors that
+  // hold their buffers go with them before an error is returned
+  const tdks_status st = tdks_set_kb(cx, n_atoms, R, a, bb, c, lmax);
+  const std::string err = cx->err;
   double* part = nullptr;
   int nblk = 0;
   const KbView* v = kb_view(cx, &part, &nblk, nullptr);
-  if (cx->kb && !v) return bfail(b, TDKS_ERR_NOMEM, "projector view");
+  const bool no_view = cx->kb && !v;
   for (BSys* S : {&b->h_half[sys], &b->h_full[sys]}) {
     S->kb = v;
     S->kb_part = v ? part : nullptr;
@@ -797,6 +800,8 @@ tdks_status tdks_batch_set_kb(tdks_batch* b, int sys, int n_atoms, const double*
   invalidate_graph(b);
   B_TRY(b, build_kb_lists(b), "projectors");
   B_TRY(b, upload_descriptors(b), "projectors");
+  if (st != TDKS_OK) return bfail(b, st, "tdks_set_kb: " + err);
+  if (no_view) return bfail(b, TDKS_ERR_NOMEM, "projector view");
   return TDKS_OK;
 }
 
