@@ -295,11 +295,7 @@ tdks_status tdks_create(const tdks_mesh_desc* m, const tdks_system_desc* s, void
   c->n_elem = (int64_t)c->nx * c->ny * c->nz;
   // tables (double and float copies)
   std::vector<double> tab(tab_size(P1), 0.0);
-  std::memcpy(&tab[tab_off_B(P1)], t.B.data(), P1 * P1 * sizeof(double));
-  std::memcpy(&tab[tab_off_Kq(P1)], t.Kq.data(), P1 * P1 * sizeof(double));
   std::memcpy(&tab[tab_off_w(P1)], t.omega.data(), P1 * sizeof(double));
-  std::memcpy(&tab[tab_off_K1(P1)], t.K1.data(), P1 * P1 * sizeof(double));
-  std::memcpy(&tab[tab_off_Mg(P1)], t.Mg.data(), P1 * P1 * sizeof(double));
   std::memcpy(&tab[tab_off_eta(P1)], t.eta.data(), P1 * sizeof(double));
   {
     // folded (even-odd) forms of B (q <- i), B^T (i <- q) and Kq

@@ -32,7 +32,7 @@ using namespace tdks;
 namespace {
 
 // ---------------------------------------------------------------------------
-// Hbar psibar, complex, contraction type T (double or float)
+// Hbar psibar, complex lines, float contractions (BF16 operands: bf_round)
 //
 // Each thread of an element's P1 x P1 plane owns one full 1-D line in every
 // stage (a z-column, a y-line or an x-line), applies the folded 1-D operator in
@@ -99,8 +99,7 @@ __device__ __forceinline__ void hbar_elem_body(const Geom& g, const T* sB, const
   }
   const long long plane = (long long)g.nix * g.niy;
   // gather: z-column (a = u, b = v); Loewdin scales of the column (once per CTA)
-  constexpr bool kF32 = std::is_same<T, float>::value;
-  constexpr bool kDF = std::is_same<T, Df>::value;
+  static_assert(std::is_same<T, float>::value, "double-float and FP32 have the split body, FP64 hbar_fx.cu");
   const int Ig = ex * g.p + u, Jg = ey * g.p + v;
   const bool inG = valid && Ig >= 1 && Ig <= g.nix && Jg >= 1 && Jg <= g.niy;
   const long long baseG = inG ? (long long)(Ig - 1) + (long long)g.nix * (Jg - 1) : 0;
@@ -116,28 +115,16 @@ __device__ __forceinline__ void hbar_elem_body(const Geom& g, const T* sB, const
     double sc = 1.0;
     if (!orb(o, in, sc)) continue;
     V col[P1], t[P1];
-    T scT;
-    if constexpr (kF32) scT = d2f_bits(sc);
-    else scT = from_d<T>(sc);
+    const T scT = d2f_bits(sc);
 #pragma unroll
     for (int c = 0; c < P1; ++c) {
       const int K = ez * g.p + c;
       vzero(col[c]);
       if (inG && K >= 1 && K <= g.niz) {
         const double2 w2 = in[baseG + plane * (K - 1)];
-        if constexpr (kF32) {   // no FP64 arithmetic in the FP32 path
-          const float f = gsc[c] * scT;
-          col[c].re = d2f_bits(w2.x) * f;
-          col[c].im = d2f_bits(w2.y) * f;
-        } else if constexpr (kDF) {   // split on the integer pipe, products in DF64
-          const Df f = df_mul(gsc[c], scT);
-          col[c].re = df_mul(d2df_bits(w2.x), f);
-          col[c].im = df_mul(d2df_bits(w2.y), f);
-        } else {
-          const double f = gsc[c] * sc;
-          col[c].re = w2.x * f;
-          col[c].im = w2.y * f;
-        }
+        const float f = gsc[c] * scT;   // no FP64 arithmetic here
+        col[c].re = d2f_bits(w2.x) * f;
+        col[c].im = d2f_bits(w2.y) * f;
       }
     }
     // forward z, y, x
@@ -186,10 +173,7 @@ __device__ __forceinline__ void hbar_elem_body(const Geom& g, const T* sB, const
       uq[q] = r;
       dot_acc(apt, col[q], r);
     }
-    double apart;
-    if constexpr (kF32) apart = f2d_bits(apt);
-    else if constexpr (kDF) apart = f2d_bits(apt.hi) + f2d_bits(apt.lo);
-    else apart = apt;
+    const double apart = f2d_bits(apt);
     __syncthreads();
     // backward z, y, x
     bf_round<kBF>(uq);
@@ -846,6 +830,12 @@ __global__ void k_diag_add(long long n, int n_orb, const double* __restrict__ vn
   }
 }
 
+// Batched element results are kept at the orbital stride of 16-byte entries for every
+// contraction type, so that under TDKS_MIXED FP32 and double-float orbitals share the
+// buffer: entries of Cx<T> per orbital = n_elem P1^3 * omul<T>.
+template <typename T>
+__host__ __device__ constexpr int batch_omul() { return (int)(sizeof(double2) / sizeof(Cx<T>)); }
+
 // ---------------------------------------------------------------------------
 // Batched apply: a persistent grid walks the work list of one degree class.
 // Item (sys, eblk, o0, o1): elements [eblk E, eblk E + E) of system sys for the
@@ -853,12 +843,6 @@ __global__ void k_diag_add(long long n, int n_orb, const double* __restrict__ vn
 // current basis vector V_j (j = K.k): the exponential's start vector for j = 0
 // (input or, after a sub-step, output), the workspace otherwise.
 // ---------------------------------------------------------------------------
-// Batched element results are kept at the orbital stride of 16-byte entries for every
-// contraction type, so that under TDKS_MIXED FP32 and double-float orbitals share the
-// buffer: entries of Cx<T> per orbital = n_elem P1^3 * omul<T>.
-template <typename T>
-__host__ __device__ constexpr int batch_omul() { return (int)(sizeof(double2) / sizeof(Cx<T>)); }
-
 template <int P1, typename T>
 __global__ void __launch_bounds__(256, SplitOcc<P1, T>::value) k_hbar_batch_split(const BSys* __restrict__ sys,
                                                     const BItem* __restrict__ items, int n_items,
@@ -1131,7 +1115,7 @@ __global__ void __launch_bounds__(256) k_gather(Geom g, const double* __restrict
     __shared__ double tot;
     if (threadIdx.x == 0) tot = v;
     __syncthreads();
-    alpha = a.cg->alpha / tot;      // CgState::alpha carries the current r . z here
+    alpha = a.cg->rz_new / tot;
   }
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const unsigned iu = (unsigned)i, row = iu / (unsigned)g.nix;   // n < 2^32: the fields of a larger mesh do not fit the device

@@ -484,7 +484,6 @@ __global__ void __launch_bounds__(256, 2) k_hbar_batch_fx(const BSys* __restrict
     auto orb = [&](int o, const double2*& in, double& sc) -> bool {
       const KryOrb& K = S.kry[o];
       if (K.status != KRY_ACTIVE) return false;
-      if (S.mixed && K.f32) return false;   // relaxed schedule: the FP32 launch takes it
       const int j = K.k;
       in = bvec(S, K, o, j);
       sc = K.s[j];

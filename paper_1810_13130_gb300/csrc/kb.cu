@@ -489,8 +489,6 @@ tdks_status kb_project(tdks_ctx* c, const ApplyArgs& a) {
                       [](double2* p) { cudaFree(p); }, [&] { kgraph_drop(c); }))
       return tdks_fail(c, TDKS_ERR_NOMEM, "projections");
     k->c_orb = a.n_orb;
-    cudaFree(k->d_view);      // as does the batched view
-    k->d_view = nullptr;
   }
   if (k->n_chunks > 0) {
     const dim3 grid(k->n_chunks, a.n_orb);

@@ -83,7 +83,7 @@ __global__ void k_cg_init_fin(const double* part, int nb, double tol, CgState* c
     cg->bb = bb;
     cg->rr = rr;
     cg->rz = 0.0;
-    cg->alpha = 0.0;
+    cg->rz_new = 0.0;
     cg->iters = 0;
     cg->first = 1;
     cg->failed = (isfinite(bb) && isfinite(rr)) ? 0 : 1;
@@ -121,7 +121,7 @@ __global__ void k_cg_dir(long long n, const double* part, int nb, const double* 
   const double rz = sum_fixed(part, nb);
   const bool first = cg->first != 0;
   const double beta = first ? 0.0 : rz / cg->rz;
-  if (blockIdx.x == 0 && threadIdx.x == 0) cg->alpha = rz;
+  if (blockIdx.x == 0 && threadIdx.x == 0) cg->rz_new = rz;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x)
     p[i] = first ? z[i] : fma(beta, p[i], z[i]);
@@ -132,7 +132,7 @@ __global__ void k_cg_fin_rr(const double* part, int nb, double tol, int maxit, C
   const double rr = sum_fixed(part, nb);
   if (threadIdx.x == 0) {
     cg->rr = rr;
-    cg->rz = cg->alpha;
+    cg->rz = cg->rz_new;
     cg->first = 0;
     cg->iters += 1;
     if (!isfinite(rr)) {
@@ -525,7 +525,6 @@ void axis_gemm(tdks_ctx* c, int axis, bool forward, const double* in, double* ou
   else go(t == 64 ? k_gemm<64> : t == 32 ? k_gemm<32> : k_gemm<16>);
 }
 
-// z = S D^-1 S^T r  (exact inverse of the separable stiffness)
 // End of a fixed-length CG: zero right-hand side -> x = 0; not converged or
 // non-finite -> error bits (4: iteration cap, 8: non-finite).
 __global__ void k_cg_graph_end(long long n, double* x, const CgState* cg, int* err) {
@@ -540,6 +539,7 @@ __global__ void k_cg_graph_end(long long n, double* x, const CgState* cg, int* e
     x[i] = 0.0;
 }
 
+// z = S D^-1 S^T r  (exact inverse of the separable stiffness)
 void fdm_apply(tdks_ctx* c, const double* r, double* z, const CgState* cg, bool df) {
   const long long n = c->n_int;
   axis_gemm(c, 0, true, r, c->d_t1, cg, df);

@@ -51,7 +51,7 @@ struct CgState {
   double bb;        // ||b||^2
   double rz;        // r.z of the previous residual
   double rr;        // ||r||^2
-  double alpha;     // r.z of the current residual, while rz still holds the previous one
+  double rz_new;    // r.z of the current residual, while rz still holds the previous one
   int iters;
   int done;         // 1 when converged
   int failed;
@@ -218,8 +218,8 @@ void tdks_fdm_axis(const Tables1D& t, int p, const double* br, int n_el, std::ve
 #endif
 
 // Device table layout (both double and float copies), offsets in elements.
-//   B [P1*P1] | Kq [P1*P1] | w [P1] | K1 [P1*P1] | Mg [P1*P1] | eta [P1]
-//   | csB | csBT | csKq      (even-odd folded forms, see cs_apply in elements.cuh)
+//   w [P1] | eta [P1] | csB | csBT | csKq | GLL weights [P1] | csK1 | csMg
+// (cs: even-odd folded forms, see cs_apply in elements.cuh)
 // A centrosymmetric n x n matrix M (M[n-1-i][n-1-j] = M[i][j]) is stored folded as
 // Me[h][h] = (M[q][i] + M[q][n-1-i])/2, Mo[h][h] = (M[q][i] - M[q][n-1-i])/2 for
 // q, i < h = n/2, then (odd n) the middle column M[q][h], the middle row M[h][i]
@@ -241,13 +241,9 @@ void fold_centrosymmetric(const T* M, int n, T* out) {
   for (int i = 0; i < h; ++i) mr[i] = (n & 1) ? M[h * n + i] : (T)0;
   mr[h] = (n & 1) ? M[h * n + h] : (T)0;
 }
-TDKS_HD inline int tab_off_B(int) { return 0; }
-TDKS_HD inline int tab_off_Kq(int P1) { return P1 * P1; }
-TDKS_HD inline int tab_off_w(int P1) { return 2 * P1 * P1; }
-TDKS_HD inline int tab_off_K1(int P1) { return 2 * P1 * P1 + P1; }
-TDKS_HD inline int tab_off_Mg(int P1) { return 3 * P1 * P1 + P1; }
-TDKS_HD inline int tab_off_eta(int P1) { return 4 * P1 * P1 + P1; }
-TDKS_HD inline int tab_off_csB(int P1) { return 4 * P1 * P1 + 2 * P1; }
+TDKS_HD inline int tab_off_w(int) { return 0; }
+TDKS_HD inline int tab_off_eta(int P1) { return P1; }
+TDKS_HD inline int tab_off_csB(int P1) { return 2 * P1; }
 TDKS_HD inline int tab_off_csBT(int P1) { return tab_off_csB(P1) + cs_size(P1); }
 TDKS_HD inline int tab_off_csK(int P1) { return tab_off_csBT(P1) + cs_size(P1); }
 TDKS_HD inline int tab_off_wl(int P1) { return tab_off_csK(P1) + cs_size(P1); }   // GLL weights
@@ -276,7 +272,7 @@ struct ApplyArgs {
   int accumulate;             // out += result instead of out = result (plain apply only)
 };
 tdks_status launch_hbar_apply(tdks_ctx* c, const ApplyArgs& a, int prec);
-// hbar_fx.cu: element results of the FP64 and double-float applications, E elements per
+// hbar_fx.cu: element results of the FP64 applications, E elements per
 // CTA (bpe CTAs) and opc orbitals per CTA; results and alpha as described there
 cudaError_t launch_hbar_fx(int P1, const Geom& g, const tdks::FxHost& h, const double* vks, const ApplyArgs& a,
                            int E, int bpe, int opc, double2* ev, cudaStream_t st);
