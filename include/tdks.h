@@ -464,7 +464,7 @@ tdks_status tdks_set_apply_tile(tdks_ctx* ctx, int orbs_per_cta);
 tdks_status tdks_set_f32_stages(tdks_ctx* ctx, unsigned mask);
 
 /* Work counters of a context (for benchmarking): kernel launches issued, Hbar
- * colour launches, element-orbital applications, and -- when timing is on --
+ * applications, element-orbital applications, and -- when timing is on --
  * the summed device time of the Hbar applications inside tdks_expm measured
  * with CUDA events on the context's stream.  reset != 0 zeroes them after
  * reading.  out may be NULL (reset only). */

@@ -359,6 +359,7 @@ tdks_status tdks_create(const tdks_mesh_desc* m, const tdks_system_desc* s, void
     if (cudaMemset(*f, 0, c->n_int * sizeof(double)) != cudaSuccess) return fail(TDKS_ERR_CUDA);
   }
   if ((st = dalloc(c, &c->d_cg, 1)) != TDKS_OK) return fail(st);
+  // partial sums of one orbital: at most hbar_blocks of an application, assemble_blocks of a norm
   const int bpc = hbar_blocks(c);
   c->part_stride = std::max<int64_t>(2048, 8 * (int64_t)bpc);
   if ((st = dalloc(c, &c->d_part, (size_t)(2 * (c->n_orb + 2) * c->part_stride + 8192))) != TDKS_OK)

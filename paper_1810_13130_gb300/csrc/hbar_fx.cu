@@ -19,13 +19,13 @@
 // part one after the other, the next orbital's columns copied to shared memory meanwhile.
 // The largest value of an element's part (real or imaginary) sets its exponent: one integer
 // maximum over the element's threads.  (With one exponent for both, the imaginary part of an
-// orbital after a weak kick kept only the bits that the real part left.)  Measured per application of 16 orbitals on 16^3
-// elements, p = 6: 4.62 ms with FP64 contractions (95 % of the FP64 pipe), 1.36 ms here
-// (7800 instructions per warp and orbital at 50 % issue activity, wide multiply-adds 44 % of
-// their pipe, two CTAs of 128 registers per SM); 5 orbitals on 20^3, p = 8: 7.1 -> 2.0 ms.
-// Three CTAs per SM (80 registers, spills) or smaller CTAs are slower (1.70, 1.53 ms).
-// A non-finite input or potential makes the results
-// of its element NaN.  The scale s_j of a Krylov vector is left out here and applied by
+// orbital after a weak kick kept only the bits that the real part left.)  Measured per
+// application of 16 orbitals on 16^3 elements, p = 6: 4.62 ms with FP64 contractions (95 % of the
+// FP64 pipe), 1.43 ms here (8300 instructions per warp and orbital at 50 % issue activity, wide
+// multiply-adds 42 % of their pipe, two CTAs of 128 registers per SM); 1.38 ms while the inputs'
+// bits below the unit were dropped and the values not raised.  Three CTAs per SM (80 registers,
+// spills) or smaller CTAs were slower (1.70, 1.53 ms).  A non-finite input or potential makes the
+// results of its element NaN.  The scale s_j of a Krylov vector is left out here and applied by
 // the assembly (and to alpha), so results are those of V_j.
 #include "elements.cuh"
 #include "fixed.cuh"
@@ -513,7 +513,7 @@ __global__ void __launch_bounds__(256, 2) k_hbar_batch_fx(const BSys* __restrict
 // contractions of the element kernel with B', one exponent per element and orbital; the
 // squares are formed and summed over the orbitals in FP64 and divided by the weights that B'
 // carries.  FP64 contractions were bound by the FP64 pipe (10 orbitals, 14^3 elements, p = 6:
-// 731 us, 394 us here; 16 orbitals, 16^3: 1.75 ms, 0.90 ms).
+// 731 us; 16 orbitals, 16^3: 1.75 ms, 0.81 ms here).
 template <int P1>
 __global__ void __launch_bounds__(256, 2) k_density_fx(Geom g, const __grid_constant__ FxTab<P1> tab,
                                                        const double2* __restrict__ psi, int64_t stride, int n_orb,

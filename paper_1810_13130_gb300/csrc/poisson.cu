@@ -514,7 +514,8 @@ void axis_gemm(tdks_ctx* c, int axis, bool forward, const double* in, double* ou
   }
   // Fixed point wherever its accumulators allow it.  Tiles of 32 while they give every SM a
   // CTA, then 16 (83 x 6889, p = 6, 14^3 elements: 16: 59, 32: 48, 64: 98 us, FP64 112 us;
-  // 95 x 9025: 73, 57, 100 us, FP64 141 us); longer axes keep the FP64 product.
+  // 95 x 9025: 73, 57, 100 us, FP64 141 us; at 55 bits, the carries of 58 add 2 us); longer axes
+  // keep the FP64 product.
   const bool fx = !df && g.K <= kFxK;
   const auto ctas = [&](int s) { return (long long)((g.M + s - 1) / s) * ((g.N + s - 1) / s) * batch; };
   const int t = !fx ? gemm_tile(g.M, g.N, batch) : ctas(32) >= 152 ? 32 : 16;
